@@ -500,8 +500,11 @@ fga_status fga_propagate(const fga_model *m, fga_beams *b, double dt, int nsteps
         FGA_TRY(launch_layered_steps(m, b, dt, nsteps, s));
         FGA_TRY(sync_layered_count(b, s));
     } else {
-        for (int n0 = 0; n0 < nsteps; n0 += 64)
-            FGA_TRY(launch_propagate(m, b, dt, std::min(64, nsteps - n0), nullptr, s));
+        // a constant medium advances any number of steps per launch (closed form); the general kernel's
+        // launches are kept short
+        const int chunk = m->dev.kind == FGA_MEDIUM_CONST ? std::max(nsteps, 1) : 64;
+        for (int n0 = 0; n0 < nsteps; n0 += chunk)
+            FGA_TRY(launch_propagate(m, b, dt, std::min(chunk, nsteps - n0), nullptr, s));
     }
     b->last_stream = s;
     return FGA_OK;
