@@ -841,10 +841,13 @@ fga_status solve_impl(const fga_model *m, const fga_init_desc *init, const fga_s
             at[(size_t)j] = n;
         }
         int js = 0;
-        for (int n = 1; n <= sd->nsteps; n++) {
+        for (int n = 0; n < sd->nsteps;) {
             if (cancel && cancel->load()) return cancelled(s);
-            FGA_TRY(launch_layered_steps(m, b, sd->dt, 1, s));
-            if (!seis || js >= sd->n_times || at[(size_t)js] != n) continue;
+            // the steps up to the next sample (or the end) as one group
+            const int to = seis && js < sd->n_times ? at[(size_t)js] : sd->nsteps;
+            FGA_TRY(launch_layered_steps(m, b, sd->dt, to - n, s));
+            n = to;
+            if (!seis || js >= sd->n_times) continue;
             FGA_TRY(sync_layered_count(b, s));
             while (js < sd->n_times && at[(size_t)js] == n) {
                 void *out = static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)js;
@@ -1189,7 +1192,7 @@ fga_status fga_beams_destroy(fga_beams *b) {
     if (!b) return FGA_OK;
     b->ws.release();
     for (DevBuf *d : {&b->state, &b->state_alt, &b->flags, &b->flags_alt, &b->id, &b->id_alt, &b->path, &b->counts,
-                      &b->n_begin})
+                      &b->events})
         d->release();
     delete b;
     return FGA_OK;

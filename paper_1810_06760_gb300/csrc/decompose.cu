@@ -443,7 +443,6 @@ static fga_status beams_allocate(fga_beams *b, const fga_init_desc *d, cudaStrea
     if (b->layered) {
         FGA_TRY(b->path.ensure(8 * b->cap));
         FGA_TRY(b->counts.ensure(16));
-        FGA_TRY(b->n_begin.ensure(8));
         const unsigned long long c0[2] = {(unsigned long long)off, 0ull};
         FGA_CUDA(cudaMemsetAsync(b->path.p, 0, 8 * b->cap, s));
         FGA_CUDA(cudaMemcpyAsync(b->counts.p, c0, sizeof c0, cudaMemcpyHostToDevice, s));

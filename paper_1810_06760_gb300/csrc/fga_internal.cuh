@@ -233,7 +233,8 @@ struct fga_beams {
     bool layered = false;
     int gmax = 4;            // a beam is dropped at its (gmax+1)-th interface
     double rel_min = 1e-6;   // children below rel_min of the incident amplitude are not created
-    fga::DevBuf path, counts, n_begin;  // lineage (parent*4 + child slot + 1); [slots used, overflow]
+    fga::DevBuf path, counts;  // lineage (parent*4 + child slot + 1); [slots used, overflow]
+    fga::DevBuf events;        // lists of beams at an interface inside a group of steps (layered.cu)
 };
 
 namespace fga {

@@ -5,10 +5,12 @@
 // Eq. Inter_DzQDzP; at a sphere all of it in the local tangent-normal frame of the crossing point), and
 // every child finishes the step.  Children are appended to the beam arrays with an atomic counter; the
 // parent's slot goes to its first child.
+#include <algorithm>
 #include <cmath>
 
 #include "fga_beam.cuh"
 #include "gather.cuh"
+#include "straight.cuh"
 
 namespace fga {
 
@@ -30,106 +32,6 @@ __device__ __forceinline__ double cabs2(Cd a) { return a.r * a.r + a.i * a.i; }
 // Layer speed of a beam (bits 4-7 of its flags hold its layer).
 template <typename R> __device__ __forceinline__ R layer_speed(const ModelDev &M, int wave, int lay) {
     return wave ? mp<R>(M.lcs[lay], M.flcs[lay]) : mp<R>(M.lcp[lay], M.flcp[lay]);
-}
-
-// dy/dt in a homogeneous layer (grad c = 0): Q' = sg c P^, P' = 0, dzQ' = sg (c/|P|) dzP (I - P^P^T),
-// dzP' = 0, amplitudes a' = (1/2) tr(Z^-1 Z') a (no SV/SH coupling: P is constant).
-template <typename R>
-__device__ __forceinline__ void layer_rhs(R sg, R c, const R *y, R *f) {
-    const R P[3] = {y[F_P], y[F_P + 1], y[F_P + 2]};
-    const R ip = Real<R>::rsqrt_(P[0] * P[0] + P[1] * P[1] + P[2] * P[2]);
-    const R Ph[3] = {P[0] * ip, P[1] * ip, P[2] * ip};
-    const R cip = c * ip;
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        f[F_Q + d] = sg * c * Ph[d];
-        f[F_P + d] = R(0);
-    }
-    C2<R> Z[3][3], Zd[3][3];
-#pragma unroll
-    for (int m = 0; m < 3; m++) {
-        R vr = R(0), vi = R(0);
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            vr += y[F_DP + 2 * (3 * m + l)] * Ph[l];
-            vi += y[F_DP + 2 * (3 * m + l) + 1] * Ph[l];
-        }
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const int e = 2 * (3 * m + j);
-            f[F_DQ + e] = sg * cip * (y[F_DP + e] - vr * Ph[j]);
-            f[F_DQ + e + 1] = sg * cip * (y[F_DP + e + 1] - vi * Ph[j]);
-            f[F_DP + e] = R(0);
-            f[F_DP + e + 1] = R(0);
-            Z[m][j] = {y[F_DQ + e] - y[F_DP + e + 1], y[F_DQ + e + 1] + y[F_DP + e]};
-            Zd[m][j] = {f[F_DQ + e], f[F_DQ + e + 1]};
-        }
-    }
-    C2<R> Cf[3][3];
-    Cf[0][0] = cmulsub(Z[1][1], Z[2][2], Z[1][2], Z[2][1]);
-    Cf[0][1] = cmulsub(Z[1][2], Z[2][0], Z[1][0], Z[2][2]);
-    Cf[0][2] = cmulsub(Z[1][0], Z[2][1], Z[1][1], Z[2][0]);
-    Cf[1][0] = cmulsub(Z[0][2], Z[2][1], Z[0][1], Z[2][2]);
-    Cf[1][1] = cmulsub(Z[0][0], Z[2][2], Z[0][2], Z[2][0]);
-    Cf[1][2] = cmulsub(Z[0][1], Z[2][0], Z[0][0], Z[2][1]);
-    Cf[2][0] = cmulsub(Z[0][1], Z[1][2], Z[0][2], Z[1][1]);
-    Cf[2][1] = cmulsub(Z[0][2], Z[1][0], Z[0][0], Z[1][2]);
-    Cf[2][2] = cmulsub(Z[0][0], Z[1][1], Z[0][1], Z[1][0]);
-    R dr = R(0), di = R(0), tr = R(0), ti = R(0);
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-        dr += Z[0][j].r * Cf[0][j].r - Z[0][j].i * Cf[0][j].i;
-        di += Z[0][j].r * Cf[0][j].i + Z[0][j].i * Cf[0][j].r;
-    }
-#pragma unroll
-    for (int m = 0; m < 3; m++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            tr += Cf[m][j].r * Zd[m][j].r - Cf[m][j].i * Zd[m][j].i;
-            ti += Cf[m][j].r * Zd[m][j].i + Cf[m][j].i * Zd[m][j].r;
-        }
-    const R idn = Real<R>::rcp_pos_(dr * dr + di * di);
-    const R gr = R(0.5) * (tr * dr + ti * di) * idn, gi = R(0.5) * (ti * dr - tr * di) * idn;
-#pragma unroll
-    for (int q = 0; q < 2; q++) {
-        const R ar = y[F_A0 + 2 * q], ai = y[F_A0 + 2 * q + 1];
-        f[F_A0 + 2 * q] = gr * ar - gi * ai;
-        f[F_A0 + 2 * q + 1] = gr * ai + gi * ar;
-    }
-}
-
-// one classical RK4 step of size h: out = y + the step's increment (summed at its own scale), Q by
-// compensated summation with the compensation qc carried in and out
-template <typename R>
-__device__ __forceinline__ void layer_rk4(R sg, R c, const R *y, R h, R *out, R *qc) {
-    R k[NF], t[NF], inc[NF];
-    layer_rhs<R>(sg, c, y, k);
-#pragma unroll
-    for (int f = 0; f < NF; f++) {
-        inc[f] = h / R(6) * k[f];
-        t[f] = y[f] + R(0.5) * h * k[f];
-    }
-    layer_rhs<R>(sg, c, t, k);
-#pragma unroll
-    for (int f = 0; f < NF; f++) {
-        inc[f] += h / R(3) * k[f];
-        t[f] = y[f] + R(0.5) * h * k[f];
-    }
-    layer_rhs<R>(sg, c, t, k);
-#pragma unroll
-    for (int f = 0; f < NF; f++) {
-        inc[f] += h / R(3) * k[f];
-        t[f] = y[f] + h * k[f];
-    }
-    layer_rhs<R>(sg, c, t, k);
-#pragma unroll
-    for (int f = 3; f < NF; f++) out[f] = y[f] + (inc[f] + h / R(6) * k[f]);
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        R q = y[F_Q + d];
-        kahan_add<R>(q, qc[d], inc[F_Q + d] + h / R(6) * k[F_Q + d]);
-        out[F_Q + d] = q;
-    }
 }
 
 // Solve the 6x6 complex system A x = b (partial pivoting); false if singular.
@@ -349,7 +251,7 @@ __device__ void make_child(const R *yc, const EventOut &ev, int k, R *out) {
 // 1 (a path may dip into it and leave again within one step); the outer sphere bounds a convex ball, so
 // only an end point beyond it means a crossing, at the positive root.  Returns false without a crossing,
 // else the fraction th of the step, the layer lb entered and the radius crossed.
-__device__ bool shell_crossing(const ModelDev &M, int L, const double q0[3], const double q1[3], double &th, int &lb,
+__device__ __noinline__ bool shell_crossing(const ModelDev &M, int L, const double q0[3], const double q1[3], double &th, int &lb,
                                double &rho) {
     double s0[3], d[3], s1[3];
     for (int c = 0; c < 3; c++) {
@@ -432,19 +334,20 @@ __device__ __forceinline__ void surf_grad(const ModelDev &M, int i, double x1, d
 // bound layer L (by a margin far above the FP32 rounding of the heights, which grows with the phase
 // k |x| of the cosines).
 __device__ __forceinline__ bool surf_clear(const ModelDev &M, int L, const float *q1) {
-    const float cc = cosf(M.fuk[0] * q1[0]) * cosf(M.fuk[1] * q1[1]);
     const float ph = M.fuk[0] * fabsf(q1[0]) + M.fuk[1] * fabsf(q1[1]);
-    if (L < M.nlay - 1) {
-        const float h = M.fzif[L] + M.fuamp[L] * cc;
-        const float m = 1e-4f * (1.0f + fabsf(M.fzif[L]) + fabsf(M.fuamp[L])) + 2e-6f * fabsf(M.fuamp[L]) * ph;
-        if (!(q1[2] < h - m)) return false;
+    float mid[2], amp[2], mar[2];   // lower and upper interface of the layer: mean depth, amplitude, margin
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+        const int i = e == 0 ? L : L - 1;
+        const bool there = i >= 0 && i < M.nlay - 1;
+        mid[e] = there ? M.fzif[i] : (e == 0 ? INFINITY : -INFINITY);
+        amp[e] = there ? M.fuamp[i] : 0.0f;
+        mar[e] = there ? 1e-4f * (1.0f + fabsf(mid[e]) + fabsf(amp[e])) + 2e-6f * fabsf(amp[e]) * ph : 0.0f;
     }
-    if (L > 0) {
-        const float h = M.fzif[L - 1] + M.fuamp[L - 1] * cc;
-        const float m = 1e-4f * (1.0f + fabsf(M.fzif[L - 1]) + fabsf(M.fuamp[L - 1])) + 2e-6f * fabsf(M.fuamp[L - 1]) * ph;
-        if (!(q1[2] >= h + m)) return false;
-    }
-    return true;
+    // outside both interfaces' bands of depth no height is needed
+    if (q1[2] < mid[0] - fabsf(amp[0]) - mar[0] && q1[2] >= mid[1] + fabsf(amp[1]) + mar[1]) return true;
+    const float cc = cosf(M.fuk[0] * q1[0]) * cosf(M.fuk[1] * q1[1]);
+    return q1[2] < mid[0] + amp[0] * cc - mar[0] && q1[2] >= mid[1] + amp[1] * cc + mar[1];
 }
 __device__ __forceinline__ bool surf_clear(const ModelDev &, int, const double *) { return false; }
 
@@ -455,7 +358,7 @@ __device__ __forceinline__ bool surf_clear(const ModelDev &, int, const double *
 // start already beyond the interface (no sign change) takes the root of g's linear interpolation (the start
 // itself when g does not change along the path).
 // Returns false without a crossing, else th, the layer lb entered and the interface index.
-__device__ bool surf_crossing(const ModelDev &M, int L, const double q0[3], const double q1[3], double &th, int &lb,
+__device__ __noinline__ bool surf_crossing(const ModelDev &M, int L, const double q0[3], const double q1[3], double &th, int &lb,
                               int &iface) {
     const double d[3] = {q1[0] - q0[0], q1[1] - q0[1], q1[2] - q0[2]};
     bool hit = false;
@@ -506,17 +409,18 @@ __device__ bool surf_crossing(const ModelDev &M, int L, const double q0[3], cons
 }  // namespace
 
 // Write child ce (with its Q compensation) of the beam in slot b: the first child takes the parent's slot,
-// the others are appended (atomic counter); children beyond cap are counted in counts[1].
+// the others are appended (atomic counter); children beyond cap are counted in counts[1].  Returns the slot
+// (-1 for a child beyond cap).
 template <typename R>
-__device__ void store_child(R *__restrict__ st, int32_t *__restrict__ flags, int32_t *__restrict__ ids,
-                            long long *__restrict__ path, int64_t cap, unsigned long long *__restrict__ counts, int64_t b,
-                            int k, const R *ce, const R *qch, int flc, int32_t id, long long pp, int slot) {
+__device__ int64_t store_child(R *__restrict__ st, int32_t *__restrict__ flags, int32_t *__restrict__ ids,
+                               long long *__restrict__ path, int64_t cap, unsigned long long *__restrict__ counts,
+                               int64_t b, int k, const R *ce, const R *qch, int flc, int32_t id, long long pp, int slot) {
     int64_t dst = b;
     if (k > 0) {
         dst = (int64_t)atomicAdd(&counts[0], 1ull);
         if (dst >= cap) {
             atomicAdd(&counts[1], 1ull);
-            return;
+            return -1;
         }
     }
 #pragma unroll
@@ -526,196 +430,289 @@ __device__ void store_child(R *__restrict__ st, int32_t *__restrict__ flags, int
     flags[dst] = flc;
     ids[dst] = id;
     path[dst] = pp * 4 + slot + 1;
+    return dst;
 }
 
-// The interface event of beam b in curved layers (SHAPE 1: spheres, SHAPE 2: undulating interfaces), at
-// fraction th of the step where it enters layer lb through the sphere of radius rho or through interface
-// iface.  The beam (still unchanged in st) advances to the crossing, which is put on the interface in FP64
-// (radially onto the sphere, vertically onto the undulating surface; its FP32 rounding goes to the Q
-// compensation), and is rotated into the local frame whose third axis is the interface's normal there; the
-// flat-interface event runs in that frame (Sec. 3.1: the tangent plane stands in for the interface), and
-// every child is rotated back and finishes the step.  Kept out of line and reading its beam from memory, so
-// that the step kernel's state stays in registers.
+// Interfaces that bound layer L of a planar medium.
+template <typename R> struct Planes {
+    R top, bot;
+    __device__ __forceinline__ Planes(const ModelDev &M, int L)
+        : top(L > 0 ? mp<R>(M.zif[L - 1], M.fzif[L - 1]) : -R(INFINITY)),
+          bot(L < M.nlay - 1 ? mp<R>(M.zif[L], M.fzif[L]) : R(INFINITY)) {}
+};
+
+// Does the step q0 -> q1 (compensations c0, c1) meet an interface of layer L?  Planes: the end point.  Curved
+// layers: FP32 steps that stay clear of the interfaces by a margin far above the rounding of the screen are
+// decided by the screen, the rest by the exact FP64 test, which also gives the crossing.
+struct Crossing {
+    double th, rho;
+    int lb, iface;
+};
 template <typename R, int SHAPE>
-__device__ __noinline__ void curved_event_step(const ModelDev &M, R *__restrict__ st, int32_t *__restrict__ flags,
-                                               int32_t *__restrict__ ids, long long *__restrict__ path, int64_t cap,
-                                               unsigned long long *__restrict__ counts, R dt, double rel_min, int64_t b,
-                                               int fl, R sg, R c, double th, int lb, double rho, int iface) {
-    R y[NF], yc[NF], qc[3];
-    for (int f = 0; f < NF; f++) y[f] = st[(int64_t)f * cap + b];
-    for (int d = 0; d < 3; d++) qc[d] = st[(int64_t)(F_QC + d) * cap + b];
-    layer_rk4<R>(sg, c, y, (R)th * dt, yc, qc);
-    double x[3], nrm[3], Rl[9];
-    for (int d = 0; d < 3; d++) x[d] = (double)yc[F_Q + d] - (double)qc[d];
-    if (SHAPE == 1) {
-        double s[3], sn = 0.0;
-        for (int d = 0; d < 3; d++) {
-            s[d] = x[d] - M.ctr[d];
-            sn += s[d] * s[d];
-        }
-        sn = sqrt(sn);
-        for (int d = 0; d < 3; d++) {
-            nrm[d] = s[d] / sn;
-            x[d] = M.ctr[d] + rho * nrm[d];
-        }
-    } else {
-        x[2] = surf_h(M, iface, x[0], x[1]);
-        double h1, h2;
-        surf_grad(M, iface, x[0], x[1], h1, h2);
-        const double nn = sqrt(1.0 + h1 * h1 + h2 * h2);
-        nrm[0] = -h1 / nn;
-        nrm[1] = -h2 / nn;
-        nrm[2] = 1.0 / nn;
-    }
+__device__ __forceinline__ bool step_crosses(const ModelDev &M, int L, const Planes<R> &pl, const R *q0, const R *c0,
+                                             const R *q1, const R *c1, Crossing &x) {
+    if (SHAPE == 0) return q1[2] < pl.top || q1[2] >= pl.bot;
+    if (sizeof(R) == 4 && (SHAPE == 1 ? shell_clear(M, L, q0, q1) : surf_clear(M, L, q1))) return false;
+    double a[3], b[3];
+#pragma unroll
     for (int d = 0; d < 3; d++) {
-        yc[F_Q + d] = (R)x[d];
-        qc[d] = (R)((double)yc[F_Q + d] - x[d]);
+        a[d] = (double)q0[d] - (double)c0[d];
+        b[d] = (double)q1[d] - (double)c1[d];
     }
-    frame_from_normal(nrm, Rl);
-    int fll = fl;
-    rotate_state<R>(Rl, false, false, yc, fll);   // Q stays global: the event does not read it
-    EventOut ev;
-    interface_event<R>(M, fll, yc, lb, rel_min, ev);
-    if (ev.n == 0) {
-        flags[b] = fl | FL_DEAD;
-        return;
-    }
-    const long long pp = path[b];
-    const int32_t id = ids[b];
-    for (int k = 0; k < ev.n; k++) {
-        R ch[NF], ce[NF], qch[3] = {qc[0], qc[1], qc[2]};
-        make_child<R>(yc, ev, k, ch);
-        int flc = ev.flags[k];
-        rotate_state<R>(Rl, true, false, ch, flc);
-        const R sgc = (flc & 1) ? R(-1) : R(1);
-        layer_rk4<R>(sgc, layer_speed<R>(M, (flc & FL_CLASS_MASK) >= 2, (flc >> 4) & 15), ch, R(1.0 - th) * dt, ce,
-                     qch);
-        store_child<R>(st, flags, ids, path, cap, counts, b, k, ce, qch, flc, id, pp, ev.slot[k]);
-    }
+    return SHAPE == 1 ? shell_crossing(M, L, a, b, x.th, x.lb, x.rho) : surf_crossing(M, L, a, b, x.th, x.lb, x.iface);
 }
 
-// One step for every beam alive at the start of the step (n_begin = *counts); children beyond the
-// first are appended at *counts (atomic); overflow beyond cap is counted in counts[1].
+// Steps s .. nsteps-1 of a beam up to the first one that meets an interface; returns that step's index (nsteps
+// without one), the state at its start in y, qc.  Every step but that one is the closed form of straight.cuh.
 template <typename R, int SHAPE>
-__global__ void __launch_bounds__(128) layered_step_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
-                                                          int32_t *__restrict__ ids, long long *__restrict__ path,
-                                                          int64_t cap, const int64_t *__restrict__ n_begin,
-                                                          unsigned long long *__restrict__ counts, R dt, int gmax,
-                                                          double rel_min) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= *n_begin) return;
-    const int fl = flags[b];
-    if (fl & FL_DEAD) return;
+__device__ __forceinline__ int layered_run(const ModelDev &M, int fl, R *y, R *qc, R dt, int s, int nsteps,
+                                           bool force_first) {
     const int wave = (fl & FL_CLASS_MASK) >= 2, L = (fl >> 4) & 15;
-    const R sg = (fl & 1) ? R(-1) : R(1);
-    R y[NF], y1[NF], qc[3], qc1[3];
-#pragma unroll
-    for (int f = 0; f < NF; f++) y[f] = st[(int64_t)f * cap + b];
-#pragma unroll
-    for (int d = 0; d < 3; d++) qc1[d] = qc[d] = st[(int64_t)(F_QC + d) * cap + b];
-    const R c = layer_speed<R>(M, wave, L);
-    layer_rk4<R>(sg, c, y, dt, y1, qc1);
-    if (SHAPE != 0) {
-        // FP32: a step that stays clear of the interfaces of its layer (by a margin far above the rounding of
-        // the screen) is decided by the screen; the rest take the exact FP64 test
-        bool hit = false;
-        double th = 0.0, rho = 0.0;
-        int lb = L, iface = 0;
-        const bool clear = sizeof(R) == 4 && (SHAPE == 1 ? shell_clear(M, L, y + F_Q, y1 + F_Q)
-                                                          : surf_clear(M, L, y1 + F_Q));
-        if (!clear) {
-            double q0[3], q1[3];
+    const R sg = (fl & 1) ? R(-1) : R(1), c = layer_speed<R>(M, wave, L);
+    const Planes<R> pl(M, L);
+    bool open = true;
+    while (open && s < nsteps) {
+        R B[18];
+        Straight<R> S;
+        straight_setup<R>(sg, c, y, B, S);
+        const int m = min(STRAIGHT_RENEW, nsteps - s);
+        C2<R> g1 = straight_gamma<R>(S, R(0));
+        int i = 0;
+        for (; i < m; i++) {
+            R q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
+            straight_q<R>(S, dt, q, qn);
+            Crossing x;
+            if (!force_first && step_crosses<R, SHAPE>(M, L, pl, y + F_Q, qc, q, qn, x)) {
+                open = false;
+                break;
+            }
+            force_first = false;
+            const R t = R(i) * dt;
+            const C2<R> g2 = straight_gamma<R>(S, t + R(0.5) * dt), g4 = straight_gamma<R>(S, t + dt);
+            straight_amplitudes<R>(y, straight_gain<R>(dt, g1, g2, g4));
+            g1 = g4;
 #pragma unroll
             for (int d = 0; d < 3; d++) {
-                q0[d] = (double)y[F_Q + d] - (double)qc[d];
-                q1[d] = (double)y1[F_Q + d] - (double)qc1[d];
+                y[F_Q + d] = q[d];
+                qc[d] = qn[d];
             }
-            hit = SHAPE == 1 ? shell_crossing(M, L, q0, q1, th, lb, rho) : surf_crossing(M, L, q0, q1, th, lb, iface);
+        }
+        const R T = R(i) * dt;
+#pragma unroll
+        for (int f = 0; f < 18; f++) y[F_DQ + f] += T * B[f];
+        s += i;
+    }
+    return s;
+}
+
+template <typename R>
+__device__ __forceinline__ void load_beam(const R *__restrict__ st, int64_t cap, int64_t b, R *y, R *qc) {
+#pragma unroll
+    for (int f = 0; f < NF; f++) y[f] = st[(int64_t)f * cap + b];
+#pragma unroll
+    for (int d = 0; d < 3; d++) qc[d] = st[(int64_t)(F_QC + d) * cap + b];
+}
+
+// append (beam slot, step) to an event list: one atomic per converged group of lanes
+__device__ __forceinline__ void push_event(int2 *__restrict__ list, unsigned *__restrict__ n, int64_t b, int s) {
+    const unsigned mask = __activemask(), lane = threadIdx.x & 31;
+    const int lead = __ffs(mask) - 1;
+    unsigned at = 0;
+    if ((int)lane == lead) at = atomicAdd(n, (unsigned)__popc(mask));
+    at = __shfl_sync(mask, at, lead) + __popc(mask & ((1u << lane) - 1u));
+    list[at] = make_int2((int)b, s);
+}
+
+// A group of nsteps steps, first part: every live beam advances until the group's end or until a step that
+// meets an interface; such beams are listed with their step (or die, past their last allowed interface).
+// One state stream per group instead of one per step: 49 reals read and 28 written per beam (P and dzP stay),
+// which bounds it.  442 k beams growing to 0.9 M, 300 steps in groups of 5, FP32: 69.6 ms (a launch per step
+// with four right-hand sides, events inside) -> 3.8 ms of these kernels and 8.7 ms of event kernels; with
+// undulating interfaces 187 -> 15.6 and 22.1 ms.
+template <typename R, int SHAPE>
+__global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
+                                                         int64_t cap, const unsigned long long *__restrict__ counts,
+                                                         R dt, int nsteps, int gmax, int2 *__restrict__ list,
+                                                         unsigned *__restrict__ nlist) {
+    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= cap || (unsigned long long)b >= counts[0]) return;
+    const int fl = flags[b];
+    if (fl & FL_DEAD) return;
+    R y[NF], qc[3];
+    load_beam<R>(st, cap, b, y, qc);
+    const int s = layered_run<R, SHAPE>(M, fl, y, qc, dt, 0, nsteps, false);
+#pragma unroll
+    for (int f = 0; f < 3; f++) st[(int64_t)f * cap + b] = y[f];
+#pragma unroll
+    for (int f = F_DQ; f < F_DP; f++) st[(int64_t)f * cap + b] = y[f];
+#pragma unroll
+    for (int f = F_A0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
+#pragma unroll
+    for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
+    if (s == nsteps) return;
+    if (((fl >> 8) & 15) >= gmax)
+        flags[b] = fl | FL_DEAD;
+    else
+        push_event(list, nlist, b, s);
+}
+
+// The listed beams: the event of step s at its interface, then every child finishes that step and advances
+// like the beams of layered_run_kernel; children that meet another interface go to the next list.  A thread
+// per event: an event costs thousands of FP64 operations, and a kernel of its own keeps whole warps on them
+// (inside the step kernel one lane of a warp held the other 31).
+//
+// In curved layers (SHAPE 1: spheres, SHAPE 2: undulating interfaces) the crossing is put on the interface in
+// FP64 (radially onto the sphere, vertically onto the undulating surface; its FP32 rounding goes to the Q
+// compensation), the beam is rotated into the local frame whose third axis is the interface's normal there, the
+// flat-interface event runs in that frame (Sec. 3.1: the tangent plane stands in for the interface), and every
+// child is rotated back.
+template <typename R, int SHAPE>
+__global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
+                                                          int32_t *__restrict__ ids, long long *__restrict__ path,
+                                                          int64_t cap, unsigned long long *__restrict__ counts, R dt,
+                                                          int nsteps, int gmax, double rel_min,
+                                                          const int2 *__restrict__ list, const unsigned *__restrict__ nlist,
+                                                          int2 *__restrict__ next, unsigned *__restrict__ nnext) {
+    const unsigned n = *nlist;
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const int64_t b = list[e].x;
+        int s = list[e].y;
+        const int fl = flags[b];
+        const int L = (fl >> 4) & 15;
+        const R sg = (fl & 1) ? R(-1) : R(1), c = layer_speed<R>(M, (fl & FL_CLASS_MASK) >= 2, L);
+        const Planes<R> pl(M, L);
+        R y[NF], qc[3];
+        load_beam<R>(st, cap, b, y, qc);
+        Crossing x{0.0, 0.0, L, 0};
+        bool hit = false;
+        while (s < nsteps) {
+            // the step's end point as layered_run forms it
+            R B[18], q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
+            Straight<R> S;
+            straight_setup<R>(sg, c, y, B, S);
+            straight_q<R>(S, dt, q, qn);
+            hit = step_crosses<R, SHAPE>(M, L, pl, y + F_Q, qc, q, qn, x);
+            if (hit) {
+                if (SHAPE == 0) {
+                    const bool down = q[2] >= pl.bot;
+                    const R zc = down ? pl.bot : pl.top;
+                    x.lb = down ? L + 1 : L - 1;
+                    const R th = (zc - y[F_Q + 2]) / (q[2] - y[F_Q + 2]);
+                    x.th = (double)th;
+                }
+                break;
+            }
+            // no crossing after all (a last-bit difference to the listing kernel): the step stands
+            s = layered_run<R, SHAPE>(M, fl, y, qc, dt, s, nsteps, true);
         }
         if (!hit) {
 #pragma unroll
-            for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y1[f];
+            for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
 #pragma unroll
-            for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc1[d];
-        } else if (((fl >> 8) & 15) >= gmax) {
-            flags[b] = fl | FL_DEAD;
-        } else {
-            curved_event_step<R, SHAPE>(M, st, flags, ids, path, cap, counts, dt, rel_min, b, fl, sg, c, th, lb, rho,
-                                        iface);
+            for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
+            continue;
         }
-        return;
+        straight_step<R>(sg, c, y, (R)x.th * dt, qc);
+        double Rl[9];
+        int fll = fl;
+        if (SHAPE == 0) {
+            y[F_Q + 2] = x.lb > L ? pl.bot : pl.top;
+            qc[2] = R(0);                 // the interface depth is exact
+        } else {
+            double p[3], nrm[3];
+            for (int d = 0; d < 3; d++) p[d] = (double)y[F_Q + d] - (double)qc[d];
+            if (SHAPE == 1) {
+                double r[3], rn = 0.0;
+                for (int d = 0; d < 3; d++) {
+                    r[d] = p[d] - M.ctr[d];
+                    rn += r[d] * r[d];
+                }
+                rn = sqrt(rn);
+                for (int d = 0; d < 3; d++) {
+                    nrm[d] = r[d] / rn;
+                    p[d] = M.ctr[d] + x.rho * nrm[d];
+                }
+            } else {
+                p[2] = surf_h(M, x.iface, p[0], p[1]);
+                double h1, h2;
+                surf_grad(M, x.iface, p[0], p[1], h1, h2);
+                const double nn = sqrt(1.0 + h1 * h1 + h2 * h2);
+                nrm[0] = -h1 / nn;
+                nrm[1] = -h2 / nn;
+                nrm[2] = 1.0 / nn;
+            }
+            for (int d = 0; d < 3; d++) {
+                y[F_Q + d] = (R)p[d];
+                qc[d] = (R)((double)y[F_Q + d] - p[d]);
+            }
+            frame_from_normal(nrm, Rl);
+            rotate_state<R>(Rl, false, false, y, fll);   // Q stays global: the event does not read it
+        }
+        EventOut ev;
+        interface_event<R>(M, fll, y, x.lb, rel_min, ev);
+        if (ev.n == 0) {
+            flags[b] = fl | FL_DEAD;
+            continue;
+        }
+        const long long pp = path[b];
+        const int32_t id = ids[b];
+        for (int k = 0; k < ev.n; k++) {
+            R ch[NF], qch[3] = {qc[0], qc[1], qc[2]};
+            make_child<R>(y, ev, k, ch);
+            int flc = ev.flags[k];
+            if (SHAPE != 0) rotate_state<R>(Rl, true, false, ch, flc);
+            straight_step<R>((flc & 1) ? R(-1) : R(1), layer_speed<R>(M, (flc & FL_CLASS_MASK) >= 2, (flc >> 4) & 15), ch,
+                             SHAPE == 0 ? (R(1) - (R)x.th) * dt : R(1.0 - x.th) * dt, qch);
+            int sc = nsteps;
+            if (!(flc & FL_DEAD)) sc = layered_run<R, SHAPE>(M, flc, ch, qch, dt, s + 1, nsteps, false);
+            const bool again = sc < nsteps;
+            if (again && ((flc >> 8) & 15) >= gmax) flc |= FL_DEAD;
+            const int64_t dst = store_child<R>(st, flags, ids, path, cap, counts, b, k, ch, qch, flc, id, pp, ev.slot[k]);
+            if (again && dst >= 0 && !(flc & FL_DEAD)) push_event(next, nnext, dst, sc);
+        }
     }
-    const R ztop = L > 0 ? mp<R>(M.zif[L - 1], M.fzif[L - 1]) : -R(INFINITY);
-    const R zbot = L < M.nlay - 1 ? mp<R>(M.zif[L], M.fzif[L]) : R(INFINITY);
-    if (y1[F_Q + 2] >= ztop && y1[F_Q + 2] < zbot) {
-#pragma unroll
-        for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y1[f];
-#pragma unroll
-        for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc1[d];
-        return;
-    }
-    // the step crosses an interface: advance to it, scatter, finish the step with every child
-    const bool down = y1[F_Q + 2] >= zbot;
-    const R zc = down ? zbot : ztop;
-    const int lb = down ? L + 1 : L - 1;
-    const R th = (zc - y[F_Q + 2]) / (y1[F_Q + 2] - y[F_Q + 2]);
-    if (((fl >> 8) & 15) >= gmax) {
-        flags[b] = fl | FL_DEAD;
-        return;
-    }
-    R yc[NF];
-    layer_rk4<R>(sg, c, y, th * dt, yc, qc);
-    yc[F_Q + 2] = zc;
-    qc[2] = R(0);                 // the interface depth is exact
-    EventOut ev;
-    interface_event<R>(M, fl, yc, lb, rel_min, ev);
-    if (ev.n == 0) {
-        flags[b] = fl | FL_DEAD;
-        return;
-    }
-    const long long pp = path[b];
-    const int32_t id = ids[b];
-    for (int k = 0; k < ev.n; k++) {
-        R ch[NF], ce[NF], qch[3] = {qc[0], qc[1], qc[2]};
-        make_child<R>(yc, ev, k, ch);
-        const int flc = ev.flags[k];
-        const R sgc = (flc & 1) ? R(-1) : R(1);
-        layer_rk4<R>(sgc, layer_speed<R>(M, (flc & FL_CLASS_MASK) >= 2, (flc >> 4) & 15), ch, (R(1) - th) * dt, ce,
-                     qch);
-        store_child<R>(st, flags, ids, path, cap, counts, b, k, ce, qch, flc, id, pp, ev.slot[k]);
-    }
-}
-
-__global__ void copy_count_kernel(const unsigned long long *counts, int64_t *n_begin, int64_t cap) {
-    const unsigned long long n = counts[0];
-    *n_begin = (int64_t)(n < (unsigned long long)cap ? n : (unsigned long long)cap);
 }
 
 fga_status launch_layered_steps(const fga_model *m, fga_beams *b, double dt, int nsteps, cudaStream_t s) {
     if (nsteps <= 0) return FGA_OK;
-    const int T = 128;
-    const unsigned blocks = (unsigned)((b->cap + T - 1) / T);
-    for (int n = 0; n < nsteps; n++) {
+    // event lists: two of cap entries, and a counter per round (a lineage meets at most gmax interfaces, 16 by
+    // its flag bits, and at most one per step)
+    const int rounds = std::max(1, std::min(std::min(b->gmax, 16), nsteps));
+    const size_t lb = sizeof(int2) * (size_t)b->cap, nb_ctr = sizeof(unsigned) * 20;
+    FGA_TRY(b->events.ensure(2 * lb + nb_ctr));
+    int2 *list[2] = {b->events.as<int2>(), b->events.as<int2>() + b->cap};
+    unsigned *ctr = reinterpret_cast<unsigned *>(b->events.as<char>() + 2 * lb);
+    FGA_CUDA(cudaMemsetAsync(ctr, 0, nb_ctr, s));
+    prof_add_beam_steps(b->nb * (int64_t)nsteps);
+    auto go = [&](auto real, auto shape) {
+        using R = decltype(real);
+        constexpr int SHAPE = decltype(shape)::value;
+        unsigned long long *counts = b->counts.as<unsigned long long>();
         {
-            ProfScope ps(P_OTHER_LAYER, s);
-            copy_count_kernel<<<1, 1, 0, s>>>(b->counts.as<unsigned long long>(), b->n_begin.as<int64_t>(), b->cap);
+            ProfScope ps(P_PROP, s);
+            layered_run_kernel<R, SHAPE><<<(unsigned)((b->cap + 127) / 128), 128, 0, s>>>(
+                m->dev, b->state.as<R>(), b->flags.as<int32_t>(), b->cap, counts, (R)dt, nsteps, b->gmax, list[0], ctr);
         }
-        prof_add_beam_steps(b->nb);
-        ProfScope ps(P_PROP, s);
-        // curved layers in their own instantiations, so that the planar kernel carries none of their code
-        auto kd = m->dev.shells ? layered_step_kernel<double, 1>
-                                : (m->dev.undul ? layered_step_kernel<double, 2> : layered_step_kernel<double, 0>);
-        auto kf = m->dev.shells ? layered_step_kernel<float, 1>
-                                : (m->dev.undul ? layered_step_kernel<float, 2> : layered_step_kernel<float, 0>);
-        if (b->precision == FGA_PREC_FP64)
-            kd<<<blocks, T, 0, s>>>(m->dev, b->state.as<double>(), b->flags.as<int32_t>(), b->id.as<int32_t>(),
-                                    b->path.as<long long>(), b->cap, b->n_begin.as<int64_t>(),
-                                    b->counts.as<unsigned long long>(), dt, b->gmax, b->rel_min);
+        for (int r = 0; r < rounds; r++) {
+            ProfScope ps(P_OTHER_LAYER, s);
+            layered_event_kernel<R, SHAPE><<<152 * 8, 64, 0, s>>>(
+                m->dev, b->state.as<R>(), b->flags.as<int32_t>(), b->id.as<int32_t>(), b->path.as<long long>(), b->cap,
+                counts, (R)dt, nsteps, b->gmax, b->rel_min, list[r & 1], ctr + r, list[(r + 1) & 1], ctr + r + 1);
+        }
+    };
+    using std::integral_constant;
+    auto shape = [&](auto real) {
+        if (m->dev.shells)
+            go(real, integral_constant<int, 1>{});
+        else if (m->dev.undul)
+            go(real, integral_constant<int, 2>{});
         else
-            kf<<<blocks, T, 0, s>>>(m->dev, b->state.as<float>(), b->flags.as<int32_t>(), b->id.as<int32_t>(),
-                                    b->path.as<long long>(), b->cap, b->n_begin.as<int64_t>(),
-                                    b->counts.as<unsigned long long>(), (float)dt, b->gmax, b->rel_min);
-    }
+            go(real, integral_constant<int, 0>{});
+    };
+    if (b->precision == FGA_PREC_FP64)
+        shape(double{});
+    else
+        shape(float{});
     FGA_CUDA(cudaGetLastError());
     return FGA_OK;
 }
