@@ -252,12 +252,10 @@ template <typename R> __device__ __forceinline__ C2<R> cmulsub(C2<R> a, C2<R> b,
 //   P: a' = gamma a;  S: a_sv' = gamma a_sv - a_sh w,  a_sh' = gamma a_sh + a_sv w,
 //      w = dN_sh/dt . N_sv = (e x P') . N_sv / |e x P|
 // ---------------------------------------------------------------------------------------------
-template <typename R, int WAVE, int MED>
-__device__ __forceinline__ void beam_rhs(const ModelDev &M, R sg, bool ref_e1, const R *__restrict__ y,
-                                         R *__restrict__ f) {
-    R cf[10];
-    const R Q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]};
-    model_eval<R, MED>(M, WAVE, Q, cf);
+// cf: the 10 model fields at the state's Q
+template <typename R, int WAVE>
+__device__ __forceinline__ void beam_rhs_at(const R cf[10], R sg, bool ref_e1, const R *__restrict__ y,
+                                            R *__restrict__ f) {
     const R c = cf[0];
     const R g[3] = {cf[1], cf[2], cf[3]};
     const R H[3][3] = {{cf[4], cf[5], cf[6]}, {cf[5], cf[7], cf[8]}, {cf[6], cf[8], cf[9]}};
@@ -277,25 +275,36 @@ __device__ __forceinline__ void beam_rhs(const ModelDev &M, R sg, bool ref_e1, c
         // FP32: each complex entry (re, im) as one packed FP32x2 value
         auto ld = [&](int off) { return make_float2(y[off], y[off + 1]); };
         auto bc = [](float v) { return make_float2(v, v); };
-        const float2 sgcip = bc(sg * cip), msgpn = bc(-sg * pn);
+        const float2 sgcip = bc(sg * cip), mcip = bc(-cip);
+        const float mp = -sg * pn;
+        float2 g2[3], P2[3], sP2[3], mg2[3], H2[3][3];   // H2: -sg |P| Hess c
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            g2[j] = bc(g[j]);
+            P2[j] = bc(Ph[j]);
+            sP2[j] = bc(sg * Ph[j]);
+            mg2[j] = bc(-sg * g[j]);
+#pragma unroll
+            for (int l = 0; l <= j; l++) H2[l][j] = H2[j][l] = bc(mp * H[l][j]);
+        }
 #pragma unroll
         for (int m = 0; m < 3; m++) {
-            float2 u = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f);
+            float2 q[3], d[3];
 #pragma unroll
             for (int l = 0; l < 3; l++) {
-                u = __ffma2_rn(ld(F_DQ + 2 * (3 * m + l)), bc(g[l]), u);
-                v = __ffma2_rn(ld(F_DP + 2 * (3 * m + l)), bc(Ph[l]), v);
+                q[l] = ld(F_DQ + 2 * (3 * m + l));
+                d[l] = ld(F_DP + 2 * (3 * m + l));
             }
-            const float2 wv = __ffma2_rn(bc(-cip), v, u);   // u - (c/|P|) v
+            const float2 u = __ffma2_rn(q[2], g2[2], __ffma2_rn(q[1], g2[1], __fmul2_rn(q[0], g2[0])));
+            const float2 v = __ffma2_rn(d[2], P2[2], __ffma2_rn(d[1], P2[1], __fmul2_rn(d[0], P2[0])));
+            const float2 wv = __ffma2_rn(mcip, v, u);   // u - (c/|P|) v
 #pragma unroll
             for (int j = 0; j < 3; j++) {
-                const float2 fq = __ffma2_rn(wv, bc(sg * Ph[j]), __fmul2_rn(sgcip, ld(F_DP + 2 * (3 * m + j))));
+                const float2 fq = __ffma2_rn(wv, sP2[j], __fmul2_rn(sgcip, d[j]));
                 f[F_DQ + 2 * (3 * m + j)] = fq.x;
                 f[F_DQ + 2 * (3 * m + j) + 1] = fq.y;
-                float2 hh = __fmul2_rn(ld(F_DQ + 2 * (3 * m)), bc(H[0][j]));
-                hh = __ffma2_rn(ld(F_DQ + 2 * (3 * m + 1)), bc(H[1][j]), hh);
-                hh = __ffma2_rn(ld(F_DQ + 2 * (3 * m + 2)), bc(H[2][j]), hh);
-                const float2 fp = __ffma2_rn(v, bc(-sg * g[j]), __fmul2_rn(msgpn, hh));
+                const float2 fp = __ffma2_rn(q[2], H2[2][j], __ffma2_rn(q[1], H2[1][j], __ffma2_rn(q[0], H2[0][j],
+                                             __fmul2_rn(v, mg2[j]))));
                 f[F_DP + 2 * (3 * m + j)] = fp.x;
                 f[F_DP + 2 * (3 * m + j) + 1] = fp.y;
             }
@@ -392,6 +401,15 @@ __device__ __forceinline__ void beam_rhs(const ModelDev &M, R sg, bool ref_e1, c
         f[F_A1] = gr * a1r - gi * a1i + om * a0r;
         f[F_A1 + 1] = gr * a1i + gi * a1r + om * a0i;
     }
+}
+
+template <typename R, int WAVE, int MED>
+__device__ __forceinline__ void beam_rhs(const ModelDev &M, R sg, bool ref_e1, const R *__restrict__ y,
+                                         R *__restrict__ f) {
+    R cf[10];
+    const R Q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]};
+    model_eval<R, MED>(M, WAVE, Q, cf);
+    beam_rhs_at<R, WAVE>(cf, sg, ref_e1, y, f);
 }
 
 // The same record from the end states and only the Q, P parts of the slopes (d0, d1: 6 values each

@@ -2,6 +2,7 @@
 // registers for all steps of a launch; reconstruction records written at sample times inside the
 // launch's steps.
 #include "fga_beam.cuh"
+#include "cell_cache.cuh"
 #include "straight.cuh"
 
 #include <algorithm>
@@ -10,9 +11,16 @@ namespace fga {
 
 // one record at index i of a buffer
 template <typename R> __device__ __forceinline__ void store_record(R *__restrict__ rec, int64_t i, const R r[REC]) {
-    R *dst = rec + i * REC;
+    // 48 or 96 bytes per record in 16-byte stores (the buffers are allocations of their own)
+    if constexpr (sizeof(R) == 4) {
+        float4 *dst = reinterpret_cast<float4 *>(rec + i * REC);
 #pragma unroll
-    for (int q = 0; q < REC; q++) dst[q] = r[q];
+        for (int q = 0; q < 3; q++) dst[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+    } else {
+        double2 *dst = reinterpret_cast<double2 *>(rec + i * REC);
+#pragma unroll
+        for (int q = 0; q < 6; q++) dst[q] = make_double2(r[2 * q], r[2 * q + 1]);
+    }
 }
 template <typename R> __device__ __forceinline__ float record_bound(const R r[REC]) {
     float m = 0.f;
@@ -41,6 +49,18 @@ template <typename R> __device__ __forceinline__ void axpy_state(R *out, const R
     } else {
 #pragma unroll
         for (int f = 0; f < NF; f++) out[f] = x[f] + h * kv[f];
+    }
+}
+
+// the same without Q (fields 3 .. N-1)
+template <int N> __device__ __forceinline__ void axpy_rest(float *out, const float *x, float h, const float *kv) {
+    const float2 h2 = make_float2(h, h);
+    out[3] = __fmaf_rn(h, kv[3], x[3]);
+#pragma unroll
+    for (int f = 4; f < N; f += 2) {
+        const float2 r = __ffma2_rn(h2, make_float2(kv[f], kv[f + 1]), make_float2(x[f], x[f + 1]));
+        out[f] = r.x;
+        out[f + 1] = r.y;
     }
 }
 
@@ -128,18 +148,139 @@ __global__ void __launch_bounds__(128) rk4_kernel(ModelDev M, R *__restrict__ st
     for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
 }
 
+// The classes' blocks of a beam set and of its records.
+struct ClassBlocks {
+    int64_t off[4], n[4];
+    int64_t n_in[4], rec_off[4];
+};
+
+// Grid media, FP32: the same RK4 loop with the model sampled through the cell cache and the position of the
+// next right-hand side formed as soon as this one's speed is known (the copies of new cells overlap with the rest
+// of it).  One launch for all classes (blockIdx.y the class), so that small beam sets fill the SMs once instead of
+// four times.  694 instructions per warp and right-hand side at 8 warps an SM (251 registers): the FMA pipe is
+// 55% busy, the issue slots 59%, the L1 data pipe 57% (rk4_kernel: 34%, 32%, 80% once the beams have spread).
+// Propagation, 200 steps: 0.44 M beams 21.5 -> 10.8 ms, 2.7 M beams 108.4 -> 65.1 ms; 8.4 M beams x 100 steps with
+// 250 samples 162 -> 112 ms.  Capped at 168 registers for 10 warps it spills: 113.6 ms on the 2.7 M beams.
+template <int WAVE>
+__device__ __forceinline__ void rk4_cell_body(const ModelDev &M, float *__restrict__ st, const int32_t *__restrict__ flags,
+                                              int64_t cap, const ClassBlocks &cc, int cls, float dt, int nsteps,
+                                              int n_samp, const int *__restrict__ samp_step,
+                                              const float *__restrict__ samp_theta, float w, float *__restrict__ rec,
+                                              int64_t rec_stride, unsigned *__restrict__ amax, float4 *smem) {
+    const int64_t n = cc.n[cls];
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int64_t b = cc.off[cls] + i;
+    const float sg = (cls & 1) ? -1.f : 1.f;
+    float y[NF], acc[NF], tmp[NF], kk[NF], qc[3];
+#pragma unroll
+    for (int f = 0; f < NF; f++) {
+        y[f] = WAVE || f < F_A1 ? st[(int64_t)f * cap + b] : 0.f;   // a P beam has one amplitude
+        acc[f] = y[f];
+        tmp[f] = y[f];
+    }
+#pragma unroll
+    for (int d = 0; d < 3; d++) qc[d] = st[(int64_t)(F_QC + d) * cap + b];
+    const bool ref_e1 = (flags[b] & FL_REF_E1) != 0;
+    CellCache cell;
+    cell.init(WAVE ? M.gs : M.gp, smem);
+    cell.prefetch(M, tmp);
+    constexpr int NW = WAVE ? NF : F_A1;   // fields that change
+    float s0[6];   // Q', P' at y_n (left slopes of the Hermite records)
+    int js = 0;
+    const float h2 = 0.5f * dt, h3 = dt / 3.f, h6 = dt / 6.f;
+    for (int it = -1; it < 4 * nsteps; it++) {
+        const int e = it & 3;
+        float cf[10];
+        cell.sample(cf);
+        const float ca = e < 2 ? h3 : h6;
+        const float ct = e == 0 ? h2 : (e == 1 ? dt : (e == 2 ? h6 : h2));
+        // Q of the next right-hand side (tq) and of y_{n+1} (qn), as in rk4_kernel
+        float tq[3], qn[3];
+        {
+            const float p2 = tmp[F_P] * tmp[F_P] + tmp[F_P + 1] * tmp[F_P + 1] + tmp[F_P + 2] * tmp[F_P + 2];
+            const float ip = rsqrtf(p2), sc = sg * cf[0];
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const float fq = sc * (tmp[F_P + d] * ip);
+                if (e < 2) {
+                    tq[d] = __fmaf_rn(ct, fq, y[F_Q + d]);
+                    acc[F_Q + d] = __fmaf_rn(ca, fq, acc[F_Q + d]);
+                } else if (e == 2) {
+                    acc[F_Q + d] = __fmaf_rn(ca, fq, acc[F_Q + d]);
+                    tq[d] = y[F_Q + d] + acc[F_Q + d];
+                } else {
+                    qn[d] = y[F_Q + d];
+                    if (it >= 0) kahan_add<float>(qn[d], qc[d], acc[F_Q + d]);
+                    tq[d] = __fmaf_rn(ct, fq, qn[d]);
+                    acc[F_Q + d] = ca * fq;   // the new step's increment so far
+                }
+            }
+        }
+        if (it + 1 < 4 * nsteps) cell.prefetch(M, tq);
+        beam_rhs_at<float, WAVE>(cf, sg, ref_e1, tmp, kk);
+        if (e == 3) {
+            const int step = it >> 2;
+            while (it >= 0 && js < n_samp && samp_step[js] == step) {
+                float mloc = 0.f;   // largest |A entry| of this thread's record
+                if (i < cc.n_in[cls]) {
+                    float y1[NF];   // y_{n+1}: acc with the compensated Q
+#pragma unroll
+                    for (int f = 0; f < NF; f++) y1[f] = f < 3 ? qn[f] : acc[f];
+                    float r[REC];
+                    beam_record6<float, WAVE>(ref_e1, y, s0, y1, kk, dt, samp_theta[js], w, r);
+                    store_record<float>(rec, (int64_t)js * rec_stride + cc.rec_off[cls] + i, r);
+                    mloc = record_bound<float>(r);
+                }
+                if (amax) sample_bound(amax + js, mloc);
+                js++;
+            }
+#pragma unroll
+            for (int f = 0; f < 6; f++) s0[f] = kk[f];
+#pragma unroll
+            for (int d = 0; d < 3; d++) y[F_Q + d] = qn[d];
+#pragma unroll
+            for (int f = 3; f < NF; f++) y[f] = acc[f];
+        }
+        // acc += ca kk;  tmp = base + ct kk, base = y (e = 0, 1) or acc before its update (e = 2, 3); Q is done
+        if (e < 2)
+            axpy_rest<NW>(tmp, y, ct, kk);
+        else
+            axpy_rest<NW>(tmp, acc, ct, kk);
+        axpy_rest<NW>(acc, acc, ca, kk);
+#pragma unroll
+        for (int d = 0; d < 3; d++) tmp[F_Q + d] = tq[d];
+    }
+#pragma unroll
+    for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
+#pragma unroll
+    for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
+}
+
+__global__ void __launch_bounds__(128) rk4_cell_kernel(ModelDev M, float *__restrict__ st, const int32_t *__restrict__ flags,
+                                                      int64_t cap, ClassBlocks cc, float dt, int nsteps, int n_samp,
+                                                      const int *__restrict__ samp_step,
+                                                      const float *__restrict__ samp_theta, float w,
+                                                      float *__restrict__ rec, int64_t rec_stride,
+                                                      unsigned *__restrict__ amax) {
+    extern __shared__ float4 cells[];
+    const int cls = blockIdx.y;
+    if (cls < 2)
+        rk4_cell_body<0>(M, st, flags, cap, cc, cls, dt, nsteps, n_samp, samp_step, samp_theta, w, rec, rec_stride, amax,
+                         cells);
+    else
+        rk4_cell_body<1>(M, st, flags, cap, cc, cls, dt, nsteps, n_samp, samp_step, samp_theta, w, rec, rec_stride, amax,
+                         cells);
+}
+
 // Constant media: nsteps RK4 steps in closed form (straight.cuh), one launch for all classes
 // (blockIdx.y the class).  Bound by the state's HBM stream in FP32 (49 reals read and 28 written per beam
 // and launch: P and dzP do not change) and by the FP64 pipe in FP64 (two reciprocals and ~80 operations a
 // step).  Against the general kernel's four right-hand sides per step: point-force experiment, 13.9 M beams
 // x 79 steps FP32, 63.7 -> 4.3 ms; homogeneous experiment, 373 k beams x 100 steps FP64, 126.7 -> 8.1 ms.
-struct ConstClasses {
-    int64_t off[4], n[4];
-    int64_t n_in[4], rec_off[4];
-};
 template <typename R>
 __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ st, const int32_t *__restrict__ flags,
-                                                   int64_t cap, ConstClasses cc, R dt, int nsteps, int n_samp,
+                                                   int64_t cap, ClassBlocks cc, R dt, int nsteps, int n_samp,
                                                    const int *__restrict__ samp_step, const R *__restrict__ samp_theta,
                                                    R w, R *__restrict__ rec, int64_t rec_stride,
                                                    unsigned *__restrict__ amax) {
@@ -216,9 +357,7 @@ __global__ void records_kernel(const R *__restrict__ st, const int32_t *__restri
     for (int d = 0; d < 3; d++) y[F_Q + d] -= st[(int64_t)(F_QC + d) * cap + b];   // compensated Q
     R r[REC];
     beam_record<R, WAVE>((flags[b] & FL_REF_E1) != 0, y, y, y, y, R(0), R(0), w, r);
-    R *dst = rec + i * REC;
-#pragma unroll
-    for (int q = 0; q < REC; q++) dst[q] = r[q];
+    store_record<R>(rec, i, r);
 }
 
 template <typename R, int WAVE, int MED>
@@ -248,17 +387,23 @@ static void launch_med(const fga_model *m, fga_beams *b, R dt, int nsteps, const
     }
 }
 
-template <typename R>
-static void launch_const(const fga_model *m, fga_beams *b, R dt, int nsteps, const SampleWindow *sw, cudaStream_t s) {
-    ConstClasses cc{};
-    int64_t most = 0;
+static ClassBlocks class_blocks(const fga_beams *b, const SampleWindow *sw, int64_t *most) {
+    ClassBlocks cc{};
+    *most = 0;
     for (int c = 0; c < 4; c++) {
         cc.off[c] = b->off_cls[c];
         cc.n[c] = b->n_cls[c];
         cc.n_in[c] = sw ? sw->n_in[c] : 0;
         cc.rec_off[c] = sw ? sw->rec_off[c] : 0;
-        most = std::max(most, cc.n[c]);
+        *most = std::max(*most, cc.n[c]);
     }
+    return cc;
+}
+
+template <typename R>
+static void launch_const(const fga_model *m, fga_beams *b, R dt, int nsteps, const SampleWindow *sw, cudaStream_t s) {
+    int64_t most;
+    const ClassBlocks cc = class_blocks(b, sw, &most);
     if (most == 0) return;
     prof_add_beam_steps(b->nb * (int64_t)nsteps);
     ProfScope ps(P_PROP, s);
@@ -270,12 +415,33 @@ static void launch_const(const fga_model *m, fga_beams *b, R dt, int nsteps, con
                                          (sw && sizeof(R) == 4) ? sw->amax : nullptr);
 }
 
+static fga_status launch_grid_f32(const fga_model *m, fga_beams *b, float dt, int nsteps, const SampleWindow *sw,
+                                  cudaStream_t s) {
+    int64_t most;
+    const ClassBlocks cc = class_blocks(b, sw, &most);
+    if (most == 0) return FGA_OK;
+    prof_add_beam_steps(b->nb * (int64_t)nsteps);
+    ProfScope ps(P_PROP, s);
+    const dim3 grid((unsigned)((most + 127) / 128), 4);
+    const int smem = 128 * CELL_STRIDE * (int)sizeof(float4);
+    FGA_CUDA(cudaFuncSetAttribute(rk4_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    rk4_cell_kernel<<<grid, 128, smem, s>>>(m->dev, b->state.as<float>(), b->flags.as<int32_t>(), b->cap, cc, dt, nsteps,
+                                            sw ? sw->n : 0, sw ? sw->step : nullptr,
+                                            sw ? static_cast<const float *>(sw->theta) : nullptr, (float)b->w,
+                                            sw ? static_cast<float *>(sw->rec) : nullptr, sw ? sw->n_rec : 0,
+                                            sw ? sw->amax : nullptr);
+    return FGA_OK;
+}
+
 template <typename R>
 static void launch_prec(const fga_model *m, fga_beams *b, R dt, int nsteps, const SampleWindow *sw, cudaStream_t s) {
     switch (m->dev.kind) {
     case FGA_MEDIUM_CONST: launch_const<R>(m, b, dt, nsteps, sw, s); break;
     case FGA_MEDIUM_SINE: launch_med<R, FGA_MEDIUM_SINE>(m, b, dt, nsteps, sw, s); break;
-    case FGA_MEDIUM_GRID: launch_med<R, FGA_MEDIUM_GRID>(m, b, dt, nsteps, sw, s); break;
+    case FGA_MEDIUM_GRID:
+        // FP32 grid media take launch_grid_f32
+        if constexpr (sizeof(R) == 8) launch_med<R, FGA_MEDIUM_GRID>(m, b, dt, nsteps, sw, s);
+        break;
     default: break;   // layered media advance by launch_layered_steps
     }
 }
@@ -285,6 +451,8 @@ fga_status launch_propagate(const fga_model *m, fga_beams *b, double dt, int nst
     if (nsteps <= 0 && (!sw || sw->n == 0)) return FGA_OK;
     if (b->precision == FGA_PREC_FP64)
         launch_prec<double>(m, b, dt, nsteps, sw, s);
+    else if (m->dev.kind == FGA_MEDIUM_GRID)
+        FGA_TRY(launch_grid_f32(m, b, (float)dt, nsteps, sw, s));
     else
         launch_prec<float>(m, b, (float)dt, nsteps, sw, s);
     FGA_CUDA(cudaGetLastError());
