@@ -670,7 +670,7 @@ static fga_status reconstruct_lattice_now(const fga_beams *b, const fga_lattice 
     const size_t rb = b->precision == FGA_PREC_FP64 ? 8 : 4;
     FGA_TRY(ws.rec.ensure(rb * REC * (size_t)std::max<int64_t>(plan.n_rec, 1)));
     FGA_TRY(launch_records_from_state(b, perm, plan.beg, plan.n_in, plan.rec_off, ws.rec.p, s));
-    return run_lattice(ws, plan, b->precision, ws.rec.p, b->k, rw, u_out, s, P_GATHER_STATE);
+    return run_lattice(ws, plan, b->precision, ws.rec.p, 0, 1, b->k, rw, u_out, 0, s, P_GATHER_STATE);
 }
 
 fga_status fga_reconstruct_lattice(const fga_beams *b, const fga_lattice *lat, double rw, void *u_out,
@@ -939,15 +939,15 @@ fga_status solve_impl(const fga_model *m, const fga_init_desc *init, const fga_s
             FGA_TRY(launch_propagate(m, b, sd->dt, nw, &sw, s));
         }
         NvtxRange nr_sums("fga_solve: sums");
-        for (int j = 0; j < ns; j++) {
-            void *out = static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)(js + j);
-            const void *rec = static_cast<const char *>(ws.rec.p) + (size_t)per_sample * j;
-            if (rxL)
-                FGA_TRY(run_lattice(ws, lplan, b->precision, rec, b->k, rw, out, s, P_GATHER,
-                                    amax ? reinterpret_cast<const float *>(amax + j) : nullptr));
-            else
-                FGA_TRY(run_sum(ws, plan, b->precision, rec, sd->rx, b->k, rw, out, s));
-        }
+        if (rxL)
+            FGA_TRY(run_lattice(ws, lplan, b->precision, ws.rec.p, per_sample / (int64_t)rb, ns, b->k, rw,
+                                static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)js, 6 * nrx, s, P_GATHER,
+                                amax ? reinterpret_cast<const float *>(amax) : nullptr));
+        else
+            for (int j = 0; j < ns; j++)
+                FGA_TRY(run_sum(ws, plan, b->precision, static_cast<const char *>(ws.rec.p) + (size_t)per_sample * j,
+                                sd->rx, b->k, rw, static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)(js + j),
+                                s));
         js = j1;
         n0 += nw;
     }

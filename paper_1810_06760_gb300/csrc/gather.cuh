@@ -27,6 +27,7 @@ struct LatticePlan {
     int ntiles = 0, nitems = 0;
     const double *ax[3] = {nullptr, nullptr, nullptr};  // DEVICE axis coordinates
     const int32_t *item_start = nullptr;
+    const int32_t *h_item_start = nullptr;   // HOST copy (in the workspace)
     const int4 *items = nullptr;
     int64_t pairs_tested = 0;
     int64_t n_in[4] = {0, 0, 0, 0}, rec_off[4] = {0, 0, 0, 0}, n_rec = 0, beg[4] = {0, 0, 0, 0};
@@ -51,9 +52,11 @@ void tile_shape_tc(const fga_lattice &L, int T[3]);
 // single-plane lattices with uniform axes 0 and 1: the warp-specialised plane kernel (tc_plane.cu)
 void tile_shape_plane(const fga_lattice &L, int T[3]);
 bool plane_tc_eligible(const LatticePlan &plan);
-// amax: DEVICE bound of the records' |A| entries (bits of a non-negative float), or NULL to compute it
-fga_status run_plane_tc(Workspace &ws, const LatticePlan &plan, const void *rec, double k, double rw, void *u,
-                        cudaStream_t s, int cat, const float *amax = nullptr);
+constexpr size_t PLANE_PARTIAL_MAX = (size_t)256 << 20;   // bytes of the plane kernel's partial sums
+// ns samples in one launch, their records rec_stride reals apart and their outputs u_stride reals apart; amax:
+// DEVICE bounds of the samples' |A| entries (bits of a non-negative float), or NULL to compute the bound (ns = 1)
+fga_status run_plane_tc(Workspace &ws, const LatticePlan &plan, const void *rec, int64_t rec_stride, int ns, double k,
+                        double rw, void *u, int64_t u_stride, cudaStream_t s, int cat, const float *amax = nullptr);
 int64_t read_plane_pair_counter(bool reset);
 // |A| bound of n records into *out (zeroed by the caller)
 fga_status rec_absmax(const float *rec, int64_t n, float *out, cudaStream_t s, int cat);
@@ -71,8 +74,10 @@ fga_status flag_nonfinite(Workspace &ws, const void *data, int64_t n, int precis
 // the same for nf fields of nb beams stored with stride cap
 fga_status flag_nonfinite_state(Workspace &ws, const void *st, int64_t cap, int64_t nb, int nf, int precision,
                                 cudaStream_t s);
-fga_status run_lattice(Workspace &ws, const LatticePlan &plan, int precision, const void *rec, double k, double rw,
-                       void *u, cudaStream_t s, int cat = P_GATHER, const float *amax = nullptr);
+// ns samples (rec_stride, u_stride: reals between them; amax as for run_plane_tc)
+fga_status run_lattice(Workspace &ws, const LatticePlan &plan, int precision, const void *rec, int64_t rec_stride, int ns,
+                       double k, double rw, void *u, int64_t u_stride, cudaStream_t s, int cat = P_GATHER,
+                       const float *amax = nullptr);
 int64_t read_lattice_pair_counter(bool reset);
 
 fga_status sort_keys_to_perm(Workspace &ws, int32_t *keys, int64_t n, int nbuckets, int32_t **perm_out,

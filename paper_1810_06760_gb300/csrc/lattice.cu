@@ -334,16 +334,16 @@ bool recurrence_ratio_ok(double k, double step, double span, double rw) {
     return k * std::fabs(step) * (span + rw + std::fabs(step)) <= 87.0;
 }
 
-// the plane kernel's runs: axis 1 in two halves of ceil(T1/2) points (step h1), axis 0 in the two
-// parities of ceil(T0/2) points (step 2 h0); cap T so every run stays within the recurrence limits
+// the plane kernel's runs: the quarters of ceil(T/4) points of each axis (one point up to T = 4, without a
+// ratio); cap T so that every run stays within the recurrence limits.  A kept beam can lie rw beyond the far end
+// of the whole tile, so the ratio's bound takes the tile's span.
 static void cap_plane_tile(const LatticePlan &plan, double k, double rw, int T[3]) {
     const double smax = recurrence_span_max(k, rw);
     for (int d = 0; d < 2; d++) {
-        if (T[d] <= 2 || !plan.uniform[d]) continue;
-        const double step = (d == 0 ? 2.0 : 1.0) * std::fabs(plan.dx[d]);
-        int J = 1 + (int)std::floor(smax / step);
-        while (J > 1 && !recurrence_ratio_ok(k, step, (J - 1) * step, rw)) J--;
-        T[d] = std::min(T[d], 2 * J);
+        if (T[d] <= 4 || !plan.uniform[d]) continue;
+        const double step = std::fabs(plan.dx[d]);
+        T[d] = (int)std::min<double>(T[d], 4.0 * (1.0 + std::floor(smax / step)));
+        while (T[d] > 4 && !recurrence_ratio_ok(k, step, (T[d] - 1) * step, rw)) T[d]--;
     }
 }
 
@@ -464,6 +464,7 @@ fga_status build_lattice_plan(Workspace &ws, const BinGrid &g, const int32_t *ce
     plan.ax[1] = dax + L.n[0];
     plan.ax[2] = dax + L.n[0] + L.n[1];
     plan.item_start = reinterpret_cast<const int32_t *>(ws.tiles.as<char>() + axb);
+    plan.h_item_start = reinterpret_cast<const int32_t *>(h + axb);
     plan.items = ws.items.as<int4>();
     return FGA_OK;
 }
@@ -532,12 +533,20 @@ fga_status lattice_reduce_f32(const float *partial, const LatticePlan &plan, voi
     return FGA_OK;
 }
 
-// FP32: the tensor-core kernel (plans built with tc = true); FP64: the CUDA-core kernel
-fga_status run_lattice(Workspace &ws, const LatticePlan &plan, int precision, const void *rec, double k, double rw,
-                       void *u, cudaStream_t s, int cat, const float *amax) {
-    if (precision == FGA_PREC_FP64) return run_lattice_t<double>(ws, plan, rec, k, rw, u, s, cat);
-    if (plane_tc_eligible(plan)) return run_plane_tc(ws, plan, rec, k, rw, u, s, cat, amax);
-    return run_lattice_tc(ws, plan, rec, k, rw, u, s, cat, amax);
+// FP32: the tensor-core kernels (plans built with tc = true); FP64: the CUDA-core kernel
+fga_status run_lattice(Workspace &ws, const LatticePlan &plan, int precision, const void *rec, int64_t rec_stride, int ns,
+                       double k, double rw, void *u, int64_t u_stride, cudaStream_t s, int cat, const float *amax) {
+    if (precision != FGA_PREC_FP64 && plane_tc_eligible(plan))
+        return run_plane_tc(ws, plan, rec, rec_stride, ns, k, rw, u, u_stride, s, cat, amax);
+    for (int j = 0; j < ns; j++) {
+        if (precision == FGA_PREC_FP64)
+            FGA_TRY(run_lattice_t<double>(ws, plan, static_cast<const double *>(rec) + rec_stride * j, k, rw,
+                                          static_cast<double *>(u) + u_stride * j, s, cat));
+        else
+            FGA_TRY(run_lattice_tc(ws, plan, static_cast<const float *>(rec) + rec_stride * j, k, rw,
+                                   static_cast<float *>(u) + u_stride * j, s, cat, amax ? amax + j : nullptr));
+    }
+    return FGA_OK;
 }
 
 }  // namespace fga

@@ -41,6 +41,18 @@ __device__ __forceinline__ uint64_t smem_desc_lbo_sbo(uint32_t saddr, uint32_t l
     return d;
 }
 
+// K-major operand of K extent 16 (rows of 32 bytes) in the 32-byte swizzle: within a group of 8 rows (256
+// bytes, SBO; groups contiguous) the two 16-byte halves of rows 4..7 are exchanged.  Base 256-byte aligned.
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+    d |= (uint64_t)1 << 16;            // leading offset: not used with one swizzle atom along K
+    d |= (uint64_t)(256 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)6 << 61;            // 32-byte swizzle
+    return d;
+}
+
 // instruction descriptor: D f32, A and B f16, both K-major, N and M
 __device__ __forceinline__ uint32_t instr_desc(int n, int m) {
     uint32_t d = 0;
@@ -139,6 +151,10 @@ __device__ __forceinline__ void alloc(uint32_t slot, uint32_t cols) {
 }
 __device__ __forceinline__ void dealloc(uint32_t tmem, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void mbar_init_n(uint32_t bar, uint32_t n) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
