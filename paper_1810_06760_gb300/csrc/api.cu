@@ -575,11 +575,11 @@ static fga_status reconstruct_now(const fga_beams *b, const double *x_dev, const
     int32_t *perm = nullptr;
     FGA_TRY(bin_beams(b, g, &perm, s));
     SumPlan plan;
-    FGA_TRY(build_sum_plan(ws, g, ws.cell_start.as<int32_t>(), 4, xh.data(), n, s, plan));  // syncs
+    FGA_TRY(build_sum_plan(ws, g, ws.cell_start.as<int32_t>(), 4, xh.data(), n, 1, s, plan));  // syncs
     const size_t rb = b->precision == FGA_PREC_FP64 ? 8 : 4;
     FGA_TRY(ws.rec.ensure(rb * REC * (size_t)std::max<int64_t>(plan.n_rec, 1)));
     FGA_TRY(launch_records_from_state(b, perm, plan.beg, plan.n_in, plan.rec_off, ws.rec.p, s));
-    return run_sum(ws, plan, b->precision, ws.rec.p, x_dev, b->k, rw, u_out, s, P_GATHER_STATE);
+    return run_sum(ws, plan, b->precision, ws.rec.p, 0, 1, x_dev, b->k, rw, u_out, 0, s, P_GATHER_STATE);
 }
 
 static fga_status check_lattice(const fga_lattice *L, const char *who) {
@@ -898,7 +898,7 @@ fga_status solve_impl(const fga_model *m, const fga_init_desc *init, const fga_s
             }
             plan.n_rec = lplan.n_rec;
         } else {
-            FGA_TRY(build_sum_plan(ws, grx, ws.cell_start.as<int32_t>(), 4, rxh.data(), sd->n_rx, s, plan));  // syncs
+            FGA_TRY(build_sum_plan(ws, grx, ws.cell_start.as<int32_t>(), 4, rxh.data(), sd->n_rx, j1 - js, s, plan));  // syncs
         }
         // shorten the window so that its samples' records fit the budget (a shorter window keeps the
         // cell margin valid)
@@ -944,10 +944,8 @@ fga_status solve_impl(const fga_model *m, const fga_init_desc *init, const fga_s
                                 static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)js, 6 * nrx, s, P_GATHER,
                                 amax ? reinterpret_cast<const float *>(amax) : nullptr));
         else
-            for (int j = 0; j < ns; j++)
-                FGA_TRY(run_sum(ws, plan, b->precision, static_cast<const char *>(ws.rec.p) + (size_t)per_sample * j,
-                                sd->rx, b->k, rw, static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)(js + j),
-                                s));
+            FGA_TRY(run_sum(ws, plan, b->precision, ws.rec.p, per_sample / (int64_t)rb, ns, sd->rx, b->k, rw,
+                            static_cast<char *>(seis_out) + rb * 6 * (size_t)nrx * (size_t)js, 6 * nrx, s));
         js = j1;
         n0 += nw;
     }

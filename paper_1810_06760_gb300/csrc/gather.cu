@@ -381,14 +381,17 @@ int64_t read_pair_counter(bool reset) {
     return (int64_t)v;
 }
 
+// FP64 (R = double): one beam at a time, every lane its point
 template <typename R>
-__global__ void __launch_bounds__(128) gather_kernel(const R *__restrict__ rec, const double *__restrict__ pts,
+__global__ void __launch_bounds__(128) gather_kernel(const R *__restrict__ rec, int64_t rec_stride,
+                                                    const double *__restrict__ pts,
                                                     const int32_t *__restrict__ tile_pts, const int4 *__restrict__ items,
                                                     R k, R rw2, R *__restrict__ partial, int count_pairs) {
     __shared__ R red[4][32][6];
     __shared__ unsigned npairs;
     if (threadIdx.x == 0) npairs = 0;
     unsigned mine = 0;
+    rec += blockIdx.y * rec_stride;
     const int4 it = items[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int pi = tile_pts[it.x * 32 + lane];
@@ -407,20 +410,12 @@ __global__ void __launch_bounds__(128) gather_kernel(const R *__restrict__ rec, 
     for (int64_t b = b0; b < b1; b++) {
         const R *r = rec + b * REC;
         R q[REC];
-        if (sizeof(R) == 4) {
-            const float4 *r4 = reinterpret_cast<const float4 *>(r);
-            const float4 u0 = __ldg(r4), u1 = __ldg(r4 + 1), u2 = __ldg(r4 + 2);
-            const float t[12] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w, u2.x, u2.y, u2.z, u2.w};
+        const double2 *r2p = reinterpret_cast<const double2 *>(r);
 #pragma unroll
-            for (int j = 0; j < REC; j++) q[j] = (R)t[j];
-        } else {
-            const double2 *r2 = reinterpret_cast<const double2 *>(r);
-#pragma unroll
-            for (int j = 0; j < 6; j++) {
-                const double2 v = __ldg(r2 + j);
-                q[2 * j] = (R)v.x;
-                q[2 * j + 1] = (R)v.y;
-            }
+        for (int j = 0; j < 6; j++) {
+            const double2 v = __ldg(r2p + j);
+            q[2 * j] = v.x;
+            q[2 * j + 1] = v.y;
         }
         const R d0 = x0 - q[0], d1 = x1 - q[1], d2 = x2 - q[2];
         const R r2 = d0 * d0 + d1 * d1 + d2 * d2;
@@ -442,29 +437,162 @@ __global__ void __launch_bounds__(128) gather_kernel(const R *__restrict__ rec, 
 #pragma unroll
         for (int j = 0; j < 6; j++) {
             const R v = (red[0][lane][j] + red[1][lane][j]) + (red[2][lane][j] + red[3][lane][j]);
-            partial[((int64_t)blockIdx.x * 32 + lane) * 6 + j] = v;
+            partial[(((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 32 + lane) * 6 + j] = v;
         }
     }
 }
 
+// The same sum in FP32.  A warp takes 32 points of the tile and a quarter of the item's beams, staged 32 at a time
+// in shared memory field by field (the next 32 in flight in registers), so that two consecutive beams are the two
+// halves of packed FP32x2 operands: coordinates and accumulators are packed once, and a pair of beams costs 30
+// packed FMAs, 6 MUFU and 12 other instructions for 64 (beam, point) pairs.  Bound by the FMA pipe (62 cycles a
+// warp and 64 pairs; MUFU 48).  Against one beam and point per lane with uniform loads (41 instructions per 32
+// pairs, long-scoreboard stalls): 1.05 M beams x 5,003 points 8.2 -> 5.3 ms, 100
+// samples of 256 receivers and 1.05 M beams 43.0 -> 21.2 ms (issue slots 65%, FMA pipe 55%).
+constexpr int GF_BEAMS = 32;
+__global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict__ rec, int64_t rec_stride,
+                                                         const double *__restrict__ pts,
+                                                         const int32_t *__restrict__ tile_pts,
+                                                         const int4 *__restrict__ items, float k, float rw2,
+                                                         float *__restrict__ partial, int count_pairs) {
+    __shared__ float stage[4][2][REC][GF_BEAMS];
+    __shared__ float red[4][32][6];
+    __shared__ unsigned npairs;
+    if (threadIdx.x == 0) npairs = 0;
+    const int4 it = items[blockIdx.x];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int pi = tile_pts[it.x * 32 + lane];
+    // padding lanes sit far away: no beam is in their window
+    const float x0 = pi >= 0 ? (float)pts[3 * (int64_t)pi] : 1e15f, x1 = pi >= 0 ? (float)pts[3 * (int64_t)pi + 1] : 1e15f,
+                x2 = pi >= 0 ? (float)pts[3 * (int64_t)pi + 2] : 1e15f;
+    const float2 X0 = make_float2(x0, x0), X1 = make_float2(x1, x1), X2 = make_float2(x2, x2);
+    const int64_t len = (int64_t)it.z - it.y;
+    const int64_t b0 = it.y + (len * warp) / 4, b1 = it.y + (len * (warp + 1)) / 4;
+    const float *r0 = rec + blockIdx.y * rec_stride;
+    const float hk2 = -0.72134752044448170368f * k;   // -k/2 in units of log 2
+    constexpr double TWO_PI = 6.283185307179586476925286766559;
+    constexpr float TP_HI = (float)TWO_PI, TP_LO = (float)(TWO_PI - (double)TP_HI), INV_TP = (float)(1.0 / TWO_PI);
+    constexpr float MAGIC = 12582912.f;   // 1.5 x 2^23: adding and subtracting it rounds to an integer
+    auto bc = [](float v) { return make_float2(v, v); };
+    float2 acc[6];
+#pragma unroll
+    for (int j = 0; j < 6; j++) acc[j] = bc(0.f);
+    unsigned mine = 0;
+    float4 n0, n1, n2;
+    // lane's record of the 32 from b; a padding beam lies outside every window
+    auto fetch = [&](int64_t b) {
+        if (b + lane < b1) {
+            const float4 *p = reinterpret_cast<const float4 *>(r0 + (b + lane) * REC);
+            n0 = __ldg(p);
+            n1 = __ldg(p + 1);
+            n2 = __ldg(p + 2);
+        } else {
+            n0 = make_float4(-1e15f, -1e15f, -1e15f, 0.f);
+            n1 = n2 = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    fetch(b0);
+    int buf = 0;
+    for (int64_t b = b0; b < b1; b += GF_BEAMS, buf ^= 1) {
+        float(*st)[GF_BEAMS] = stage[warp][buf];
+        st[0][lane] = -n0.x;
+        st[1][lane] = -n0.y;
+        st[2][lane] = -n0.z;
+        st[3][lane] = k * n0.w;
+        st[4][lane] = k * n1.x;
+        st[5][lane] = k * n1.y;
+        st[6][lane] = n1.z;
+        st[7][lane] = n1.w;
+        st[8][lane] = n2.x;
+        st[9][lane] = n2.y;
+        st[10][lane] = n2.z;
+        st[11][lane] = n2.w;
+        __syncwarp();   // the other half was last read before the previous synchronisation of this kind
+        if (b + GF_BEAMS < b1) fetch(b + GF_BEAMS);
+        const int nb = (int)(b1 - b < GF_BEAMS ? b1 - b : GF_BEAMS);
+        for (int j = 0; j < nb; j += 4) {
+            float4 f[6];
+#pragma unroll
+            for (int c = 0; c < 6; c++) f[c] = *reinterpret_cast<const float4 *>(&st[c][j]);
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                auto pr = [&](const float4 &v) { return h ? make_float2(v.z, v.w) : make_float2(v.x, v.y); };
+                const float2 d0 = __fadd2_rn(X0, pr(f[0])), d1 = __fadd2_rn(X1, pr(f[1])), d2 = __fadd2_rn(X2, pr(f[2]));
+                const float2 r2 = __ffma2_rn(d2, d2, __ffma2_rn(d1, d1, __fmul2_rn(d0, d0)));
+                const bool in0 = r2.x <= rw2, in1 = r2.y <= rw2;
+                if (!__any_sync(0xffffffffu, in0 || in1)) continue;
+                mine += (in0 ? 1u : 0u) + (in1 ? 1u : 0u);
+                const float2 ph = __ffma2_rn(pr(f[5]), d2, __ffma2_rn(pr(f[4]), d1, __fmul2_rn(pr(f[3]), d0)));
+                // Cody-Waite reduction of the phase by 2 pi (two-part constant)
+                const float2 n = __fadd2_rn(__ffma2_rn(ph, bc(INV_TP), bc(MAGIC)), bc(-MAGIC));
+                const float2 r = __ffma2_rn(n, bc(-TP_LO), __ffma2_rn(n, bc(-TP_HI), ph));
+                const float2 am = __fmul2_rn(r2, bc(hk2));
+                float2 e, s, c;
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(am.x));
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(am.y));
+                __sincosf(r.x, &s.x, &c.x);
+                __sincosf(r.y, &s.y, &c.y);
+                e.x = in0 ? e.x : 0.f;
+                e.y = in1 ? e.y : 0.f;
+                const float2 er = __fmul2_rn(e, c), ei = __fmul2_rn(e, s), mi = make_float2(-ei.x, -ei.y);
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const float2 ar = *reinterpret_cast<const float2 *>(&st[6 + 2 * d][j + 2 * h]);
+                    const float2 ai = *reinterpret_cast<const float2 *>(&st[7 + 2 * d][j + 2 * h]);
+                    acc[2 * d] = __ffma2_rn(ai, mi, __ffma2_rn(ar, er, acc[2 * d]));
+                    acc[2 * d + 1] = __ffma2_rn(ai, er, __ffma2_rn(ar, ei, acc[2 * d + 1]));
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 6; j++) red[warp][lane][j] = acc[j].x + acc[j].y;
+    __syncthreads();
+    if (count_pairs) {
+        atomicAdd(&npairs, mine);
+        __syncthreads();
+        if (threadIdx.x == 0) atomicAdd(&g_pairs_in_window, (unsigned long long)npairs);
+    }
+    if (warp == 0) {
+        float *dst = partial + (((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 32 + lane) * 6;
+#pragma unroll
+        for (int j = 0; j < 6; j++) dst[j] = (red[0][lane][j] + red[1][lane][j]) + (red[2][lane][j] + red[3][lane][j]);
+    }
+}
+
+// u at the points of a tile (blockIdx.x) and sample (blockIdx.y): RD_WARPS warps stride over the tile's items, then
+// their FP64 sums are added in a fixed order.  (A single warp per tile walked thousands of items alone: 100 samples of
+// 256 receivers and 1.05 M beams 17.0 -> 0.5 ms.)
+constexpr int RD_WARPS = 16;
 template <typename R>
-__global__ void reduce_kernel(const R *__restrict__ partial, const int32_t *__restrict__ tile_pts,
-                              const int32_t *__restrict__ item_start, int ntiles, R *__restrict__ u) {
-    const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x & 31;
-    if (t >= ntiles) return;
+__global__ void __launch_bounds__(32 * RD_WARPS) reduce_kernel(const R *__restrict__ partial,
+                                                              const int32_t *__restrict__ tile_pts,
+                                                              const int32_t *__restrict__ item_start, int nitems,
+                                                              R *__restrict__ u, int64_t u_stride) {
+    __shared__ double sh[RD_WARPS][6][32];
+    const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const R *p = partial + ((int64_t)blockIdx.y * nitems * 32 + lane) * 6;
+    double acc[6] = {0, 0, 0, 0, 0, 0};
+    for (int i = item_start[t] + warp; i < item_start[t + 1]; i += RD_WARPS)
+#pragma unroll
+        for (int j = 0; j < 6; j++) acc[j] += (double)p[(int64_t)i * 192 + j];
+#pragma unroll
+    for (int j = 0; j < 6; j++) sh[warp][j][lane] = acc[j];
+    __syncthreads();
+    if (warp > 0) return;
     const int pi = tile_pts[t * 32 + lane];
     if (pi < 0) return;
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = item_start[t]; i < item_start[t + 1]; i++)
+    R *dst = u + blockIdx.y * u_stride + (int64_t)pi * 6;
 #pragma unroll
-        for (int j = 0; j < 6; j++) acc[j] += (double)partial[((int64_t)i * 32 + lane) * 6 + j];
+    for (int j = 0; j < 6; j++) {
 #pragma unroll
-    for (int j = 0; j < 6; j++) u[(int64_t)pi * 6 + j] = (R)acc[j];
+        for (int w = 1; w < RD_WARPS; w++) acc[j] += sh[w][j][lane];
+        dst[j] = (R)acc[j];
+    }
 }
 
 fga_status build_sum_plan(Workspace &ws, const BinGrid &g, const int32_t *cell_start_dev, int nclasses,
-                          const double *pts_host, int64_t npts, cudaStream_t s, SumPlan &plan) {
+                          const double *pts_host, int64_t npts, int samples, cudaStream_t s, SumPlan &plan) {
     plan.ntiles = 0;
     plan.nitems = 0;
     if (npts == 0) return FGA_OK;
@@ -537,8 +665,12 @@ fga_status build_sum_plan(Workspace &ws, const BinGrid &g, const int32_t *cell_s
                 }
         }
     }
-    // chunk size: aim at >= ~4096 work items so that every SM has several CTAs
-    int64_t B = std::max<int64_t>(512, (total + 4095) / 4096);
+    // chunk size: work items of at least 512 beams, up to ~16384 of them for one sample (some 15 waves of the
+    // ~1064 resident CTAs, so that the last wave's idle share is small: 4096 items are 6.2 waves, 5.73 against
+    // 5.33 ms on 1.05 M beams x 5,003 points) and up to ~4096 a sample for several in one launch (fewer partial
+    // sums: reductions of 100 samples 0.5 against 1.7 ms)
+    const int64_t most = samples < 4 ? 16384 : 4096;
+    int64_t B = std::max<int64_t>(512, (total + most - 1) / most);
     B = (B + 127) / 128 * 128;
     std::vector<int32_t> item_start((size_t)ntiles + 1, 0);
     std::vector<int4> items;
@@ -574,34 +706,41 @@ fga_status build_sum_plan(Workspace &ws, const BinGrid &g, const int32_t *cell_s
 
 const int32_t *plan_host_cell_start(const Workspace &ws) { return ws.h_cell_start.as<int32_t>(); }
 
-fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void *rec_sorted, const double *pts_dev,
-                   double k, double rw, void *u_out, cudaStream_t s, int cat) {
+fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void *rec, int64_t rec_stride, int ns,
+                   const double *pts_dev, double k, double rw, void *u_out, int64_t u_stride, cudaStream_t s, int cat) {
     if (plan.ntiles == 0) return FGA_OK;
     const size_t rb = precision == FGA_PREC_FP64 ? 8 : 4;
-    FGA_TRY(ws.partial.ensure(rb * 32 * 6 * (size_t)std::max(plan.nitems, 1)));
+    // as many samples per launch as keep the partial sums under SUM_PARTIAL_MAX bytes
+    const size_t per_sample = rb * 32 * 6 * (size_t)std::max(plan.nitems, 1);
+    const int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)ns, SUM_PARTIAL_MAX / per_sample, 65535}));
+    FGA_TRY(ws.partial.ensure(per_sample * (size_t)chunk));
     const int cnt = prof_counting() ? 1 : 0;
-    prof_add_pairs_tested(plan.pairs_tested);
-    if (plan.nitems > 0) {
-        ProfScope ps(cat, s);
+    prof_add_pairs_tested(plan.pairs_tested * ns);
+    for (int s0 = 0; s0 < ns; s0 += chunk) {
+        const int m = std::min(chunk, ns - s0);
+        if (plan.nitems > 0) {
+            ProfScope ps(cat, s);
+            const dim3 grid((unsigned)plan.nitems, (unsigned)m);
+            if (rb == 8)
+                gather_kernel<double><<<grid, 128, 0, s>>>((const double *)rec + rec_stride * s0, rec_stride, pts_dev,
+                                                           plan.tile_pts, plan.items, k, rw * rw, ws.partial.as<double>(),
+                                                           cnt);
+            else
+                gather_f32_kernel<<<grid, 128, 0, s>>>((const float *)rec + rec_stride * s0, rec_stride, pts_dev,
+                                                       plan.tile_pts, plan.items, (float)k, (float)(rw * rw),
+                                                       ws.partial.as<float>(), cnt);
+            FGA_CUDA(cudaGetLastError());
+        }
+        ProfScope ps(P_REDUCE, s);
+        const dim3 grid((unsigned)plan.ntiles, (unsigned)m);
         if (rb == 8)
-            gather_kernel<double><<<plan.nitems, 128, 0, s>>>((const double *)rec_sorted, pts_dev, plan.tile_pts,
-                                                              plan.items, k, rw * rw, ws.partial.as<double>(), cnt);
+            reduce_kernel<double><<<grid, 32 * RD_WARPS, 0, s>>>(ws.partial.as<double>(), plan.tile_pts, plan.item_start,
+                                                                 plan.nitems, (double *)u_out + u_stride * s0, u_stride);
         else
-            gather_kernel<float><<<plan.nitems, 128, 0, s>>>((const float *)rec_sorted, pts_dev, plan.tile_pts,
-                                                             plan.items, (float)k, (float)(rw * rw), ws.partial.as<float>(),
-                                                             cnt);
+            reduce_kernel<float><<<grid, 32 * RD_WARPS, 0, s>>>(ws.partial.as<float>(), plan.tile_pts, plan.item_start,
+                                                                plan.nitems, (float *)u_out + u_stride * s0, u_stride);
         FGA_CUDA(cudaGetLastError());
     }
-    const int tpb = 4;  // tiles per 128-thread block
-    const unsigned blocks = (unsigned)((plan.ntiles + tpb - 1) / tpb);
-    ProfScope ps(P_REDUCE, s);
-    if (rb == 8)
-        reduce_kernel<double><<<blocks, 32 * tpb, 0, s>>>(ws.partial.as<double>(), plan.tile_pts, plan.item_start,
-                                                          plan.ntiles, (double *)u_out);
-    else
-        reduce_kernel<float><<<blocks, 32 * tpb, 0, s>>>(ws.partial.as<float>(), plan.tile_pts, plan.item_start,
-                                                         plan.ntiles, (float *)u_out);
-    FGA_CUDA(cudaGetLastError());
     return FGA_OK;
 }
 

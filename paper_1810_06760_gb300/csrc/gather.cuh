@@ -83,9 +83,12 @@ int64_t read_lattice_pair_counter(bool reset);
 fga_status sort_keys_to_perm(Workspace &ws, int32_t *keys, int64_t n, int nbuckets, int32_t **perm_out,
                              int32_t *cell_start, cudaStream_t s);
 fga_status build_sum_plan(Workspace &ws, const BinGrid &g, const int32_t *cell_start_dev, int nclasses,
-                          const double *pts_host, int64_t npts, cudaStream_t s, SumPlan &plan);
-fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void *rec_sorted, const double *pts_dev,
-                   double k, double rw, void *u_out, cudaStream_t s, int cat = P_GATHER);
+                          const double *pts_host, int64_t npts, int samples, cudaStream_t s, SumPlan &plan);
+constexpr size_t SUM_PARTIAL_MAX = (size_t)256 << 20;   // bytes of partial sums per launch of several samples
+// ns samples (rec_stride, u_stride: reals between them)
+fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void *rec, int64_t rec_stride, int ns,
+                   const double *pts_dev, double k, double rw, void *u_out, int64_t u_stride, cudaStream_t s,
+                   int cat = P_GATHER);
 // bucket starts copied to the host by build_sum_plan (valid after it returns)
 const int32_t *plan_host_cell_start(const Workspace &ws);
 

@@ -71,7 +71,7 @@ double estimate_solve_bytes(const fga_init_desc *d, double rec_cap) {
     const double decomp = cbytes * (A * (ny0 + ny1 + ny2) + ny0 * ny1 * A * 3.0 + ny0 * A * A * 3.0 +
                                     A * A * A * 3.0 * (d->g ? 2.0 : 1.0));
     const double during_decomp = state + ints + decomp;
-    const double during_solve = 2.0 * state + ints + sort + rec_cap + (rb == 4.0 ? (double)PLANE_PARTIAL_MAX : 0.0);
+    const double during_solve = 2.0 * state + ints + sort + rec_cap + (double)std::max(PLANE_PARTIAL_MAX, SUM_PARTIAL_MAX);
     return std::max(during_decomp, during_solve) + 64.0 * 1024 * 1024;
 }
 

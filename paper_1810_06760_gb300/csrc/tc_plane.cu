@@ -31,6 +31,11 @@
 //  - A group's last block of an item is marked; when every group has sent it, the accumulator (one of two, 256
 //    columns each) is handed to the epilogue warps, which copy it to the item's partial sums while the next item
 //    accumulates in the other one.
+// What bounds it: the producers' issue slots (860 warp instructions per 16 beams, 62% of the slots used; tensor
+// pipe 34%, shared memory 46%; 378 cycles per 16 beams and SM).  Sums of a solve, against one launch per sample with
+// seven single-warp producers and padded operands: 200 samples of 2.7 M beams on 16 x 16 receivers 48.7 -> 26.9 ms
+// (0.44 M beams: 13.4 -> 5.7 ms), 250 samples of 8.4 M beams on 20 x 20 receivers 192 -> 118 ms; the reductions
+// 4.9 -> 1.0, 3.3 -> 0.5 and 7.1 -> 3.2 ms.
 // Every wait is bounded: a wait that runs out sets the call's error word, which ends the other waits of the launch;
 // the producers then run through their barrier schedule without waiting or writing, the other roles leave their
 // loops, the MMA thread waits (bounded) for its outstanding MMAs, and the tensor memory is freed.
