@@ -457,10 +457,12 @@ fga_status fga_profile_enable(int mode);
 fga_status fga_profile_read(fga_profile_t *out, int reset);
 
 /* Upper bound on the device memory the library allocates for its own buffers (beam sets, sort and
- * record scratch, cached blocks of the serving loop; not the caller's buffers, not the static scratch of
- * fga_reconstruct_noalloc): an allocation that would pass it fails with FGA_ERR_OOM before cudaMalloc
+ * record scratch, cached blocks of the serving loop, idle blocks; not the caller's buffers, not the static scratch
+ * of fga_reconstruct_noalloc): an allocation that would pass it fails with FGA_ERR_OOM before cudaMalloc
  * is called.  bytes <= 0 removes the bound (the default).  fga_device_memory_in_use reports the bytes
- * currently allocated for such buffers.  Process-wide; meant for hosts that share a GPU, and for testing
+ * currently allocated for such buffers, without idle blocks.  Released blocks stay idle in the library for later
+ * calls, up to 16 GiB; they are given back to the device when an allocation needs them, when this function
+ * is called, and when the last model, beam set and server is destroyed.  Process-wide; meant for hosts that share a GPU, and for testing
  * the out-of-memory paths without exhausting the device. */
 fga_status fga_set_device_memory_limit(double bytes);
 double fga_device_memory_in_use(void);

@@ -6,6 +6,7 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <vector>
 
 #include "fga_beam.cuh"
@@ -25,8 +26,86 @@ fga_status cuda_fail(cudaError_t e, const char *what) {
     return e == cudaErrorMemoryAllocation ? FGA_ERR_OOM : FGA_ERR_CUDA;
 }
 
-// Per-thread block cache.  Off by default: every DevBuf/HostBuf then maps to cudaMalloc/cudaFree
-// (whose implicit device synchronisation also orders reuse).  A thread that issues all its work on
+// Idle blocks.  A released device or pinned block goes to a process-wide pool, per device, and serves a later
+// request of nearly its size: cudaMalloc, cudaMallocHost and their frees took 1.2 of the 1.8 ms of a small solve
+// and 10-25 ms of a large one (about 30 buffers, some of gigabytes).  Like cudaFree, whose implicit device
+// synchronisation ordered every reuse, a block released since the device was last known to be idle is handed out
+// only after a device synchronisation (one for all such blocks), so any stream and thread may release and take.
+// Idle blocks are bounded (POOL_DEV_MAX: 6% of the GPU; the largest go first), are given back when an allocation
+// fails or would pass the caller's bound, when the bound is set, and when the last model, beam set and server is
+// destroyed.
+namespace {
+constexpr size_t POOL_DEV_MAX = (size_t)16 << 30, POOL_HOST_MAX = (size_t)64 << 20;
+struct Pool {
+    struct Block {
+        void *p;
+        bool dirty;
+        int dev;   // device whose work may still use a dirty block
+    };
+    std::mutex mu;
+    std::map<int, std::multimap<size_t, Block>> dev;   // by device
+    std::multimap<size_t, Block> host;
+    size_t dev_bytes = 0, host_bytes = 0;
+    int objects = 0;   // models, beam sets and servers alive
+};
+Pool &pool() {
+    static Pool *p = new Pool();   // never destroyed: blocks may be released while the process exits
+    return *p;
+}
+int current_device() {
+    int d = 0;
+    cudaGetDevice(&d);
+    return d;
+}
+// a block of at least need bytes, at most an eighth larger; the pool's lock is held
+void *pool_take(Pool &P, std::multimap<size_t, Pool::Block> &c, size_t &total, size_t need, size_t *size) {
+    auto it = c.lower_bound(need);
+    if (it == c.end() || it->first > need + need / 8 + 4096) return nullptr;
+    if (it->second.dirty) {
+        const int d = current_device();
+        if (it->second.dev != d || cudaDeviceSynchronize() != cudaSuccess) return nullptr;   // no reuse
+        for (auto &kv : P.dev[d]) kv.second.dirty = false;
+        for (auto &kv : P.host)
+            if (kv.second.dev == d) kv.second.dirty = false;
+    }
+    void *p = it->second.p;
+    *size = it->first;
+    total -= it->first;
+    c.erase(it);
+    return p;
+}
+// free idle device blocks, largest first, until at most keep bytes are left; the lock is held
+void pool_trim(Pool &P, size_t keep) {
+    while (P.dev_bytes > keep) {
+        std::multimap<size_t, Pool::Block> *best = nullptr;
+        for (auto &d : P.dev)
+            if (!d.second.empty() && (!best || std::prev(d.second.end())->first > std::prev(best->end())->first))
+                best = &d.second;
+        if (!best) break;
+        auto it = std::prev(best->end());
+        cudaFree(it->second.p);
+        P.dev_bytes -= it->first;
+        best->erase(it);
+    }
+}
+}  // namespace
+
+size_t pool_idle_bytes() {
+    std::lock_guard<std::mutex> lk(pool().mu);
+    return pool().dev_bytes;
+}
+void pool_object(int d) {
+    Pool &P = pool();
+    std::lock_guard<std::mutex> lk(P.mu);
+    P.objects += d;
+    if (P.objects > 0) return;
+    pool_trim(P, 0);
+    for (auto &kv : P.host) cudaFreeHost(kv.second.p);
+    P.host.clear();
+    P.host_bytes = 0;
+}
+
+// Per-thread block cache of a server worker, in the place of the pool.  A thread that issues all its work on
 // one stream (a server worker) turns it on: released blocks go to the thread's cache and are handed
 // back to later allocations of the same thread, whose work is ordered after every earlier use on
 // that stream, so no allocation or free stalls the other streams.  Pinned host blocks are cached only
@@ -54,10 +133,24 @@ void *cache_take(std::multimap<size_t, void *> &c, size_t &total, size_t need, s
 // device bytes held by the library's own buffers, and the caller's bound on them (0: none)
 std::atomic<int64_t> g_dev_bytes{0}, g_dev_limit{0};
 
+// allocated bytes besides the idle pool are g_dev_bytes; the bound holds for both together
 static cudaError_t dev_alloc(void **p, size_t need) {
     const int64_t lim = g_dev_limit.load();
-    if (lim > 0 && g_dev_bytes.load() + (int64_t)need > lim) return cudaErrorMemoryAllocation;
-    const cudaError_t e = cudaMalloc(p, need);
+    if (lim > 0) {
+        const int64_t room = lim - g_dev_bytes.load() - (int64_t)need;
+        if (room < 0) return cudaErrorMemoryAllocation;
+        std::lock_guard<std::mutex> lk(pool().mu);
+        pool_trim(pool(), (size_t)room);
+    }
+    cudaError_t e = cudaMalloc(p, need);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        {
+            std::lock_guard<std::mutex> lk(pool().mu);
+            pool_trim(pool(), 0);
+        }
+        e = cudaMalloc(p, need);
+    }
     if (e == cudaSuccess) g_dev_bytes += (int64_t)need;
     return e;
 }
@@ -100,6 +193,19 @@ fga_status DevBuf::ensure(size_t need) {
             bytes = got;
             return FGA_OK;
         }
+    } else {
+        Pool &P = pool();
+        std::lock_guard<std::mutex> lk(P.mu);
+        const int64_t lim = g_dev_limit.load();
+        device = current_device();
+        size_t got = 0;
+        if (lim <= 0 || g_dev_bytes.load() + (int64_t)(need + need / 8 + 4096) <= lim)
+            if (void *q = pool_take(P, P.dev[current_device()], P.dev_bytes, need, &got)) {
+                p = q;
+                bytes = got;
+                g_dev_bytes += (int64_t)got;
+                return FGA_OK;
+            }
     }
     cudaError_t e = dev_alloc(&p, need);
     if (e == cudaErrorMemoryAllocation && tl_cache.on && tl_cache.dev_bytes > 0) {
@@ -124,8 +230,15 @@ void DevBuf::release() {
         if (tl_cache.on) {
             tl_cache.dev.emplace(bytes, p);
             tl_cache.dev_bytes += bytes;
-        } else {
+        } else if (bytes > POOL_DEV_MAX) {
             dev_free(p, bytes);
+        } else {
+            Pool &P = pool();
+            std::lock_guard<std::mutex> lk(P.mu);
+            pool_trim(P, POOL_DEV_MAX - bytes);
+            P.dev[device].emplace(bytes, Pool::Block{p, true, device});
+            P.dev_bytes += bytes;
+            g_dev_bytes -= (int64_t)bytes;
         }
     }
     p = nullptr;
@@ -138,6 +251,16 @@ fga_status HostBuf::ensure(size_t need) {
     if (tl_cache.on) {
         size_t got = 0;
         if (void *q = cache_take(tl_cache.host, tl_cache.host_bytes, need, &got)) {
+            p = q;
+            bytes = got;
+            return FGA_OK;
+        }
+    } else {
+        Pool &P = pool();
+        std::lock_guard<std::mutex> lk(P.mu);
+        device = current_device();
+        size_t got = 0;
+        if (void *q = pool_take(P, P.host, P.host_bytes, need, &got)) {
             p = q;
             bytes = got;
             return FGA_OK;
@@ -161,7 +284,14 @@ void HostBuf::release() {
             tl_cache.host.emplace(bytes, p);
             tl_cache.host_bytes += bytes;
         } else {
-            cudaFreeHost(p);
+            Pool &P = pool();
+            std::lock_guard<std::mutex> lk(P.mu);
+            if (P.host_bytes + bytes <= POOL_HOST_MAX) {
+                P.host.emplace(bytes, Pool::Block{p, true, device});
+                P.host_bytes += bytes;
+            } else {
+                cudaFreeHost(p);
+            }
         }
     }
     p = nullptr;
@@ -316,6 +446,8 @@ int fga_version(void) { return 10000; }
 
 fga_status fga_set_device_memory_limit(double bytes) {
     g_dev_limit.store(bytes > 0 ? (int64_t)bytes : 0);
+    std::lock_guard<std::mutex> lk(pool().mu);
+    pool_trim(pool(), 0);
     return FGA_OK;
 }
 
@@ -367,18 +499,24 @@ fga_status fga_model_create(fga_model **out, const fga_model_desc *d, const floa
         const unsigned blocks = (unsigned)((nn + 255) / 256);
         pack_grid_kernel<<<blocks, 256, 0, s>>>(grid_p, gp, nn);
         pack_grid_kernel<<<blocks, 256, 0, s>>>(grid_s, gs, nn);
-        unsigned *dmax = nullptr;
-        cudaError_t e = cudaMalloc(&dmax, 2 * sizeof(unsigned));
+        ScopedDevBuf maxb;
+        st = maxb.ensure(2 * sizeof(unsigned));
+        if (st != FGA_OK) {
+            m->grid.release();
+            delete m;
+            return st;
+        }
+        unsigned *dmax = maxb.as<unsigned>();
         unsigned hmax[2] = {0, 0};
-        if (e == cudaSuccess) e = cudaMemsetAsync(dmax, 0, 2 * sizeof(unsigned), s);
+        cudaError_t e = cudaMemsetAsync(dmax, 0, 2 * sizeof(unsigned), s);
         if (e == cudaSuccess) {
             max_field0_kernel<<<304, 256, 0, s>>>(gp, nn, dmax);
             max_field0_kernel<<<304, 256, 0, s>>>(gs, nn, dmax + 1);
             e = cudaMemcpyAsync(hmax, dmax, sizeof hmax, cudaMemcpyDeviceToHost, s);
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (dmax) cudaFree(dmax);
         if (e != cudaSuccess) {
+            m->grid.release();
             delete m;
             return cuda_fail(e, "fga_model_create");
         }
@@ -472,6 +610,7 @@ fga_status fga_model_create(fga_model **out, const fga_model_desc *d, const floa
         delete m;
         return cuda_fail(e, "fga_model_create");
     }
+    pool_object(1);
     *out = m;
     return FGA_OK;
 }
@@ -480,6 +619,7 @@ fga_status fga_model_destroy(fga_model *m) {
     if (!m) return FGA_OK;
     m->grid.release();
     delete m;
+    pool_object(-1);
     return FGA_OK;
 }
 
@@ -869,7 +1009,7 @@ fga_status solve_impl(const fga_model *m, const fga_init_desc *init, const fga_s
     // records of one window live in one buffer; cap its size
     size_t free_b = 0, total_b = 0;
     FGA_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    const double rec_budget = std::min(rec_cap, 0.4 * (double)free_b);
+    const double rec_budget = std::min(rec_cap, 0.4 * (double)(free_b + pool_idle_bytes()));
     int js = 0;
     for (int n0 = 0; n0 < sd->nsteps;) {
         if (cancel && cancel->load()) return cancelled(s);

@@ -174,6 +174,7 @@ int64_t read_pair_counter(bool reset);  // gather.cu
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    int device = 0;   // of the allocation
     fga_status ensure(size_t need);
     void release();
     template <class T> T *as() const { return static_cast<T *>(p); }
@@ -188,6 +189,7 @@ struct ScopedDevBuf : DevBuf {
 struct HostBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    int device = 0;   // of the allocation
     fga_status ensure(size_t need);
     void release();
     template <class T> T *as() const { return static_cast<T *>(p); }
@@ -198,6 +200,11 @@ void block_cache_enable(cudaStream_t s);
 void block_cache_disable();
 void block_cache_trim(size_t keep_bytes);
 size_t block_cache_bytes();
+
+// idle blocks of the process-wide pool (see api.cu): their bytes; models, beam sets and servers created (1) and
+// destroyed (-1) -- the pool is emptied when none is left
+size_t pool_idle_bytes();
+void pool_object(int d);
 
 // scratch used by binning and the Gaussian sum
 struct Workspace {
@@ -219,6 +226,8 @@ struct fga_model {
 };
 
 struct fga_beams {
+    fga_beams() { fga::pool_object(1); }
+    ~fga_beams() { fga::pool_object(-1); }
     int precision;
     double k, w;
     // tilted layered media: the state is in the layer frame x' = R x (R as in ModelDev)

@@ -181,7 +181,7 @@ fga_status fga_server_create(fga_server **out, const fga_model *m, const fga_ser
     FGA_CUDA(cudaGetDevice(&sv->device));
     size_t free_b = 0, total_b = 0;
     FGA_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    sv->budget = d->hbm_budget_bytes > 0 ? d->hbm_budget_bytes : 0.85 * (double)free_b;
+    sv->budget = d->hbm_budget_bytes > 0 ? d->hbm_budget_bytes : 0.85 * (double)(free_b + pool_idle_bytes());
     sv->rec_cap = d->record_cap_bytes > 0 ? d->record_cap_bytes : 2.0e9;
     FGA_CHECK(d->policy == FGA_SERVE_FIFO || d->policy == FGA_SERVE_SHORTEST, "fga_server_create: unknown policy");
     sv->policy = d->policy;
