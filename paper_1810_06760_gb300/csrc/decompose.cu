@@ -5,6 +5,7 @@
 #include <cstring>
 
 #include "fga_beam.cuh"
+#include "tc_gemm.cuh"
 
 namespace fga {
 
@@ -111,64 +112,39 @@ struct TransformScratch {
     double S[3] = {1, 1, 1}; // max over kernel rows of sum_i |K_d[a][i]| per axis (bounds of the stages)
 };
 
-template <typename R>
-static fga_status stage_gemm(const double2 *A, int64_t sAz, int64_t sAm, int64_t sAk, const C2<R> *B, int64_t sBn,
-                             int64_t sBk, C2<R> *Cm, int64_t sCz, int64_t sCm, int64_t sCn, int Z, int64_t M, int N,
-                             int K, R scale, const TransformScratch &ts, double factor, cudaStream_t s);
-template <typename R>
-static fga_status stage_gemm(const C2<R> *A, int64_t sAz, int64_t sAm, int64_t sAk, const C2<R> *B, int64_t sBn,
-                             int64_t sBk, C2<R> *Cm, int64_t sCz, int64_t sCm, int64_t sCn, int Z, int64_t M, int N,
-                             int K, R scale, const TransformScratch &ts, double factor, cudaStream_t s);
-
-template <>
-fga_status stage_gemm<double>(const double2 *A, int64_t sAz, int64_t sAm, int64_t sAk, const C2<double> *B,
-                              int64_t sBn, int64_t sBk, C2<double> *Cm, int64_t sCz, int64_t sCm, int64_t sCn, int Z,
-                              int64_t M, int N, int K, double scale, const TransformScratch &, double, cudaStream_t s) {
-    return cgemm<double, double2>(A, sAz, sAm, sAk, B, sBn, sBk, Cm, sCz, sCm, sCn, Z, M, N, K, scale, s);
-}
-template <>
-fga_status stage_gemm<double>(const C2<double> *A, int64_t sAz, int64_t sAm, int64_t sAk, const C2<double> *B,
-                              int64_t sBn, int64_t sBk, C2<double> *Cm, int64_t sCz, int64_t sCm, int64_t sCn, int Z,
-                              int64_t M, int N, int K, double scale, const TransformScratch &, double, cudaStream_t s) {
-    return cgemm<double, C2<double>>(A, sAz, sAm, sAk, B, sBn, sBk, Cm, sCz, sCm, sCn, Z, M, N, K, scale, s);
-}
-template <>
-fga_status stage_gemm<float>(const double2 *A, int64_t sAz, int64_t sAm, int64_t sAk, const C2<float> *B, int64_t sBn,
-                             int64_t sBk, C2<float> *Cm, int64_t sCz, int64_t sCm, int64_t sCn, int Z, int64_t M, int N,
-                             int K, float scale, const TransformScratch &ts, double factor, cudaStream_t s) {
-    return tc_cgemm<double2>(A, sAz, sAm, sAk, reinterpret_cast<const float2 *>(B), sBn, sBk,
-                             reinterpret_cast<float2 *>(Cm), sCz, sCm, sCn, Z, M, N, K, scale, ts.amax, (float)factor,
-                             ts.err, s);
-}
-template <>
-fga_status stage_gemm<float>(const C2<float> *A, int64_t sAz, int64_t sAm, int64_t sAk, const C2<float> *B,
-                             int64_t sBn, int64_t sBk, C2<float> *Cm, int64_t sCz, int64_t sCm, int64_t sCn, int Z,
-                             int64_t M, int N, int K, float scale, const TransformScratch &ts, double factor,
-                             cudaStream_t s) {
-    return tc_cgemm<float2>(reinterpret_cast<const float2 *>(A), sAz, sAm, sAk, reinterpret_cast<const float2 *>(B),
-                            sBn, sBk, reinterpret_cast<float2 *>(Cm), sCz, sCm, sCn, Z, M, N, K, scale, ts.amax,
-                            (float)factor, ts.err, s);
-}
-
-template <typename R>
-static fga_status fbi_transform(const fga_init_desc *d, const double2 *f, C2<R> *const Kax[3], C2<R> *T1, C2<R> *T2,
-                                C2<R> *F, const TransformScratch &ts, cudaStream_t s) {
+static fga_status fbi_transform_f64(const fga_init_desc *d, const double2 *f, C2<double> *const Kax[3], C2<double> *T1,
+                                    C2<double> *T2, C2<double> *F, cudaStream_t s) {
+    using D2 = C2<double>;
     const int A = d->nq * d->np;
     const int n0 = d->ny[0], n1 = d->ny[1], n2 = d->ny[2];
-    if (sizeof(R) == 4) FGA_TRY(tc_absmax(f, (int64_t)n0 * n1 * n2 * 3, ts.amax, s));
+    // stage 1 (contract y2), one GEMM per component c: T1[(y0,y1)][a2][c]
+    FGA_TRY((cgemm<double, double2>(f, 1, (int64_t)n2 * 3, 3, Kax[2], n2, 1, T1, 1, (int64_t)A * 3, 3, 3, (int64_t)n0 * n1,
+                                    A, n2, 1.0, s)));
+    // stage 2 (contract y1): T2[y0][a1][(a2,c)] ; batch y0, m = (a2,c), n = a1, k = y1
+    FGA_TRY((cgemm<double, D2>(T1, (int64_t)n1 * A * 3, 1, (int64_t)A * 3, Kax[1], n1, 1, T2, (int64_t)A * A * 3, 1,
+                               (int64_t)A * 3, n0, (int64_t)A * 3, A, n1, 1.0, s)));
+    // stage 3 (contract y0): F[a0][(a1,a2,c)], m = (a1,a2,c), n = a0, k = y0
+    const double vol = d->dy[0] * d->dy[1] * d->dy[2];
+    return cgemm<double, D2>(T2, 0, 1, (int64_t)A * A * 3, Kax[0], n0, 1, F, 0, 1, (int64_t)A * A * 3, 1,
+                             (int64_t)A * A * 3, A, n0, vol, s);
+}
+
+// the same on the tensor cores; stage 1 takes the components as rows (m = 3 (y0,y1) + c), so that the data are read
+// in one pass
+static fga_status fbi_transform_f32(const fga_init_desc *d, const double2 *f, const KernelMatrices &K, float2 *T1,
+                                    float2 *T2, float2 *F, const TransformScratch &ts, cudaStream_t s) {
+    const int A = d->nq * d->np;
+    const int n0 = d->ny[0], n1 = d->ny[1], n2 = d->ny[2];
+    const int64_t A3 = (int64_t)A * 3;
+    FGA_TRY(tc_absmax(f, (int64_t)n0 * n1 * n2 * 3, ts.amax, s));
     // |Re|, |Im| of a stage's output <= sqrt(2) max(|Re|, |Im|) of its input x sum_i |K[a][i]|
     const double g1 = std::sqrt(2.0) * ts.S[2], g2 = g1 * std::sqrt(2.0) * ts.S[1];
-    // stage 1 (contract y2), one GEMM per component c: T1[(y0,y1)][a2][c]
-    FGA_TRY((stage_gemm<R>(f, 1, (int64_t)n2 * 3, 3, Kax[2], n2, 1, T1, 1, (int64_t)A * 3, 3, 3, (int64_t)n0 * n1, A,
-                           n2, R(1), ts, 1.0, s)));
-    // stage 2 (contract y1): T2[y0][a1][(a2,c)] ; batch y0, m = (a2,c), n = a1, k = y1
-    FGA_TRY((stage_gemm<R>((const C2<R> *)T1, (int64_t)n1 * A * 3, 1, (int64_t)A * 3, Kax[1], n1, 1, T2,
-                           (int64_t)A * A * 3, 1, (int64_t)A * 3, n0, (int64_t)A * 3, A, n1, R(1), ts, g1, s)));
-    // stage 3 (contract y0): F[a0][(a1,a2,c)], m = (a1,a2,c), n = a0, k = y0
-    const R vol = (R)(d->dy[0] * d->dy[1] * d->dy[2]);
-    FGA_TRY((stage_gemm<R>((const C2<R> *)T2, 0, 1, (int64_t)A * A * 3, Kax[0], n0, 1, F, 0, 1, (int64_t)A * A * 3, 1,
-                           (int64_t)A * A * 3, A, n0, vol, ts, g2, s)));
-    return FGA_OK;
+    FGA_TRY((tc_cgemm<double2>(f, 0, (int64_t)n2 * 3, 3, K.ax[2], T1, 0, A3, 3, 3, 1, (int64_t)n0 * n1 * 3, A, 1.f, ts.amax,
+                               1.f, ts.err, s)));
+    FGA_TRY((tc_cgemm<float2>(T1, n1 * A3, 1, A3, K.ax[1], T2, A * A3, 1, A3, 1, n0, A3, A, 1.f, ts.amax, (float)g1, ts.err,
+                              s)));
+    const float vol = (float)(d->dy[0] * d->dy[1] * d->dy[2]);
+    return tc_cgemm<float2>(T2, 0, 1, A * A3, K.ax[0], F, 0, 1, A * A3, 1, 1, A * A3, A, vol, ts.amax, (float)g2, ts.err, s);
 }
 
 // max over the q nodes of sum_i exp(-k (y_i - q)^2 / 2): the largest row sum of |K| on one axis
@@ -381,19 +357,6 @@ static fga_status transform_typed(const fga_init_desc *d, const double2 *f, cons
                                   cudaStream_t s) {
     const int A = d->nq * d->np;
     ScopedDevBuf Kb, T1, T2, tsb;
-    const size_t kbytes = sizeof(C2<R>) * (size_t)A * (d->ny[0] + d->ny[1] + d->ny[2]);
-    FGA_TRY(Kb.ensure(kbytes));
-    C2<R> *Kax[3];
-    Kax[0] = Kb.as<C2<R>>();
-    Kax[1] = Kax[0] + (size_t)A * d->ny[0];
-    Kax[2] = Kax[1] + (size_t)A * d->ny[1];
-    for (int ax = 0; ax < 3; ax++) {
-        const int tot = A * d->ny[ax];
-        ProfScope ps(P_DECOMP, s);
-        fbi_axis_kernel<R><<<(tot + 255) / 256, 256, 0, s>>>(Kax[ax], d->nq, d->np, d->ny[ax], d->q0[ax], d->dq[ax],
-                                                            d->p0[ax], d->dp[ax], d->y0[ax], d->dy[ax], d->k);
-    }
-    FGA_CUDA(cudaGetLastError());
     FGA_TRY(T1.ensure(sizeof(C2<R>) * (size_t)d->ny[0] * d->ny[1] * A * 3));
     FGA_TRY(T2.ensure(sizeof(C2<R>) * (size_t)d->ny[0] * A * A * 3));
     FGA_TRY(tsb.ensure(64));
@@ -401,15 +364,55 @@ static fga_status transform_typed(const fga_init_desc *d, const double2 *f, cons
     ts.amax = tsb.as<float>();
     ts.err = reinterpret_cast<int *>(tsb.as<char>() + 16);
     FGA_CUDA(cudaMemsetAsync(tsb.p, 0, 64, s));
-    for (int a = 0; a < 3; a++)
-        ts.S[a] = kernel_row_sum_max(d->nq, d->q0[a], d->dq[a], d->ny[a], d->y0[a], d->dy[a], d->k);
-    FGA_TRY(fbi_transform<R>(d, f, Kax, T1.as<C2<R>>(), T2.as<C2<R>>(), F, ts, s));
-    if (g && G) FGA_TRY(fbi_transform<R>(d, g, Kax, T1.as<C2<R>>(), T2.as<C2<R>>(), G, ts, s));
+    if constexpr (sizeof(R) == 4) {
+        KernelMatrices K;
+        K.nq = d->nq;
+        K.np = d->np;
+        K.k = d->k;
+        size_t total = 0;
+        for (int a = 0; a < 3; a++) {
+            KernelMatrix &X = K.ax[a];
+            tc_kernel_shape(A, d->ny[a], X);
+            X.q0 = d->q0[a];
+            X.dq = d->dq[a];
+            X.p0 = d->p0[a];
+            X.dp = d->dp[a];
+            X.y0 = d->y0[a];
+            X.dy = d->dy[a];
+            total += X.bytes;
+            ts.S[a] = kernel_row_sum_max(d->nq, d->q0[a], d->dq[a], d->ny[a], d->y0[a], d->dy[a], d->k);
+        }
+        FGA_TRY(Kb.ensure(total));
+        unsigned char *at = Kb.as<unsigned char>();
+        for (int a = 0; a < 3; a++) {
+            K.ax[a].B = at;
+            at += K.ax[a].bytes;
+        }
+        FGA_TRY(tc_kernel_matrices(K, s));
+        float2 *t1 = T1.as<float2>(), *t2 = T2.as<float2>();
+        FGA_TRY(fbi_transform_f32(d, f, K, t1, t2, reinterpret_cast<float2 *>(F), ts, s));
+        if (g && G) FGA_TRY(fbi_transform_f32(d, g, K, t1, t2, reinterpret_cast<float2 *>(G), ts, s));
+    } else {
+        FGA_TRY(Kb.ensure(sizeof(C2<R>) * (size_t)A * (d->ny[0] + d->ny[1] + d->ny[2])));
+        C2<R> *Kax[3];
+        Kax[0] = Kb.as<C2<R>>();
+        Kax[1] = Kax[0] + (size_t)A * d->ny[0];
+        Kax[2] = Kax[1] + (size_t)A * d->ny[1];
+        for (int ax = 0; ax < 3; ax++) {
+            const int tot = A * d->ny[ax];
+            ProfScope ps(P_DECOMP, s);
+            fbi_axis_kernel<R><<<(tot + 255) / 256, 256, 0, s>>>(Kax[ax], d->nq, d->np, d->ny[ax], d->q0[ax], d->dq[ax],
+                                                                d->p0[ax], d->dp[ax], d->y0[ax], d->dy[ax], d->k);
+        }
+        FGA_CUDA(cudaGetLastError());
+        FGA_TRY(fbi_transform_f64(d, f, Kax, T1.as<C2<R>>(), T2.as<C2<R>>(), F, s));
+        if (g && G) FGA_TRY(fbi_transform_f64(d, g, Kax, T1.as<C2<R>>(), T2.as<C2<R>>(), G, s));
+    }
     // the temporaries are released when this scope ends; make sure the stream is done with them
+    int terr = 0;
+    if (sizeof(R) == 4) FGA_CUDA(cudaMemcpyAsync(&terr, ts.err, sizeof terr, cudaMemcpyDeviceToHost, s));
     FGA_CUDA(cudaStreamSynchronize(s));
     if (sizeof(R) == 4) {
-        int terr = 0;
-        FGA_CUDA(cudaMemcpy(&terr, ts.err, sizeof terr, cudaMemcpyDeviceToHost));
         if (terr) {
             set_error("wave-packet transform: a tensor-core wait ran out");
             return FGA_ERR_TIMEOUT;
