@@ -22,6 +22,15 @@
 // Re/Im of the 3 T0 complex (i,c) pairs.  Operand blocks are single-buffered: the records and factors
 // of the next block are formed while the tensor cores work on the current one.  The partial sums go
 // to the plan's per-item buffer in the layout of the CUDA-core lattice kernel and are reduced by it.
+//
+// The factors sit point by point with the block's 32 beams side by side (Re, then Im; rows padded to 272 bytes): a
+// warp forms one chunk of points for its 32 lanes' beams without divergence or bank conflicts, and an operand task
+// reads 16-byte runs, multiplies two beams per packed FP32x2 operation and splits them in pairs; rows that share E2
+// and columns that share E0 are formed by one thread.  The operands' power-of-two scales are folded into the
+// factors, and the copies of B' that repeat or negate another are stored, not formed again.  Bound by shared
+// memory: 960 wavefronts of operand reads by the tensor cores and 1,790 of stores and loads per block of 32 beams,
+// 86% of its 3,210 cycles (tensor pipe 36%).  61 x 64 x 57 points (64 tiles), 1.05 M beams: 16.1 -> 12.8 ms; 64^3
+// snapshot of 8.4 M beams 136 -> 99 ms.
 #include <algorithm>
 #include <cstdio>
 #include <cmath>
@@ -62,18 +71,20 @@ constexpr int LT_CAND = 4096;           // candidates filtered per round (per-CT
 
 // shared-memory layout; the B operand copies and the tensor-memory columns are sized to the tile's
 // real width NR, so narrow tiles (single receiver planes) fit three CTAs per SM
+constexpr int LT_ES = 68;               // floats per point of the factor buffer: Re[32], Im[32], 4 of padding
+constexpr int LT_RS = 36;               // floats per record field: 32 beams, 4 of padding
+
 struct LtSmem {
-    int a, b, e, rec, w, x, cnt, bar, bytes, bbytes;
+    int a, b, e, rec, x, cnt, bar, bytes, bbytes;
     uint32_t tcols;
-    __host__ __device__ void init(int TA, bool with_w, int NR) {
+    __host__ __device__ void init(int TA, int NR) {
         bbytes = NR * LT_KB * 2;
         tcols = NR <= 32 ? 32u : (NR <= 64 ? 64u : (NR <= 128 ? 128u : 256u));
         a = 0;
         b = a + 4 * LT_A_BYTES;
-        e = b + 4 * bbytes;                     // 2 x [32][TA] float2
-        rec = e + 2 * LT_KB * TA * 8;           // 2 x [32][REC] float
-        w = rec + 2 * LT_KB * REC * 4;          // 2 x [32][3] float2: A_c E2 of single-plane tiles
-        x = w + (with_w ? 2 * LT_KB * 3 * 8 : 0);
+        e = b + 4 * bbytes;                     // [TA][LT_ES] float
+        rec = e + TA * LT_ES * 4;               // 2 x [REC][LT_RS] float
+        x = rec + 2 * LT_RS * REC * 4;
         cnt = (x + TA * 4 + 15) / 16 * 16;
         bar = cnt + (LT_THREADS / 32 + 1) * 4;
         bar = (bar + 15) / 16 * 16;
@@ -102,9 +113,8 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sA = smem + S.a;
     unsigned char *sB = smem + S.b;
-    float2 *sE0 = reinterpret_cast<float2 *>(smem + S.e);   // 2 x [32][TA]: E0 (T0), E1 (T1), E2 (T2)
-    float *sR0 = reinterpret_cast<float *>(smem + S.rec);   // 2 x [32][REC]
-    float2 *sW0 = reinterpret_cast<float2 *>(smem + S.w);   // 2 x [32][3]
+    float *sE = reinterpret_cast<float *>(smem + S.e);      // [TA][LT_ES]: E0 (T0), E1 (T1), E2 (T2)
+    float *sR0 = reinterpret_cast<float *>(smem + S.rec);   // 2 x [REC][LT_RS]
     float *sX = reinterpret_cast<float *>(smem + S.x);      // tile coordinates, axis 0 | 1 | 2
     int *sCnt = reinterpret_cast<int *>(smem + S.cnt);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + S.bar);
@@ -153,7 +163,8 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
     const float hk = -0.5f * k;
     // exact small-integer division by float reciprocals (quotients below 2^12, divisors below 2^8)
     const int nch = X.nch[0] + X.nch[1] + X.nch[2];
-    const float inv_nch = 1.0f / (float)nch, inv_R = 1.0f / (float)R_used, inv_nc = 1.0f / (float)nc_used;
+    const int ntask_a = 4 * (crow ? R_used : T2 * ((T1 + 1) >> 1)), ntask_a32 = (ntask_a + 31) / 32 * 32, ntask_b = 4 * T0;
+    const float inv_a = 4.0f / (float)ntask_a, inv_T0 = 1.0f / (float)T0;
     const float inv_T2 = 1.0f / (float)T2, inv_3 = 1.0f / 3.0f;
 
     const float blo0 = sX[0], bhi0 = sX[e0 - 1], blo1 = sX[T0], bhi1 = sX[T0 + e1 - 1];
@@ -170,10 +181,10 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
             const int64_t c = c0 + tid;
             bool kp = false;
             if (c < cend) {
-                const float *q = rec + c * REC;
-                const float g0 = fmaxf(fmaxf(blo0 - q[0], q[0] - bhi0), 0.f);
-                const float g1 = fmaxf(fmaxf(blo1 - q[1], q[1] - bhi1), 0.f);
-                const float g2 = fmaxf(fmaxf(blo2 - q[2], q[2] - bhi2), 0.f);
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(rec + c * REC));
+                const float g0 = fmaxf(fmaxf(blo0 - q.x, q.x - bhi0), 0.f);
+                const float g1 = fmaxf(fmaxf(blo1 - q.y, q.y - bhi1), 0.f);
+                const float g2 = fmaxf(fmaxf(blo2 - q.z, q.z - bhi2), 0.f);
                 kp = g0 * g0 + g1 * g1 + g2 * g2 <= rw2;
             }
             const unsigned bl = __ballot_sync(0xffffffffu, kp);
@@ -194,47 +205,49 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
 
         auto load_records = [&](int blk, float *dst) {
             const int kb0 = blk * LT_KB, nb = min(LT_KB, nk - kb0);
-            for (int q = tid; q < LT_KB * REC; q += LT_THREADS) {
-                const int b = q / REC;
-                dst[q] = b < nb ? rec[(it.y + keptc[kb0 + b]) * REC + (q - b * REC)] : 0.0f;
+            if (warp < 3) {   // 16 bytes of one record per thread
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (lane < nb)
+                    v = __ldg(reinterpret_cast<const float4 *>(rec + (it.y + keptc[kb0 + lane]) * REC) + warp);
+                float *d = dst + 4 * warp * LT_RS + lane;
+                d[0] = v.x;
+                d[LT_RS] = v.y;
+                d[2 * LT_RS] = v.z;
+                d[3 * LT_RS] = v.w;
             }
         };
-        auto factors = [&](int blk, const float *sR, float2 *sE, float2 *sW) {
+        // a warp per chunk of points, a lane per beam
+        auto factors = [&](int blk, const float *sR) {
             const int nb = min(LT_KB, nk - blk * LT_KB);
-            for (int q = tid; q < LT_KB * nch; q += LT_THREADS) {
-                const int b = (int)(((float)q + 0.5f) * inv_nch), c = q - b * nch;
+            for (int c = warp; c < nch; c += NW) {
                 const int d = c < X.nch[0] ? 0 : (c < X.nch[0] + X.nch[1] ? 1 : 2);
                 const int cc = c - (d == 0 ? 0 : (d == 1 ? X.nch[0] : X.nch[0] + X.nch[1]));
                 const int off = d == 0 ? 0 : (d == 1 ? T0 : T0 + T1), Td = d == 0 ? T0 : (d == 1 ? T1 : T2);
                 const int a0 = cc * X.len[d], a1 = min(a0 + X.len[d], Td);
-                float2 *dst = sE + b * TA + off;
-                const bool wfold = crow && d == 2 && T2 == 1;   // also A_c E2 for the component rows
-                if (b >= nb) {
-                    for (int a = a0; a < a1; a++) dst[a] = make_float2(0.f, 0.f);
-                    if (wfold)
-                        for (int c = 0; c < 3; c++) sW[b * 3 + c] = make_float2(0.f, 0.f);
-                    continue;
-                }
-                const float Qd = sR[b * REC + d], Pd = sR[b * REC + 3 + d];
+                float *dst = sE + (off + a0) * LT_ES + lane;
+                const float Qd = sR[d * LT_RS + lane], Pd = sR[(3 + d) * LT_RS + lane];
                 const float x = sX[off + a0] - Qd;
+                // E0 and E1 carry the operand scales (powers of two); padding beams are zero
+                const float scl = lane < nb ? (d == 0 ? sB_scale : (d == 1 ? sA_scale : 1.0f)) : 0.0f;
                 float er, ei;
                 gauss_phase_exp<float>(k * Pd * x, hk * x * x, &er, &ei);
-                dst[a0] = make_float2(er, ei);
-                if (wfold)
-                    for (int c = 0; c < 3; c++) {
-                        const float ar = sR[b * REC + 6 + 2 * c], ai = sR[b * REC + 7 + 2 * c];
-                        sW[b * 3 + c] = make_float2(ar * er - ai * ei, ar * ei + ai * er);
-                    }
+                er *= scl;
+                ei *= scl;
+                dst[0] = er;
+                dst[LT_KB] = ei;
                 if (a1 - a0 > 1) {
                     const float h = X.dx[d];
                     float rr, ri;
                     gauss_phase_exp<float>(k * Pd * h, -k * h * (x + 0.5f * h), &rr, &ri);
+                    if (lane >= nb) rr = ri = 0.0f;
                     const float g = __expf(-k * h * h);
                     for (int a = a0 + 1; a < a1; a++) {
                         const float nr = er * rr - ei * ri, ni = er * ri + ei * rr;
                         er = nr;
                         ei = ni;
-                        dst[a] = make_float2(er, ei);
+                        dst += LT_ES;
+                        dst[0] = er;
+                        dst[LT_KB] = ei;
                         rr *= g;
                         ri *= g;
                     }
@@ -247,8 +260,8 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
                     const int b = q / np, rem = q - b * np;
                     const int i = rem / (T1 * T2), r = rem - i * (T1 * T2), j = r / T2, l = r - j * T2;
                     if (i < e0 && j < e1 && l < e2) {
-                        const float *rb = sR + b * REC;
-                        const float d0 = sX[i] - rb[0], d1 = sX[T0 + j] - rb[1], d2 = sX[T0 + T1 + l] - rb[2];
+                        const float *rb = sR + b;
+                        const float d0 = sX[i] - rb[0], d1 = sX[T0 + j] - rb[LT_RS], d2 = sX[T0 + T1 + l] - rb[2 * LT_RS];
                         if (d0 * d0 + d1 * d1 + d2 * d2 <= rw2) mine++;
                     }
                 }
@@ -258,91 +271,110 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
         };
 
         // ---- software pipeline over the round's blocks of 32 kept beams ----
-        // block n: operands from (sR, sE)[n % 2]; while the tensor cores run block n, the factors of
-        // n+1 are formed and the records of n+2 loaded
+        // block n: operands from sR[n % 2] and sE; while the tensor cores run block n, the factors of n+1 are formed
+        // and the records of n+2 loaded
         if (nblk > 0) load_records(0, sR0);
         __syncthreads();
-        if (nblk > 0) factors(0, sR0, sE0, sW0);
-        if (nblk > 1) load_records(1, sR0 + LT_KB * REC);
+        if (nblk > 0) factors(0, sR0);
+        if (nblk > 1) load_records(1, sR0 + LT_RS * REC);
         for (int n = 0; n < nblk; n++) {
-            const float *sR = sR0 + (n & 1) * LT_KB * REC;
-            const float2 *sE = sE0 + (n & 1) * LT_KB * TA;
+            const float *sR = sR0 + (n & 1) * LT_RS * REC;
             bool arrived = true;
             if (issued > 0 && tid == 0) arrived = tc::mbar_wait(tc::smem_u32(bar), parity);
             ok = __syncthreads_and(arrived ? 1 : 0) != 0;   // factors(n) visible; the previous MMAs done
             tc::fence_after();
             if (!ok) break;
             if (issued > 0) parity ^= 1u;
-        // operands: consecutive threads take consecutive rows (conflict-free 16-byte stores)
-        const float2 *sW = sW0 + (n & 1) * LT_KB * 3;
-        for (int q = tid; q < R_used * 4; q += LT_THREADS) {
-            const int o = (int)(((float)q + 0.5f) * inv_R), r = q - o * R_used;
-            float re[8], im[8];
-            if (!crow) {
-                const int j = (int)(((float)r + 0.5f) * inv_T2), l = r - j * T2;
+        // operand tasks of 8 beams, A's then B's: two rows (j, j+1; l) that share E2, and the three columns (i, c)
+        // that share E0; one row or column each when the components are rows.  Consecutive threads' 16-byte stores
+        // fall into distinct banks.  8 beams of a complex factor as packed pairs:
+        struct Oct {
+            float2 r[4], i[4];
+            __device__ __forceinline__ void load(const float *p, int im = LT_KB) {   // Re at p, Im at p + im
 #pragma unroll
-                for (int u = 0; u < 8; u++) {
-                    const int b = 8 * o + u;
-                    const float2 a1 = sE[b * TA + T0 + j], a2 = sE[b * TA + T0 + T1 + l];
-                    re[u] = a1.x * a2.x - a1.y * a2.y;
-                    im[u] = a1.x * a2.y + a1.y * a2.x;
+                for (int u = 0; u < 2; u++) {
+                    const float4 a = *reinterpret_cast<const float4 *>(p + 4 * u);
+                    const float4 b = *reinterpret_cast<const float4 *>(p + im + 4 * u);
+                    r[2 * u] = make_float2(a.x, a.y);
+                    r[2 * u + 1] = make_float2(a.z, a.w);
+                    i[2 * u] = make_float2(b.x, b.y);
+                    i[2 * u + 1] = make_float2(b.z, b.w);
                 }
-            } else {
-                const int jl = (int)(((float)r + 0.5f) * inv_3), c = r - 3 * jl;
-                if (T2 == 1) {
+            }
+            __device__ __forceinline__ void mul(const Oct &o) {
 #pragma unroll
-                    for (int u = 0; u < 8; u++) {
-                        const int b = 8 * o + u;
-                        const float2 e = sE[b * TA + T0 + jl], wv = sW[b * 3 + c];
-                        re[u] = wv.x * e.x - wv.y * e.y;
-                        im[u] = wv.x * e.y + wv.y * e.x;
+                for (int u = 0; u < 4; u++) {
+                    const float2 mi = make_float2(-i[u].x, -i[u].y);
+                    const float2 re = __ffma2_rn(mi, o.i[u], __fmul2_rn(r[u], o.r[u]));
+                    i[u] = __ffma2_rn(i[u], o.r[u], __fmul2_rn(r[u], o.i[u]));
+                    r[u] = re;
+                }
+            }
+        };
+        auto put_a = [&](int r, int o, const Oct &v) {
+            uint4 hr, lr, hi, li;
+            tc::split8p(v.r, hr, lr);
+            tc::split8p(v.i, hi, li);
+            unsigned char *dst = sA + tc::kmaj_off(r, 8 * o);
+            *reinterpret_cast<uint4 *>(dst) = hr;
+            *reinterpret_cast<uint4 *>(dst + LT_A_BYTES) = lr;
+            *reinterpret_cast<uint4 *>(dst + 2 * LT_A_BYTES) = hi;
+            *reinterpret_cast<uint4 *>(dst + 3 * LT_A_BYTES) = li;
+        };
+        auto put_b = [&](int cq, int o, const Oct &v) {   // B'_re = [Re X ; Im X], B'_im = [-Im X ; Re X]
+            uint4 hr, lr, hi, li;
+            tc::split8p(v.r, hr, lr);
+            tc::split8p(v.i, hi, li);
+            unsigned char *top = sB + tc::kmaj_off(cq, 8 * o), *bot = sB + tc::kmaj_off(nc_tile + cq, 8 * o);
+            const uint32_t sgn = 0x80008000u;
+            *reinterpret_cast<uint4 *>(top) = hr;
+            *reinterpret_cast<uint4 *>(top + LT_B_BYTES) = lr;
+            *reinterpret_cast<uint4 *>(bot) = hi;
+            *reinterpret_cast<uint4 *>(bot + LT_B_BYTES) = li;
+            *reinterpret_cast<uint4 *>(top + 2 * LT_B_BYTES) = make_uint4(hi.x ^ sgn, hi.y ^ sgn, hi.z ^ sgn, hi.w ^ sgn);
+            *reinterpret_cast<uint4 *>(top + 3 * LT_B_BYTES) = make_uint4(li.x ^ sgn, li.y ^ sgn, li.z ^ sgn, li.w ^ sgn);
+            *reinterpret_cast<uint4 *>(bot + 2 * LT_B_BYTES) = hr;
+            *reinterpret_cast<uint4 *>(bot + 3 * LT_B_BYTES) = lr;
+        };
+        for (int q = tid; q < ntask_a32 + ntask_b; q += LT_THREADS) {
+            Oct v, w;
+            if (q < ntask_a) {
+                const int o = (int)(((float)q + 0.5f) * inv_a), r = q - o * (ntask_a >> 2);
+                if (!crow) {
+                    const int jp = (int)(((float)r + 0.5f) * inv_T2), l = r - jp * T2, j = 2 * jp;
+                    w.load(sE + (T0 + T1 + l) * LT_ES + 8 * o);
+                    v.load(sE + (T0 + j) * LT_ES + 8 * o);
+                    v.mul(w);
+                    put_a(j * T2 + l, o, v);
+                    if (j + 1 < T1) {
+                        v.load(sE + (T0 + j + 1) * LT_ES + 8 * o);
+                        v.mul(w);
+                        put_a((j + 1) * T2 + l, o, v);
                     }
                 } else {
+                    const int jl = (int)(((float)r + 0.5f) * inv_3), c = r - 3 * jl;
                     const int j = (int)(((float)jl + 0.5f) * inv_T2), l = jl - j * T2;
+                    v.load(sE + (T0 + j) * LT_ES + 8 * o);
+                    w.load(sE + (T0 + T1 + l) * LT_ES + 8 * o);
+                    v.mul(w);
+                    w.load(sR + (6 + 2 * c) * LT_RS + 8 * o, LT_RS);
+                    v.mul(w);
+                    put_a(r, o, v);
+                }
+            } else if (q >= ntask_a32) {
+                const int qb = q - ntask_a32, o = (int)(((float)qb + 0.5f) * inv_T0), i = qb - o * T0;
+                w.load(sE + i * LT_ES + 8 * o);
+                if (!crow) {
 #pragma unroll
-                    for (int u = 0; u < 8; u++) {
-                        const int b = 8 * o + u;
-                        const float2 a1 = sE[b * TA + T0 + j], a2 = sE[b * TA + T0 + T1 + l];
-                        const float er = a1.x * a2.x - a1.y * a2.y, ei = a1.x * a2.y + a1.y * a2.x;
-                        const float ar = sR[b * REC + 6 + 2 * c], ai = sR[b * REC + 7 + 2 * c];
-                        re[u] = ar * er - ai * ei;
-                        im[u] = ar * ei + ai * er;
+                    for (int c = 0; c < 3; c++) {
+                        v.load(sR + (6 + 2 * c) * LT_RS + 8 * o, LT_RS);
+                        v.mul(w);
+                        put_b(3 * i + c, o, v);
                     }
+                } else {
+                    put_b(i, o, w);
                 }
             }
-            const uint32_t off = tc::kmaj_off(r, 8 * o);
-            tc::split8(sA + 0 * LT_A_BYTES, sA + 1 * LT_A_BYTES, off, re, sA_scale);
-            tc::split8(sA + 2 * LT_A_BYTES, sA + 3 * LT_A_BYTES, off, im, sA_scale);
-        }
-        for (int q = tid; q < nc_used * 4; q += LT_THREADS) {
-            const int o = (int)(((float)q + 0.5f) * inv_nc), cq = q - o * nc_used;
-            float re[8], im[8], nim[8];
-            if (!crow) {
-                const int i = (int)(((float)cq + 0.5f) * inv_3), c = cq - 3 * i;
-#pragma unroll
-                for (int u = 0; u < 8; u++) {
-                    const int b = 8 * o + u;
-                    const float2 e = sE[b * TA + i];
-                    const float ar = sR[b * REC + 6 + 2 * c], ai = sR[b * REC + 7 + 2 * c];
-                    re[u] = ar * e.x - ai * e.y;
-                    im[u] = ar * e.y + ai * e.x;
-                    nim[u] = -im[u];
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < 8; u++) {
-                    const float2 e = sE[(8 * o + u) * TA + cq];
-                    re[u] = e.x;
-                    im[u] = e.y;
-                    nim[u] = -e.y;
-                }
-            }
-            const uint32_t top = tc::kmaj_off(cq, 8 * o), bot = tc::kmaj_off(nc_tile + cq, 8 * o);
-            // B'_re = [Re X ; Im X], B'_im = [-Im X ; Re X]
-            tc::split8(sB + 0 * LT_B_BYTES, sB + 1 * LT_B_BYTES, top, re, sB_scale);
-            tc::split8(sB + 0 * LT_B_BYTES, sB + 1 * LT_B_BYTES, bot, im, sB_scale);
-            tc::split8(sB + 2 * LT_B_BYTES, sB + 3 * LT_B_BYTES, top, nim, sB_scale);
-            tc::split8(sB + 2 * LT_B_BYTES, sB + 3 * LT_B_BYTES, bot, re, sB_scale);
         }
         tc::fence_async_smem();
         tc::fence_before();
@@ -366,10 +398,8 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
         }
         issued++;
         // while the tensor cores work: factors of block n+1, records of block n+2
-        if (n + 1 < nblk)
-            factors(n + 1, sR0 + ((n + 1) & 1) * LT_KB * REC, sE0 + ((n + 1) & 1) * LT_KB * TA,
-                    sW0 + ((n + 1) & 1) * LT_KB * 3);
-        if (n + 2 < nblk) load_records(n + 2, sR0 + (n & 1) * LT_KB * REC);
+        if (n + 1 < nblk) factors(n + 1, sR0 + ((n + 1) & 1) * LT_RS * REC);
+        if (n + 2 < nblk) load_records(n + 2, sR0 + (n & 1) * LT_RS * REC);
         }
         __syncthreads();   // the round's kept list and staging buffers are reused by the next round
     }
@@ -558,7 +588,7 @@ fga_status run_lattice_tc(Workspace &ws, const LatticePlan &plan, const void *re
         return FGA_ERR_UNSUPPORTED;
     }
     LtSmem S;
-    S.init(T0 + T1 + T2, crow && T2 == 1, NR);
+    S.init(T0 + T1 + T2, NR);
     // three CTAs per SM when their tensor memory (3 x tcols <= 512) and shared memory fit
     const bool three = S.tcols <= 128 && S.bytes <= 74 * 1024;
     LtAxes X;

@@ -132,6 +132,21 @@ __device__ __forceinline__ void split8(unsigned char *hi, unsigned char *lo, uin
     *reinterpret_cast<uint4 *>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
+// the hi/lo split of 8 values given as packed pairs (already scaled), as two 16-byte words
+__device__ __forceinline__ void split8p(const float2 v[4], uint4 &hi, uint4 &lo) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const __half2 hh = __float22half2_rn(v[q]);
+        const float2 hf = __half22float2(hh);
+        const __half2 ll = __float22half2_rn(__fadd2_rn(v[q], make_float2(-hf.x, -hf.y)));
+        h[q] = *reinterpret_cast<const uint32_t *>(&hh);
+        l[q] = *reinterpret_cast<const uint32_t *>(&ll);
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
 __device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
