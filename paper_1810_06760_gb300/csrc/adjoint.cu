@@ -15,9 +15,11 @@
 //      ybar_n.
 //   3. the cotangent of the initial amplitudes gives dL/dc(q) through the initial-velocity term.
 // Node-field cotangents are scattered with atomics through the interpolation weights (GradAcc).
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
+#include "cell_cache.cuh"
 #include "fga_beam.cuh"
 #include "gather.cuh"
 
@@ -136,16 +138,62 @@ __device__ __forceinline__ void model_vjp(const ModelDev &M, int wave, const R x
             }
 }
 
+// The model and its adjoint read from global memory.
+template <typename R, int WAVE, int MED, class G> struct DirectModel {
+    const ModelDev &M;
+    G grad;
+    __device__ __forceinline__ void eval(const R Q[3], R cf[10]) const { model_eval<R, MED>(M, WAVE, Q, cf); }
+    __device__ __forceinline__ void vjp(const R Q[3], const R cb[10], R Qb[3]) const {
+        model_vjp<R, MED>(M, WAVE, Q, cb, Qb, grad);
+    }
+};
+// The same through the thread's copy of its grid cell (FP32 grid media; the cell of Q has been prefetched).
+struct CellModel {
+    const ModelDev &M;
+    const CellCache &cell;
+    DeferAcc<float> grad;
+    __device__ __forceinline__ void eval(const float[3], float cf[10]) const { cell.sample(cf); }
+    __device__ __forceinline__ void vjp(const float Q[3], const float cb[10], float Qb[3]) const {
+        grad.put(Q, cb);
+        float dfr[3];   // d fr/dx, zero where x is clamped
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            const float t = (Q[d] - M.fo[d]) * M.finv_h[d];
+            dfr[d] = t < 0.f || t > (float)(M.n[d] - 1) ? 0.f : M.finv_h[d];
+        }
+        const float2 b01 = make_float2(cb[0], cb[1]), b23 = make_float2(cb[2], cb[3]), b45 = make_float2(cb[4], cb[5]),
+                     b67 = make_float2(cb[6], cb[7]), b89 = make_float2(cb[8], cb[9]);
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const float w0 = (c >> 2) ? cell.fr[0] : 1.f - cell.fr[0], w1 = (c >> 1) & 1 ? cell.fr[1] : 1.f - cell.fr[1],
+                        w2 = c & 1 ? cell.fr[2] : 1.f - cell.fr[2];
+            const float g0 = (c >> 2) ? dfr[0] : -dfr[0], g1 = (c >> 1) & 1 ? dfr[1] : -dfr[1], g2 = c & 1 ? dfr[2] : -dfr[2];
+            const float4 *p = cell.col + 3 * c;
+            const float4 u0 = p[0], u1 = p[1];
+            const float2 u2 = *reinterpret_cast<const float2 *>(p + 2);
+            float2 s = __fmul2_rn(b01, make_float2(u0.x, u0.y));
+            s = __ffma2_rn(b23, make_float2(u0.z, u0.w), s);
+            s = __ffma2_rn(b45, make_float2(u1.x, u1.y), s);
+            s = __ffma2_rn(b67, make_float2(u1.z, u1.w), s);
+            s = __ffma2_rn(b89, u2, s);
+            const float dot = s.x + s.y;
+            Qb[0] += dot * g0 * w1 * w2;
+            Qb[1] += dot * w0 * g1 * w2;
+            Qb[2] += dot * w0 * w1 * g2;
+        }
+    }
+};
+
 // ---------------------------------------------------------------------------------------------
 // adjoint of dy/dt (the right-hand side of beam_rhs): yb += (d rhs / dy)^T fb, node-field
-// cotangents to grad.  Complex cotangents follow zb = dL/dRe z + i dL/dIm z.
+// cotangents to the model's accumulator.  Complex cotangents follow zb = dL/dRe z + i dL/dIm z.
 // ---------------------------------------------------------------------------------------------
-template <typename R, int WAVE, int MED, class FB, class G>
-__device__ __forceinline__ void rhs_vjp(const ModelDev &M, R sg, bool ref_e1, const R *__restrict__ y, FB fb,
-                                        R *__restrict__ yb, G grad) {
+template <typename R, int WAVE, class Model, class FB>
+__device__ __forceinline__ void rhs_vjp(const Model &mdl, R sg, bool ref_e1, const R *__restrict__ y, FB fb,
+                                        R *__restrict__ yb) {
     R cf[10];
     const R Q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]};
-    model_eval<R, MED>(M, WAVE, Q, cf);
+    mdl.eval(Q, cf);
     const R c = cf[0];
     const R g[3] = {cf[1], cf[2], cf[3]};
     const R H[3][3] = {{cf[4], cf[5], cf[6]}, {cf[5], cf[7], cf[8]}, {cf[6], cf[8], cf[9]}};
@@ -356,7 +404,7 @@ __device__ __forceinline__ void rhs_vjp(const ModelDev &M, R sg, bool ref_e1, co
 #pragma unroll
     for (int d = 0; d < 3; d++) yb[F_P + d] += Pb[d] + (Phb[d] - Ph[d] * phd) * ip + pnb * Ph[d];
     R Qb[3] = {R(0), R(0), R(0)};
-    model_vjp<R, MED>(M, WAVE, Q, cb, Qb, grad);
+    mdl.vjp(Q, cb, Qb);
 #pragma unroll
     for (int d = 0; d < 3; d++) yb[F_Q + d] += Qb[d];
 }
@@ -543,7 +591,8 @@ __global__ void __launch_bounds__(128) adj_forward_kernel(ModelDev M, const R *_
 }
 
 // Reverse step n, split into one kernel per part so that each keeps about three 46-real arrays
-// live (a single kernel holding the step's state, slopes and cotangents spilled to local memory):
+// live (a single kernel holding the step's state, slopes and cotangents spilled to local memory); FP32 grid media take
+// the last four parts as one kernel with shared-memory columns, adj_step_kernel below:
 //   adj_records_kernel  (steps with samples) record cotangents: ybar_{n+1} += those of y_{n+1} (with
 //                       the adjoint of its slope when a sample lies inside the step); the cotangents of
 //                       y_n and of k1 (Q, P) go to RB;
@@ -641,7 +690,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_records_kernel(ModelDev M, co
         record_vjp<R, WAVE>(e1, y, k1, y1, d1, dt, th, w, rb, y0b, f0b, y1b, f1b);
     }
     if constexpr (D1) {
-        rhs_vjp<R, WAVE, MED>(M, sg, e1, y1, QPBar<R>{f1b}, y1b, grad);
+        rhs_vjp<R, WAVE>(DirectModel<R, WAVE, MED, GradAcc<R>>{M, grad}, sg, e1, y1, QPBar<R>{f1b}, y1b);
 #pragma unroll
         for (int f = 0; f < NF; f++) YB[(int64_t)f * cap + b] += y1b[f];
     } else {
@@ -689,7 +738,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_stage4_kernel(ModelDev M, con
     R sb[NF];
 #pragma unroll
     for (int f = 0; f < NF; f++) sb[f] = R(0);
-    rhs_vjp<R, WAVE, MED>(M, sg, e1, t, fb, sb, grad);
+    rhs_vjp<R, WAVE>(DirectModel<R, WAVE, MED, DeferAcc<R>>{M, grad}, sg, e1, t, fb, sb);
     store_state(SB4, cap, b, sb);
 }
 
@@ -710,7 +759,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_stage_kernel(ModelDev M, cons
     load_state(T, cap, b, t);
 #pragma unroll
     for (int f = 0; f < NF; f++) sb[f] = R(0);
-    rhs_vjp<R, WAVE, MED>(M, sg, e1, t, fb, sb, grad);
+    rhs_vjp<R, WAVE>(DirectModel<R, WAVE, MED, DeferAcc<R>>{M, grad}, sg, e1, t, fb, sb);
     store_state(SBout, cap, b, sb);
 }
 
@@ -741,8 +790,97 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_stage1_kernel(ModelDev M, con
 #pragma unroll
         for (int f = 0; f < 4; f++) yb[F_A0 + f] += RB[(int64_t)(6 + f) * cap + b];
     }
-    rhs_vjp<R, WAVE, MED>(M, sg, e1, y, fb, yb, grad);
+    rhs_vjp<R, WAVE>(DirectModel<R, WAVE, MED, DeferAcc<R>>{M, grad}, sg, e1, y, fb, yb);
     store_state(YB, cap, b, yb);
+}
+
+// The four stage kernels of a reverse step as one (FP32 grid media).  Apart they move about 970 reals per beam and step
+// through HBM (stage inputs, slope cotangents and ybar, written and read again) and gather 24 nodes eleven times from
+// L1.  Here the slope cotangent and the running sum ybar + sb4 + sb3 + sb2 are columns of shared memory, the model
+// is sampled through the cell cache, and the stage inputs t2, t3 pass through a scratch of the resident threads
+// (14 MB: it stays in L2), so HBM sees y_n, ybar in and out and the four node-cotangent records: 190 reals.  The
+// three right-hand sides are one loop and the four adjoints another, so that each is compiled once.  Persistent:
+// two CTAs of 128 threads per SM (96 KB of shared memory each) stride over the class's beams.
+// 1.05 M beams, 200 steps: 245 -> 183 ms (12,100 instructions per warp and step, issue slots 42%: the loads of ybar and
+// the stage inputs from L2 at 8 warps per SM).
+constexpr int ADJ_STEP_SMEM = ADJ_THREADS * (CELL_STRIDE * 16 + 2 * NF * 4);
+template <int WAVE>
+__global__ void __launch_bounds__(ADJ_THREADS, 2) adj_step_kernel(ModelDev M, const float *__restrict__ Sn, float *YB,
+                                                                 const float *__restrict__ RB, float *scratch,
+                                                                 int64_t cap, const int32_t *__restrict__ flags,
+                                                                 int64_t off, int64_t n, float sg, float dt, float *CB,
+                                                                 int64_t rst) {
+    extern __shared__ float4 cells[];
+    float *fbc = reinterpret_cast<float *>(cells + ADJ_THREADS * CELL_STRIDE) + threadIdx.x;
+    float *acc = fbc + NF * ADJ_THREADS;
+    const int64_t nth = (int64_t)gridDim.x * ADJ_THREADS, th = (int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x;
+    float *T = scratch + th;   // field f of t2 at T[f nth], of t3 at T[(NF + f) nth]
+    CellCache cell;
+    cell.init(WAVE ? M.gs : M.gp, cells);
+    const float h = 0.5f * dt;
+    for (int64_t i = th; i < n; i += nth) {
+        const int64_t b = off + i;
+        const bool e1 = (flags[b] & FL_REF_E1) != 0;
+        float t[NF];
+        {
+            float y[NF], kk[NF];
+            load_state(Sn, cap, b, y);
+#pragma unroll
+            for (int f = 0; f < NF; f++) t[f] = y[f];
+            cell.prefetch(M, t);
+#pragma unroll 1
+            for (int e = 0; e < 3; e++) {
+                const float hh = e == 2 ? dt : h;
+                float cf[10], tq[3];
+                cell.sample(cf);
+                // the next position first: its cell is copied while the rest is formed
+                const float ip = rsqrtf(t[F_P] * t[F_P] + t[F_P + 1] * t[F_P + 1] + t[F_P + 2] * t[F_P + 2]), sc = sg * cf[0];
+#pragma unroll
+                for (int d = 0; d < 3; d++) tq[d] = y[F_Q + d] + hh * (sc * (t[F_P + d] * ip));
+                cell.prefetch(M, tq);
+                beam_rhs_at<float, WAVE>(cf, sg, e1, t, kk);
+#pragma unroll
+                for (int f = 0; f < NF; f++) t[f] = f < 3 ? tq[f] : y[f] + hh * kk[f];
+                if (e < 2)
+#pragma unroll
+                    for (int f = 0; f < NF; f++) T[(int64_t)(e * NF + f) * nth] = t[f];
+            }
+        }
+        float sb[NF];
+#pragma unroll
+        for (int f = 0; f < NF; f++) sb[f] = 0.f;
+#pragma unroll 1
+        for (int v = 0; v < 4; v++) {   // stages 4, 3, 2, 1
+            if (v > 0) {
+                const float *src = v == 3 ? Sn + b : T + (int64_t)(v == 1 ? NF : 0) * nth;
+                const int64_t st = v == 3 ? cap : nth;
+#pragma unroll
+                for (int f = 0; f < NF; f++) t[f] = src[(int64_t)f * st];
+                cell.prefetch(M, t);
+            }
+            // slope cotangent a ybar + c sb (+ the records' k1 part), and the running sum
+            const float a = v == 0 || v == 3 ? dt / 6.f : dt / 3.f, c = v == 1 ? dt : h;
+#pragma unroll
+            for (int f = 0; f < NF; f++) {
+                const float yb = YB[(int64_t)f * cap + b];
+                float w = a * yb + c * sb[f];   // sb is zero at stage 4
+                float s = v == 0 ? yb : acc[f * ADJ_THREADS] + sb[f];
+                if (RB) {
+                    if (v == 3 && f < 6) w += RB[(int64_t)(10 + f) * cap + b];
+                    if (v == 0 && f < 6) s += RB[(int64_t)f * cap + b];
+                    if (v == 0 && f >= F_A0) s += RB[(int64_t)(6 + f - F_A0) * cap + b];
+                }
+                fbc[f * ADJ_THREADS] = w;
+                acc[f * ADJ_THREADS] = s;
+            }
+#pragma unroll
+            for (int f = 0; f < NF; f++) sb[f] = 0.f;
+            rhs_vjp<float, WAVE>(CellModel{M, cell, DeferAcc<float>{CB + (int64_t)v * rst, cap, b}}, sg, e1, t,
+                                 StagedBar<float>{fbc}, sb);
+        }
+#pragma unroll
+        for (int f = 0; f < NF; f++) __stcs(YB + (int64_t)f * cap + b, acc[f * ADJ_THREADS] + sb[f]);
+    }
 }
 
 // Node cotangents of the last few reverse steps: nrec stage records (DEFER_FIELDS reals each, record r
@@ -871,8 +1009,9 @@ template <typename R, int WAVE, int MED>
 fga_status reverse_step(const ModelDev &dev, const R *Sn, const R *Sn1, R *YB, R *RS, int64_t cap, int64_t slot,
                         const int32_t *fl, int64_t off, int64_t nc, R sg, R dt, R w, R k, R rw2, int nrx,
                         const R *rx, const R *ubs, const StepSamples &ss, size_t smem, GradAcc<R> gr, int jst,
-                        bool scatter, cudaStream_t s) {
-    R *T2 = RS, *T3 = RS + slot, *SB4 = RS + 2 * slot, *SB3 = RS + 3 * slot, *RB = RS + 4 * slot;
+                        bool scatter, R *scratch, int ctas, cudaStream_t s) {
+    constexpr bool fused = sizeof(R) == 4 && MED == FGA_MEDIUM_GRID;   // RS then holds no state slots
+    R *T2 = RS, *T3 = RS + slot, *SB4 = RS + 2 * slot, *SB3 = RS + 3 * slot, *RB = RS + (fused ? 0 : 4 * slot);
     R *SB2 = T3;  // t3 is dead once sb3 is formed
     const int64_t rst = (int64_t)DEFER_FIELDS * cap;
     // records in path order (latest first): step j holds stage 4, 3, 2, 1 at records 4j .. 4j+3
@@ -885,16 +1024,44 @@ fga_status reverse_step(const ModelDev &dev, const R *Sn, const R *Sn1, R *YB, R
             FGA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<blocks, ADJ_THREADS, smem, s>>>(dev, Sn, Sn1, YB, RB, cap, fl, off, nc, sg, dt, w, k, rw2, nrx, rx, ubs, ss, gr);
     }
-    adj_stage4_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, Sn, YB, T2, T3, SB4, cap, fl, off, nc, sg, dt,
-                                                                  CB);
-    adj_stage_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, T3, YB, SB4, SB3, cap, fl, off, nc, sg, dt / R(3), dt,
-                                                                 CB + rst);
-    adj_stage_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, T2, YB, SB3, SB2, cap, fl, off, nc, sg, dt / R(3),
-                                                                 R(0.5) * dt, CB + 2 * rst);
-    adj_stage1_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, Sn, YB, SB4, SB3, SB2, ss.nsj > 0 ? RB : nullptr,
-                                                                  cap, fl, off, nc, sg, dt, CB + 3 * rst);
+    if constexpr (fused) {
+        FGA_CUDA(cudaFuncSetAttribute(adj_step_kernel<WAVE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ADJ_STEP_SMEM));
+        adj_step_kernel<WAVE><<<(unsigned)std::min<int64_t>(ctas, blocks), ADJ_THREADS, ADJ_STEP_SMEM, s>>>(
+            dev, Sn, YB, ss.nsj > 0 ? RB : nullptr, scratch, cap, fl, off, nc, sg, dt, CB, rst);
+    } else {
+        adj_stage4_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, Sn, YB, T2, T3, SB4, cap, fl, off, nc, sg, dt,
+                                                                      CB);
+        adj_stage_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, T3, YB, SB4, SB3, cap, fl, off, nc, sg, dt / R(3), dt,
+                                                                     CB + rst);
+        adj_stage_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, T2, YB, SB3, SB2, cap, fl, off, nc, sg, dt / R(3),
+                                                                     R(0.5) * dt, CB + 2 * rst);
+        adj_stage1_kernel<R, WAVE, MED><<<blocks, ADJ_THREADS, 0, s>>>(dev, Sn, YB, SB4, SB3, SB2, ss.nsj > 0 ? RB : nullptr,
+                                                                      cap, fl, off, nc, sg, dt, CB + 3 * rst);
+    }
     if (MED == FGA_MEDIUM_GRID && scatter)
         adj_scatter_kernel<R, WAVE><<<blocks, ADJ_THREADS, 0, s>>>(dev, CB0, 4 * (jst + 1), cap, off, nc, gr);
+    FGA_CUDA(cudaGetLastError());
+    return FGA_OK;
+}
+
+// nsteps steps from slot 0 of S, the state after every every-th in the next slot
+template <typename R, int MED>
+fga_status forward_states(const ModelDev &dev, const fga_beams *b, R *S, int64_t cap, int64_t slot, R dt, int nsteps,
+                          int every, cudaStream_t s) {
+    const int32_t *fl = b->flags.as<int32_t>();
+    for (int cls = 0; cls < 4; cls++) {
+        const int64_t nc = b->n_cls[cls];
+        if (!nc) continue;
+        const R sg = (cls & 1) ? R(-1) : R(1);
+        const unsigned blocks = (unsigned)((nc + 127) / 128);
+        ProfScope ps(P_ADJ_FWD, s);
+        if (cls < 2)
+            adj_forward_kernel<R, 0, MED><<<blocks, 128, 0, s>>>(dev, S, S, cap, slot, fl, b->off_cls[cls], nc, sg, dt,
+                                                                nsteps, every);
+        else
+            adj_forward_kernel<R, 1, MED><<<blocks, 128, 0, s>>>(dev, S, S, cap, slot, fl, b->off_cls[cls], nc, sg, dt,
+                                                                nsteps, every);
+    }
     FGA_CUDA(cudaGetLastError());
     return FGA_OK;
 }
@@ -929,9 +1096,19 @@ fga_status run_vjp(const fga_model *m, const fga_init_desc *init, const fga_solv
     }
     // reverse-step scratch: t2, t3 (t3's slot then holds sb2), sb4, sb3, RB_FIELDS record fields and the
     // deferred node cotangents of SCATTER_STEPS steps
-    ScopedDevBuf rs;
-    FGA_TRY(rs.ensure(sizeof(R) *
-                      ((size_t)slot * 4 + (size_t)(RB_FIELDS + 4 * SCATTER_STEPS * DEFER_FIELDS) * (size_t)cap)));
+    // (the fused step needs no state slots, but a scratch of two states per resident thread)
+    constexpr bool fused = sizeof(R) == 4 && MED == FGA_MEDIUM_GRID;
+    ScopedDevBuf rs, scr;
+    FGA_TRY(rs.ensure(sizeof(R) * ((fused ? 0 : (size_t)slot * 4) +
+                                   (size_t)(RB_FIELDS + 4 * SCATTER_STEPS * DEFER_FIELDS) * (size_t)cap)));
+    int ctas = 0;
+    if (fused) {
+        int dev = 0, sms = 152;
+        FGA_CUDA(cudaGetDevice(&dev));
+        FGA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        ctas = 2 * sms;
+        FGA_TRY(scr.ensure(sizeof(R) * 2 * NF * ADJ_THREADS * (size_t)ctas));
+    }
     R *CK = ck.as<R>(), *SEG = seg.as<R>(), *YB = yb.as<R>(), *RS = rs.as<R>();
     const int64_t nn = MED == FGA_MEDIUM_GRID ? (int64_t)m->dev.n[0] * m->dev.n[1] * m->dev.n[2] : 0;
     ScopedDevBuf sgp, sgs;
@@ -945,19 +1122,7 @@ fga_status run_vjp(const fga_model *m, const fga_init_desc *init, const fga_solv
     const R dt = (R)sd->dt;
     // 1. checkpoints at steps C, 2C, ... (the last one at N when C does not divide N is not needed)
     NvtxRange nr_fwd("fga_solve_vjp: checkpoints");
-    for (int cls = 0; cls < 4; cls++) {
-        const int64_t nc = b->n_cls[cls];
-        if (!nc) continue;
-        const R sg = (cls & 1) ? R(-1) : R(1);
-        const unsigned blocks = (unsigned)((nc + 127) / 128);
-        ProfScope ps(P_ADJ_FWD, s);
-        if (cls < 2)
-            adj_forward_kernel<R, 0, MED><<<blocks, 128, 0, s>>>(m->dev, CK, CK, cap, slot, fl, b->off_cls[cls], nc, sg,
-                                                                dt, (nseg - 1) * C, C);
-        else
-            adj_forward_kernel<R, 1, MED><<<blocks, 128, 0, s>>>(m->dev, CK, CK, cap, slot, fl, b->off_cls[cls], nc, sg,
-                                                                dt, (nseg - 1) * C, C);
-    }
+    FGA_TRY((forward_states<R, MED>(m->dev, b, CK, cap, slot, dt, (nseg - 1) * C, C, s)));
     FGA_CUDA(cudaGetLastError());
     const size_t smem_max = 200 * 1024;
     int j = (int)sstep.size() - 1;
@@ -967,20 +1132,7 @@ fga_status run_vjp(const fga_model *m, const fga_init_desc *init, const fga_solv
         const int n0 = sgi * C, len = std::min(C, N - n0);
         // 2a. the segment's states: slot 0 = checkpoint, slots 1..len recomputed
         FGA_CUDA(cudaMemcpyAsync(SEG, CK + (size_t)sgi * slot, sizeof(R) * (size_t)slot, cudaMemcpyDeviceToDevice, s));
-        for (int cls = 0; cls < 4; cls++) {
-            const int64_t nc = b->n_cls[cls];
-            if (!nc) continue;
-            const R sg = (cls & 1) ? R(-1) : R(1);
-            const unsigned blocks = (unsigned)((nc + 127) / 128);
-            ProfScope ps(P_ADJ_FWD, s);
-            if (cls < 2)
-                adj_forward_kernel<R, 0, MED><<<blocks, 128, 0, s>>>(m->dev, SEG, SEG, cap, slot, fl, b->off_cls[cls],
-                                                                    nc, sg, dt, len, 1);
-            else
-                adj_forward_kernel<R, 1, MED><<<blocks, 128, 0, s>>>(m->dev, SEG, SEG, cap, slot, fl, b->off_cls[cls],
-                                                                    nc, sg, dt, len, 1);
-        }
-        FGA_CUDA(cudaGetLastError());
+        FGA_TRY((forward_states<R, MED>(m->dev, b, SEG, cap, slot, dt, len, 1, s)));
         // 2b. reverse steps
         for (int n = n0 + len - 1; n >= n0; n--) {
             StepSamples ss{};
@@ -1011,11 +1163,11 @@ fga_status run_vjp(const fga_model *m, const fga_init_desc *init, const fga_solv
                 if (cls < 2)
                     FGA_TRY((reverse_step<R, 0, MED>(m->dev, Sn, Sn1, YB, RS, cap, slot, fl, b->off_cls[cls], nc,
                                                      (cls & 1) ? R(-1) : R(1), dt, (R)b->w, (R)b->k, (R)(rw * rw),
-                                                     (int)nrx, rxd.as<R>(), ubs, ss, smem, accp, jst, scatter, s)));
+                                                     (int)nrx, rxd.as<R>(), ubs, ss, smem, accp, jst, scatter, scr.as<R>(), ctas, s)));
                 else
                     FGA_TRY((reverse_step<R, 1, MED>(m->dev, Sn, Sn1, YB, RS, cap, slot, fl, b->off_cls[cls], nc,
                                                      (cls & 1) ? R(-1) : R(1), dt, (R)b->w, (R)b->k, (R)(rw * rw),
-                                                     (int)nrx, rxd.as<R>(), ubs, ss, smem, accs, jst, scatter, s)));
+                                                     (int)nrx, rxd.as<R>(), ubs, ss, smem, accs, jst, scatter, scr.as<R>(), ctas, s)));
             }
             FGA_CUDA(cudaGetLastError());
             jst = scatter ? 0 : jst + 1;
