@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "fga_beam.cuh"
 #include "tc_gemm.cuh"
@@ -162,22 +163,42 @@ static double kernel_row_sum_max(int nq, double q0, double dq, int ny, double y0
     return best;
 }
 
-// initial state and flags of the beam of mesh point mi and class cls
-template <typename R, int MED>
-__device__ __forceinline__ void beam_init_state(const ModelDev &Md, const C2<R> *__restrict__ F,
-                                                const C2<R> *__restrict__ G, int nq, int np, double3 q0, double3 dq,
-                                                double3 p0, double3 dp, double k, int64_t mi, int cls, R *y, int &fl) {
-    const int64_t NP = (int64_t)np * np * np;
-    const int64_t iq = mi / NP, ip = mi % NP;
-    const int qi[3] = {(int)(iq / ((int64_t)nq * nq)), (int)((iq / nq) % nq), (int)(iq % nq)};
-    const int pj[3] = {(int)(ip / ((int64_t)np * np)), (int)((ip / np) % np), (int)(ip % np)};
-    const double qd[3] = {q0.x + qi[0] * dq.x, q0.y + qi[1] * dq.y, q0.z + qi[2] * dq.z};
-    const double pd[3] = {p0.x + pj[0] * dp.x, p0.y + pj[1] * dp.y, p0.z + pj[2] * dp.z};
+struct MeshIndex {
+    int q[3], p[3];
+    int64_t f;   // of F's first component at the point
+};
+
+__device__ __forceinline__ MeshIndex mesh_index(int nq, int np, uint32_t mi) {
+    const uint32_t p1 = (uint32_t)np, q1 = (uint32_t)nq;
+    MeshIndex x;
+    uint32_t t = mi / p1;
+    x.p[2] = (int)(mi - t * p1);
+    uint32_t u = t / p1;
+    x.p[1] = (int)(t - u * p1);
+    t = u / p1;
+    x.p[0] = (int)(u - t * p1);
+    u = t / q1;
+    x.q[2] = (int)(t - u * q1);
+    t = u / q1;
+    x.q[1] = (int)(u - t * q1);
+    x.q[0] = (int)t;
     const int A = nq * np;
-    const int64_t fidx = (((int64_t)(qi[0] * np + pj[0]) * A + (qi[1] * np + pj[1])) * A + (qi[2] * np + pj[2])) * 3;
+    x.f = (((int64_t)(x.q[0] * np + x.p[0]) * A + (x.q[1] * np + x.p[1])) * A + (x.q[2] * np + x.p[2])) * 3;
+    return x;
+}
+
+__device__ __forceinline__ double axis_node(double3 o, double3 d, int axis, int i) {
+    const double a = axis == 0 ? o.x : axis == 1 ? o.y : o.z, h = axis == 0 ? d.x : axis == 1 ? d.y : d.z;
+    return a + i * h;
+}
+
+// initial amplitudes (2^{3/2} psi, two components) and flags of the beam at q, p (qd: q in FP64, read in layered media
+// only) of class cls
+template <typename R, int MED>
+__device__ __forceinline__ void beam_amplitudes(const ModelDev &Md, const C2<R> *__restrict__ F,
+                                                const C2<R> *__restrict__ G, int64_t fidx, const double *qd, const R *q,
+                                                const R *p, double k, int cls, R *amp, int &fl) {
     const int wave = cls >= 2;
-    R q[3] = {(R)qd[0], (R)qd[1], (R)qd[2]};
-    R p[3] = {(R)pd[0], (R)pd[1], (R)pd[2]};
     R cf[10];
     // layered media: the layer of q from its depth along the layer normal (x3 unless the layers are tilted),
     // minus its distance to the centre of spherical layers, or the undulating interfaces at or above it;
@@ -217,7 +238,7 @@ __device__ __forceinline__ void beam_init_state(const ModelDev &Md, const C2<R> 
         nd = 2;
     }
     const R a0 = R(2.8284271247461900976033774484194);  // 2^{3/2}
-    R amp[4] = {R(0), R(0), R(0), R(0)};
+    for (int j = 0; j < 4; j++) amp[j] = R(0);
     for (int j = 0; j < nd; j++) {
         R fr = R(0), fi = R(0), gr = R(0), gi = R(0);
         for (int d = 0; d < 3; d++) {
@@ -233,6 +254,22 @@ __device__ __forceinline__ void beam_init_state(const ModelDev &Md, const C2<R> 
         amp[2 * j + 1] = a0 * R(0.5) * (fi + gsc * gr);
     }
     if (MED == FGA_MEDIUM_LAYERED) fl |= (lay << 4) | (cls << FL_ROOT_SHIFT);
+}
+
+// initial state and flags of the beam of mesh point mi and class cls
+template <typename R, int MED>
+__device__ __forceinline__ void beam_init_state(const ModelDev &Md, const C2<R> *__restrict__ F,
+                                                const C2<R> *__restrict__ G, int nq, int np, double3 q0, double3 dq,
+                                                double3 p0, double3 dp, double k, uint32_t mi, int cls, R *y, int &fl) {
+    const MeshIndex x = mesh_index(nq, np, mi);
+    double qd[3];
+    R q[3], p[3], amp[4];
+    for (int d = 0; d < 3; d++) {
+        qd[d] = axis_node(q0, dq, d, x.q[d]);
+        q[d] = (R)qd[d];
+        p[d] = (R)axis_node(p0, dp, d, x.p[d]);
+    }
+    beam_amplitudes<R, MED>(Md, F, G, x.f, qd, q, p, k, cls, amp, fl);
     for (int f = 0; f < NF; f++) y[f] = R(0);
     for (int d = 0; d < 3; d++) {
         y[F_Q + d] = q[d];
@@ -246,9 +283,9 @@ __device__ __forceinline__ void beam_init_state(const ModelDev &Md, const C2<R> 
     y[F_A1 + 1] = amp[3];
 }
 
-// |psi|^2 of a beam from its initial amplitudes (2^{3/2} psi): the same value on every pass
-template <typename R> __device__ __forceinline__ R psi_mag2(const R *y) {
-    return y[F_A0] * y[F_A0] + y[F_A0 + 1] * y[F_A0 + 1] + y[F_A1] * y[F_A1] + y[F_A1 + 1] * y[F_A1 + 1];
+// |psi|^2 of a beam from its initial amplitudes (2^{3/2} psi)
+template <typename R> __device__ __forceinline__ R psi_mag2(const R *a) {
+    return a[0] * a[0] + a[1] * a[1] + a[2] * a[2] + a[3] * a[3];
 }
 
 // keep rule of the psi-threshold selection: |psi|^2 > eps^2 max|psi|^2 (amax2 holds the bits of the max)
@@ -264,20 +301,18 @@ template <> struct MaxBits<double> {
     static __device__ double val(U u) { return __longlong_as_double((long long)u); }
 };
 
-// one beam per (mesh point, requested class); with sel != NULL only the beams whose sel[mi] differs
-// from sel[mi + 1] (an exclusive scan of the keep flags) are written, at off + sel[mi]
+// one beam per (mesh point, requested class)
 template <typename R, int MED>
 __global__ void beam_init_kernel(ModelDev Md, const C2<R> *__restrict__ F, const C2<R> *__restrict__ G, int nq, int np,
                                  double3 q0, double3 dq, double3 p0, double3 dp, double k, int64_t M, int cls,
                                  int64_t off, int64_t cap, R *__restrict__ st, int32_t *__restrict__ flags,
-                                 int32_t *__restrict__ ids, const uint32_t *__restrict__ sel) {
+                                 int32_t *__restrict__ ids) {
     const int64_t mi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (mi >= M) return;
-    if (sel && sel[mi + 1] == sel[mi]) return;
     R y[NF];
     int fl;
-    beam_init_state<R, MED>(Md, F, G, nq, np, q0, dq, p0, dp, k, mi, cls, y, fl);
-    const int64_t b = off + (sel ? (int64_t)sel[mi] : mi);
+    beam_init_state<R, MED>(Md, F, G, nq, np, q0, dq, p0, dp, k, (uint32_t)mi, cls, y, fl);
+    const int64_t b = off + mi;
     for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
     flags[b] = fl;
     ids[b] = (int32_t)mi;
@@ -299,54 +334,174 @@ __global__ void rotate_to_layer_frame_kernel(ModelDev Md, R *__restrict__ st, in
     for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
 }
 
-// pass 1 of the selection: the largest |psi|^2 over the class (block maximum, one atomic per block)
-template <typename R, int MED>
-__global__ void __launch_bounds__(128) psi_max_kernel(ModelDev Md, const C2<R> *__restrict__ F,
-                                                      const C2<R> *__restrict__ G, int nq, int np, double3 q0,
-                                                      double3 dq, double3 p0, double3 dp, double k, int64_t M, int cls,
-                                                      typename MaxBits<R>::U *__restrict__ amax2) {
-    const int64_t mi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    R m2 = R(0);
-    if (mi < M) {
-        R y[NF];
-        int fl;
-        beam_init_state<R, MED>(Md, F, G, nq, np, q0, dq, p0, dp, k, mi, cls, y, fl);
-        m2 = psi_mag2<R>(y);
-        if (!(m2 == m2)) m2 = R(0);   // a NaN amplitude is reported by the solve, not selected on
+// The psi-threshold selection (beams with |psi| > eps max|psi|) takes three passes over the mesh, each with all
+// requested classes: the largest |psi|^2, the keep masks (a byte a point) with the counts of every tile and class,
+// and the initial states of the kept beams at their places in mesh order (exclusive scan of the counts, class by class).
+// What bounds it: the points' transform values (24 B, 48 B with initial velocities) read twice from HBM, and
+// the index and frame arithmetic of two passes.  The axis nodes come from tables in shared memory (in FP64 per point
+// they took longer than the rest), the classes of a point share its loads, and the third pass lists the tile's kept
+// beams first, so that whole warps form and store them.  22 M points, 13.9 M beams kept, FP32, constant medium: one launch
+// per class and pass with scanned 4-byte flags 7.9 ms, this 1.9 ms (0.45 + 0.45 + 1.0).
+constexpr int SEL_THREADS = 256, SEL_TILE = 1024;
+
+struct MeshDev {
+    int nq, np;
+    double3 q0, dq, p0, dp;
+    double k;
+    uint32_t M, classes;
+};
+
+// the block's axis tables: q as Q (FP64 where the layers are decided on it), then p
+template <typename R, int MED> struct MeshTable {
+    using Q = typename std::conditional<MED == FGA_MEDIUM_LAYERED, double, R>::type;
+    Q *q;
+    R *p;
+    __device__ MeshTable(const MeshDev &m, double *smem) : q(reinterpret_cast<Q *>(smem)), p(reinterpret_cast<R *>(q + 3 * m.nq)) {
+        for (int i = threadIdx.x; i < 3 * m.nq; i += blockDim.x) q[i] = (Q)axis_node(m.q0, m.dq, i / m.nq, i % m.nq);
+        for (int i = threadIdx.x; i < 3 * m.np; i += blockDim.x) p[i] = (R)axis_node(m.p0, m.dp, i / m.np, i % m.np);
+        __syncthreads();
     }
-    for (int o = 16; o; o >>= 1) m2 = max(m2, __shfl_xor_sync(0xffffffffu, m2, o));
-    __shared__ R wm[4];
-    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const R b = max(max(wm[0], wm[1]), max(wm[2], wm[3]));
-        atomicMax(amax2, MaxBits<R>::bits(b));
+    static size_t bytes(const MeshDev &m) { return 3 * ((size_t)m.nq * sizeof(Q) + (size_t)m.np * sizeof(R)); }
+};
+
+// |psi|^2 of the requested classes at point mi
+template <typename R, int MED>
+__device__ __forceinline__ void point_mags(const ModelDev &Md, const C2<R> *__restrict__ F, const C2<R> *__restrict__ G,
+                                           const MeshDev &m, const MeshTable<R, MED> &tab, uint32_t mi, R *mag) {
+    const MeshIndex x = mesh_index(m.nq, m.np, mi);
+    double qd[3];
+    R q[3], p[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const auto v = tab.q[d * m.nq + x.q[d]];
+        qd[d] = v;
+        q[d] = (R)v;
+        p[d] = tab.p[d * m.np + x.p[d]];
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        if (m.classes >> c & 1) {
+            R amp[4];
+            int fl;
+            beam_amplitudes<R, MED>(Md, F, G, x.f, qd, q, p, m.k, c, amp, fl);
+            mag[c] = psi_mag2<R>(amp);
+        }
     }
 }
 
-// pass 2: keep[mi] = 1 for |psi|^2 > eps2 * max|psi|^2, keep[M] = 0 (room for the scan's total); the
-// class's survivor count is added to *count
 template <typename R, int MED>
-__global__ void __launch_bounds__(128) psi_keep_kernel(ModelDev Md, const C2<R> *__restrict__ F,
-                                                       const C2<R> *__restrict__ G, int nq, int np, double3 q0,
-                                                       double3 dq, double3 p0, double3 dp, double k, int64_t M,
-                                                       int cls, const typename MaxBits<R>::U *__restrict__ amax2,
-                                                       R eps2, uint32_t *__restrict__ keep,
-                                                       unsigned long long *__restrict__ count) {
-    const int64_t mi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned kf = 0;
-    if (mi < M) {
+__global__ void __launch_bounds__(SEL_THREADS) psi_max_kernel(ModelDev Md, const C2<R> *__restrict__ F,
+                                                              const C2<R> *__restrict__ G, MeshDev m,
+                                                              typename MaxBits<R>::U *__restrict__ amax2) {
+    extern __shared__ double tabs[];
+    const MeshTable<R, MED> tab(m, tabs);
+    R m2 = R(0);
+    for (uint64_t mi = (uint64_t)blockIdx.x * SEL_THREADS + threadIdx.x; mi < m.M; mi += (uint64_t)gridDim.x * SEL_THREADS) {
+        R mag[4];
+        point_mags<R, MED>(Md, F, G, m, tab, (uint32_t)mi, mag);
+#pragma unroll
+        for (int c = 0; c < 4; c++)   // a NaN amplitude is reported by the solve, not selected on
+            if ((m.classes >> c & 1) && mag[c] > m2) m2 = mag[c];
+    }
+    for (int o = 16; o; o >>= 1) m2 = max(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+    if ((threadIdx.x & 31) == 0 && m2 > R(0)) atomicMax(amax2, MaxBits<R>::bits(m2));
+}
+
+// keep[mi]: bit c set for |psi|^2 > eps2 max|psi|^2; tile_count[c][tile] and the classes' totals
+template <typename R, int MED>
+__global__ void __launch_bounds__(SEL_THREADS) psi_keep_kernel(ModelDev Md, const C2<R> *__restrict__ F,
+                                                               const C2<R> *__restrict__ G, MeshDev m,
+                                                               const typename MaxBits<R>::U *__restrict__ amax2, R eps2,
+                                                               uint8_t *__restrict__ keep, uint32_t *__restrict__ tile_count,
+                                                               unsigned long long *__restrict__ count) {
+    extern __shared__ double tabs[];
+    __shared__ unsigned n[4];
+    if (threadIdx.x < 4) n[threadIdx.x] = 0;
+    const MeshTable<R, MED> tab(m, tabs);
+    const R lim = eps2 * MaxBits<R>::val(*amax2);
+    unsigned wn[4] = {0, 0, 0, 0};
+    for (int j = 0; j < SEL_TILE / SEL_THREADS; j++) {
+        const uint64_t mi = (uint64_t)blockIdx.x * SEL_TILE + j * SEL_THREADS + threadIdx.x;
+        unsigned kf = 0;
+        if (mi < m.M) {
+            R mag[4];
+            point_mags<R, MED>(Md, F, G, m, tab, (uint32_t)mi, mag);
+#pragma unroll
+            for (int c = 0; c < 4; c++)
+                if ((m.classes >> c & 1) && mag[c] > lim) kf |= 1u << c;
+            keep[mi] = (uint8_t)kf;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; c++) wn[c] += __popc(__ballot_sync(0xffffffffu, kf >> c & 1));
+    }
+    if ((threadIdx.x & 31) == 0)
+        for (int c = 0; c < 4; c++)
+            if (wn[c]) atomicAdd(&n[c], wn[c]);
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        tile_count[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = n[threadIdx.x];
+        if (n[threadIdx.x]) atomicAdd(&count[threadIdx.x], (unsigned long long)n[threadIdx.x]);
+    }
+}
+
+// the kept beams of a tile: listed in shared memory in class and mesh order, then formed and stored
+template <typename R, int MED>
+__global__ void __launch_bounds__(SEL_THREADS) beam_init_kept_kernel(ModelDev Md, const C2<R> *__restrict__ F,
+                                                                     const C2<R> *__restrict__ G, MeshDev m,
+                                                                     const uint8_t *__restrict__ keep,
+                                                                     const uint32_t *__restrict__ tile_off, int64_t cap,
+                                                                     R *__restrict__ st, int32_t *__restrict__ flags,
+                                                                     int32_t *__restrict__ ids) {
+    constexpr int NW = SEL_THREADS / 32, PER = SEL_TILE / SEL_THREADS;
+    __shared__ uint16_t list[4 * SEL_TILE];       // class << 10 | point of the tile
+    __shared__ unsigned cnt[4 * NW], first[4 * NW + 1];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t tile0 = (uint64_t)blockIdx.x * SEL_TILE;
+    unsigned bal[PER][4], n[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < PER; j++) {   // a warp's points are consecutive
+        const uint64_t mi = tile0 + (w * PER + j) * 32 + lane;
+        const unsigned kf = mi < m.M ? keep[mi] : 0u;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            bal[j][c] = __ballot_sync(0xffffffffu, kf >> c & 1);
+            n[c] += __popc(bal[j][c]);
+        }
+    }
+    if (lane == 0)
+        for (int c = 0; c < 4; c++) cnt[c * NW + w] = n[c];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned t = 0;
+        for (int i = 0; i < 4 * NW; i++) {
+            first[i] = t;
+            t += cnt[i];
+        }
+        first[4 * NW] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        unsigned at = first[c * NW + w];
+#pragma unroll
+        for (int j = 0; j < PER; j++) {
+            if (bal[j][c] >> lane & 1)
+                list[at + __popc(bal[j][c] & ((1u << lane) - 1))] = (uint16_t)(c << 10 | ((w * PER + j) * 32 + lane));
+            at += __popc(bal[j][c]);
+        }
+    }
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < first[4 * NW]; i += SEL_THREADS) {
+        const int c = list[i] >> 10;
+        const uint32_t mi = (uint32_t)tile0 + (list[i] & (SEL_TILE - 1));
         R y[NF];
         int fl;
-        beam_init_state<R, MED>(Md, F, G, nq, np, q0, dq, p0, dp, k, mi, cls, y, fl);
-        const R lim = eps2 * MaxBits<R>::val(*amax2);
-        kf = psi_mag2<R>(y) > lim ? 1u : 0u;
-        keep[mi] = kf;
-    } else if (mi == M) {
-        keep[M] = 0u;
+        beam_init_state<R, MED>(Md, F, G, m.nq, m.np, m.q0, m.dq, m.p0, m.dp, m.k, mi, c, y, fl);
+        const int64_t b = (int64_t)tile_off[(int64_t)c * gridDim.x + blockIdx.x] + (i - first[c * NW]);
+        for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
+        flags[b] = fl;
+        ids[b] = (int32_t)mi;
     }
-    const unsigned n = __popc(__ballot_sync(0xffffffffu, kf));
-    if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
 }
 
 // F (and G from g, if both are given) = the transform of Eq. psi in the per-axis pair layout
@@ -462,33 +617,30 @@ static fga_status decompose_medium(const fga_model *m, const fga_init_desc *d, f
     const double3 p0 = {d->p0[0], d->p0[1], d->p0[2]}, dp = {d->dp[0], d->dp[1], d->dp[2]};
     const bool select = d->psi_rel_min > 0;
     using U = typename MaxBits<R>::U;
-    ScopedDevBuf keepb, selb;
-    U *amax2 = nullptr;
-    unsigned long long *cnt = nullptr;
-    uint32_t *keep = nullptr;
-    const R eps2 = (R)(d->psi_rel_min * d->psi_rel_min);
-    const unsigned kblocks = (unsigned)((M + 1 + 127) / 128);
+    ScopedDevBuf keepb, tileb, selb;
+    const MeshDev mesh = {d->nq, d->np, q0, dq, p0, dp, d->k, (uint32_t)M, d->class_mask};
+    const unsigned tiles = (unsigned)((M + SEL_TILE - 1) / SEL_TILE);
     if (select) {
         // Step 1 of Fig. fig:FGA_alg chooses the beams worth propagating: |psi| > eps max|psi|, the maximum
         // over every requested class and mesh point
+        using U = typename MaxBits<R>::U;
+        const R eps2 = (R)(d->psi_rel_min * d->psi_rel_min);
+        const size_t smem = MeshTable<R, MED>::bytes(mesh);
         FGA_TRY(selb.ensure(64));
-        amax2 = selb.as<U>();
-        cnt = reinterpret_cast<unsigned long long *>(selb.as<char>() + 16);
+        U *amax2 = selb.as<U>();
+        unsigned long long *cnt = reinterpret_cast<unsigned long long *>(selb.as<char>() + 16);
         FGA_CUDA(cudaMemsetAsync(selb.p, 0, 64, s));
-        FGA_TRY(keepb.ensure(sizeof(uint32_t) * (size_t)(M + 1)));
-        keep = keepb.as<uint32_t>();
-        for (int cls = 0; cls < 4; cls++) {
-            if (!(d->class_mask & (1u << cls))) continue;
+        FGA_TRY(keepb.ensure((size_t)M));
+        FGA_TRY(tileb.ensure(sizeof(uint32_t) * 4 * (size_t)tiles));
+        {
             ProfScope ps(P_DECOMP, s);
-            psi_max_kernel<R, MED><<<(unsigned)((M + 127) / 128), 128, 0, s>>>(m->dev, F, G, d->nq, d->np, q0, dq, p0,
-                                                                              dp, d->k, M, cls, amax2);
+            psi_max_kernel<R, MED><<<std::min(tiles, 152u * 8u), SEL_THREADS, smem, s>>>(m->dev, F, G, mesh, amax2);
         }
         FGA_CUDA(cudaGetLastError());
-        for (int cls = 0; cls < 4; cls++) {
-            if (!(d->class_mask & (1u << cls))) continue;
+        {
             ProfScope ps(P_DECOMP, s);
-            psi_keep_kernel<R, MED><<<kblocks, 128, 0, s>>>(m->dev, F, G, d->nq, d->np, q0, dq, p0, dp, d->k, M, cls,
-                                                            amax2, eps2, keep, cnt + cls);
+            psi_keep_kernel<R, MED><<<tiles, SEL_THREADS, smem, s>>>(m->dev, F, G, mesh, amax2, eps2, keepb.as<uint8_t>(),
+                                                                     tileb.as<uint32_t>(), cnt);
         }
         FGA_CUDA(cudaGetLastError());
         unsigned long long hc[4];
@@ -496,7 +648,7 @@ static fga_status decompose_medium(const fga_model *m, const fga_init_desc *d, f
         FGA_CUDA(cudaStreamSynchronize(s));
         int64_t tot = 0;
         for (int c = 0; c < 4; c++) {
-            b->n_cls[c] = (d->class_mask & (1u << c)) ? (int64_t)hc[c] : 0;
+            b->n_cls[c] = (int64_t)hc[c];
             tot += b->n_cls[c];
         }
         FGA_CHECK(tot < (int64_t)1 << 31, "fga_decompose: more than 2^31 selected beams");
@@ -504,21 +656,20 @@ static fga_status decompose_medium(const fga_model *m, const fga_init_desc *d, f
         for (int c = 0; c < 4; c++) b->n_cls[c] = (d->class_mask & (1u << c)) ? M : 0;
     }
     FGA_TRY(beams_allocate(b, d, s));
-    for (int cls = 0; cls < 4; cls++) {
+    if (select && b->nb > 0) {
+        FGA_TRY(scan_exclusive_u32(tileb.as<uint32_t>(), 4 * (int64_t)tiles, s));
+        ProfScope ps(P_DECOMP, s);
+        beam_init_kept_kernel<R, MED><<<tiles, SEL_THREADS, 0, s>>>(m->dev, F, G, mesh, keepb.as<uint8_t>(),
+                                                                    tileb.as<uint32_t>(), b->cap, b->state.as<R>(),
+                                                                    b->flags.as<int32_t>(), b->id.as<int32_t>());
+        FGA_CUDA(cudaGetLastError());
+    }
+    for (int cls = 0; cls < 4 && !select; cls++) {
         if (!b->n_cls[cls]) continue;
-        if (select) {
-            {
-                ProfScope ps(P_DECOMP, s);
-                psi_keep_kernel<R, MED><<<kblocks, 128, 0, s>>>(m->dev, F, G, d->nq, d->np, q0, dq, p0, dp, d->k, M,
-                                                                cls, amax2, eps2, keep, cnt + 4);
-            }
-            FGA_CUDA(cudaGetLastError());
-            FGA_TRY(scan_exclusive_u32(keep, M + 1, s));
-        }
         ProfScope ps(P_DECOMP, s);
         beam_init_kernel<R, MED><<<(unsigned)((M + 127) / 128), 128, 0, s>>>(
             m->dev, F, G, d->nq, d->np, q0, dq, p0, dp, d->k, M, cls, b->off_cls[cls], b->cap, b->state.as<R>(),
-            b->flags.as<int32_t>(), b->id.as<int32_t>(), select ? keep : nullptr);
+            b->flags.as<int32_t>(), b->id.as<int32_t>());
         FGA_CUDA(cudaGetLastError());
     }
     if (MED == FGA_MEDIUM_LAYERED && m->dev.tilted) {
