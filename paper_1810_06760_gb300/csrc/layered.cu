@@ -23,10 +23,6 @@ __device__ __forceinline__ Cd cadd(Cd a, Cd b) { return {a.r + b.r, a.i + b.i}; 
 __device__ __forceinline__ Cd csub2(Cd a, Cd b) { return {a.r - b.r, a.i - b.i}; }
 __device__ __forceinline__ Cd cmulx(Cd a, Cd b) { return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r}; }
 __device__ __forceinline__ Cd cscale(Cd a, double s) { return {a.r * s, a.i * s}; }
-__device__ __forceinline__ Cd cdivx(Cd a, Cd b) {
-    const double d = b.r * b.r + b.i * b.i;
-    return {(a.r * b.r + a.i * b.i) / d, (a.i * b.r - a.r * b.i) / d};
-}
 __device__ __forceinline__ double cabs2(Cd a) { return a.r * a.r + a.i * a.i; }
 
 // Layer speed of a beam (bits 4-7 of its flags hold its layer).
@@ -34,209 +30,205 @@ template <typename R> __device__ __forceinline__ R layer_speed(const ModelDev &M
     return wave ? mp<R>(M.lcs[lay], M.flcs[lay]) : mp<R>(M.lcp[lay], M.flcp[lay]);
 }
 
-// Solve the 6x6 complex system A x = b (partial pivoting); false if singular.
-__device__ bool csolve6_dev(Cd A[6][6], Cd b[6], Cd x[6]) {
-    for (int c = 0; c < 6; c++) {
-        int piv = c;
-        for (int r = c + 1; r < 6; r++)
-            if (cabs2(A[r][c]) > cabs2(A[piv][c])) piv = r;
-        if (cabs2(A[piv][c]) < 1e-300) return false;
-        if (piv != c) {
-            for (int j = 0; j < 6; j++) {
-                const Cd t = A[c][j];
-                A[c][j] = A[piv][j];
-                A[piv][j] = t;
+// Children of an event (w = 0 reflected P, 1 reflected S, 2 transmitted P, 3 transmitted S), FP64.
+struct EventOut {
+    int n;
+    int slot[4], flags[4];
+    double P[4][3];
+    Cd a0[4], a1[4];        // P: a0; S: (a_sv, a_sh) in the child's own frame
+    double gh[4], f22[4];   // the jump of dzQ, dzP: g = gh Ph + (f22 - 1) n
+    double Ph[3];           // the part of P along the interface
+};
+
+// cos and sin of the angle, seen along P, from the S frame of P (reference e1 or e3) to the unit vector nsh normal to P:
+// nsh = sin N_sv + cos N_sh
+__device__ __forceinline__ void frame_angle(const double P[3], double pn, bool r1, const double nsh[3], double &c, double &s) {
+    double v[3];
+    if (r1) {
+        v[0] = 0.0;
+        v[1] = -P[2];
+        v[2] = P[1];
+    } else {
+        v[0] = -P[1];
+        v[1] = P[0];
+        v[2] = 0.0;
+    }
+    const double iv = rsqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+    c = iv * (v[0] * nsh[0] + v[1] * nsh[1] + v[2] * nsh[2]);
+    s = iv / pn *
+        ((v[1] * P[2] - v[2] * P[1]) * nsh[0] + (v[2] * P[0] - v[0] * P[2]) * nsh[1] + (v[0] * P[1] - v[1] * P[0]) * nsh[2]);
+}
+
+// The scattering at an interface with unit normal n (e3 for SHAPE 0) between layer la (incident side) and lb; y holds
+// the incident state.  Polarisations: P along P/|P|; SH along nsh = n x P/|n x P| (common to all waves of the event; e2
+// at normal incidence); SV along nsh x P/|P|.  Displacement and traction on the interface are continuous.
+//
+// In the plane of P and n the six conditions separate.  With p = |P_h|, normal components zeta (P) and eta (S) of every
+// medium, and S amplitudes signed by the wave's direction along n, the pairs (u_h, sigma_nn) and (u_n, sigma_hn) of
+// waves to either side differ only in sign, so that, amplitudes divided by |P| of their wave,
+//   M_a (i + r) = M_b t,  N_a (i - r) = N_b t,  M = [p 1; G -2 mu p] diag(1, eta),  N = [1 -p; 2 mu p G] diag(zeta, 1),
+//   G = rho om^2 - 2 mu p^2,  det = -+ rho om^2,
+// a 2x2 complex system for the transmitted P and SV; SH is a ratio.  About 200 FP64 operations in a short chain where
+// elimination on the 6x6 complex system takes 3,000 in local memory (an event kernel runs few warps, and the FP64 pipe
+// issues one warp instruction in 16 cycles: the chain is what bounds it).
+template <typename R, int SHAPE>
+__device__ __forceinline__ bool interface_event(const ModelDev &M, int fl, const R *y, const double n[3], int lb,
+                                                double rel_min, EventOut &ev) {
+    const int la = (fl >> 4) & 15, cls = fl & FL_CLASS_MASK, wave = cls >= 2;
+    const double sgn = (cls & 1) ? -1.0 : 1.0;
+    const double P[3] = {(double)y[F_P], (double)y[F_P + 1], (double)y[F_P + 2]};
+    const double cin = wave ? M.lcs[la] : M.lcp[la];
+    const double pin = sqrt(P[0] * P[0] + P[1] * P[1] + P[2] * P[2]), om = cin * pin;
+    const double pz = SHAPE == 0 ? P[2] : P[0] * n[0] + P[1] * n[1] + P[2] * n[2];
+#pragma unroll
+    for (int d = 0; d < 3; d++) ev.Ph[d] = SHAPE == 0 ? (d < 2 ? P[d] : 0.0) : P[d] - pz * n[d];
+    const double ph2 = ev.Ph[0] * ev.Ph[0] + ev.Ph[1] * ev.Ph[1] + ev.Ph[2] * ev.Ph[2];
+    double ph = 0.0, nsh[3] = {0.0, 1.0, 0.0};
+    if (ph2 > 0.0) {
+        const double ip = rsqrt(ph2);
+        ph = ph2 * ip;
+        nsh[0] = SHAPE == 0 ? -ip * P[1] : ip * (n[1] * ev.Ph[2] - n[2] * ev.Ph[1]);
+        nsh[1] = SHAPE == 0 ? ip * P[0] : ip * (n[2] * ev.Ph[0] - n[0] * ev.Ph[2]);
+        nsh[2] = SHAPE == 0 ? 0.0 : ip * (n[0] * ev.Ph[1] - n[1] * ev.Ph[0]);
+    } else if (SHAPE != 0) {
+        double Rl[9];
+        frame_from_normal(n, Rl);
+        for (int d = 0; d < 3; d++) nsh[d] = Rl[3 + d];
+    }
+    // incident amplitudes along P/|P|, or along SV and SH of the interface
+    const Cd a0 = {(double)y[F_A0], (double)y[F_A0 + 1]}, a1 = {(double)y[F_A1], (double)y[F_A1 + 1]};
+    double ain2 = cabs2(a0);
+    Cd iP = a0, iS = {0.0, 0.0}, iH = {0.0, 0.0};
+    if (wave) {
+        iP = {0.0, 0.0};
+        iS = a0;
+        iH = a1;
+        ain2 += cabs2(a1);
+        if (SHAPE != 0 || (fl & FL_REF_E1) || !(ph2 > 0.0)) {
+            double c, s;
+            frame_angle(P, pin, (fl & FL_REF_E1) != 0, nsh, c, s);
+            iS = csub2(cscale(a0, c), cscale(a1, s));
+            iH = cadd(cscale(a0, s), cscale(a1, c));
+        }
+    }
+    const double sz = pz >= 0.0 ? 1.0 : -1.0;
+    double kw[4], cw[4], zr[4];   // |P|, speed and |normal component| of the waves
+    bool prop[4];
+    Cd z[4];
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+        const int L = w >= 2 ? lb : la;
+        cw[w] = w & 1 ? M.lcs[L] : M.lcp[L];
+        kw[w] = om / cw[w];
+        const double pz2 = kw[w] * kw[w] - ph2;
+        prop[w] = pz2 >= 0.0;
+        zr[w] = sqrt(fabs(pz2));
+        z[w] = prop[w] ? Cd{zr[w], 0.0} : Cd{0.0, sgn * zr[w]};   // decays away from the interface
+    }
+    const double mua = M.lrho[la] * M.lcs[la] * M.lcs[la], mub = M.lrho[lb] * M.lcs[lb] * M.lcs[lb];
+    const double om2 = om * om, Ga = M.lrho[la] * om2 - 2.0 * mua * ph2, Gb = M.lrho[lb] * om2 - 2.0 * mub * ph2;
+    const double iD = 1.0 / (M.lrho[la] * om2);
+    const double u = (2.0 * mua * ph2 + Gb) * iD, v = (Ga + 2.0 * mub * ph2) * iD, x = 2.0 * ph * (mua - mub) * iD,
+                 wq = ph * (Ga - Gb) * iD;
+    const Cd jP = cscale(iP, 1.0 / kw[0]), jS = cscale(iS, sz / kw[1]);
+    const Cd A11 = cadd(cscale(z[0], u), cscale(z[2], v)), A22 = cadd(cscale(z[3], v), cscale(z[1], u));
+    Cd A12 = cscale(cmulx(z[0], z[3]), x), A21 = cscale(cmulx(z[1], z[2]), -x);
+    A12.r -= wq;
+    A21.r += wq;
+    const Cd det = csub2(cmulx(A11, A22), cmulx(A12, A21));
+    const Cd denH = cadd(cscale(z[1], mua), cscale(z[3], mub));
+    const double d2 = cabs2(det), h2 = cabs2(denH);
+    if (!(d2 > 0.0) || !(h2 > 0.0)) return false;
+    const Cd id = {det.r / d2, -det.i / d2};
+    const Cd b1 = cscale(cmulx(z[0], jP), 2.0), b2 = cscale(cmulx(z[1], jS), 2.0);
+    const Cd tP = cmulx(csub2(cmulx(b1, A22), cmulx(A12, b2)), id), tS = cmulx(csub2(cmulx(A11, b2), cmulx(A21, b1)), id);
+    const Cd rP = csub2(cadd(cscale(tP, u), cscale(cmulx(z[3], tS), x)), jP);
+    const Cd rS = csub2(cadd(jS, cscale(cmulx(z[2], tP), x)), cscale(tS, u));
+    Cd tH = {0.0, 0.0}, rH = {0.0, 0.0};
+    if (wave) {
+        const Cd ih = {denH.r / h2, -denH.i / h2};
+        tH = cmulx(cmulx(cscale(z[1], 2.0 * mua), iH), ih);
+        rH = csub2(tH, iH);
+    }
+    const Cd am[4] = {cscale(rP, kw[0]), cscale(rS, -sz * kw[1]), cscale(tP, kw[2]), cscale(tS, sz * kw[3])};
+    const int gen = (fl >> 8) & 15;
+    const double ipz = 1.0 / pz, icin2 = 1.0 / (cin * cin);
+    int m = 0;
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+        const int sw = w & 1, trans = w >= 2;
+        Cd b0 = am[w], b1c = sw ? (trans ? tH : rH) : Cd{0.0, 0.0};
+        const double amag2 = cabs2(b0) + cabs2(b1c);
+        if (!prop[w] || !(amag2 >= rel_min * rel_min * ain2) || amag2 == 0.0) continue;
+        const double zz = trans ? sz * zr[w] : -sz * zr[w];
+        double Pc[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) Pc[d] = SHAPE == 0 ? (d < 2 ? P[d] : zz) : ev.Ph[d] + zz * n[d];
+        int flc = (sw ? 2 : 0) | (cls & 1) | ((trans ? lb : la) << 4) | ((gen + 1) << 8) | (fl & (3 << FL_ROOT_SHIFT));
+        if (sw) {
+            // SV/SH of the interface -> the child's own frame (e3 unless its P is near vertical)
+            const double h = Pc[0] * Pc[0] + Pc[1] * Pc[1];
+            const bool r1 = h < 0.01 * (h + Pc[2] * Pc[2]);
+            if (r1) flc |= FL_REF_E1;
+            if (SHAPE != 0 || r1) {
+                double c, s;
+                frame_angle(Pc, kw[w], r1, nsh, c, s);
+                const Cd t0 = b0, t1 = b1c;
+                b0 = cadd(cscale(t0, c), cscale(t1, s));
+                b1c = csub2(cscale(t1, c), cscale(t0, s));
             }
-            const Cd t = b[c];
-            b[c] = b[piv];
-            b[piv] = t;
         }
-        for (int r = c + 1; r < 6; r++) {
-            const Cd f = cdivx(A[r][c], A[c][c]);
-            for (int j = c; j < 6; j++) A[r][j] = csub2(A[r][j], cmulx(f, A[c][j]));
-            b[r] = csub2(b[r], cmulx(f, b[c]));
-        }
+        ev.slot[m] = w;
+        ev.flags[m] = flc;
+        ev.a0[m] = b0;
+        ev.a1[m] = b1c;
+        const double kappa = cw[w] * cw[w] * icin2;
+        ev.gh[m] = (kappa - 1.0) * ipz;
+        ev.f22[m] = kappa * zz * ipz;
+#pragma unroll
+        for (int d = 0; d < 3; d++) ev.P[m][d] = Pc[d];
+        m++;
     }
-    for (int r = 5; r >= 0; r--) {
-        Cd s = b[r];
-        for (int j = r + 1; j < 6; j++) s = csub2(s, cmulx(A[r][j], x[j]));
-        x[r] = cdivx(s, A[r][r]);
-    }
+    ev.n = m;
     return true;
 }
 
-// Child i of the event (0 reflected P, 1 reflected S, 2 transmitted P, 3 transmitted S), FP64.
-struct EventOut {
-    int n;
-    int slot[4];
-    double P[4][3];
-    Cd a0[4], a1[4];  // P: a0; S: (a_sv, a_sh) in the child's own frame
-    int flags[4];
-    double kappa[4];
-};
-
-// The scattering at an interface between layer la (incident side) and lb.  y holds the incident
-// state (its Q on the interface).  Polarisations: P along P/|P|; SH along nsh = e3 x P/|e3 x P|
-// (common to all waves of the event; e2 at normal incidence); SV along nsh x P/|P|.  Unknown
-// amplitudes (rP, rSV, rSH, tP, tSV, tSH) make displacement and traction sigma.e3 continuous.
-template <typename R>
-__device__ __noinline__ void interface_event(const ModelDev &M, int fl, const R *y, int lb, double rel_min,
-                                             EventOut &ev) {
-    const int la = (fl >> 4) & 15, cls = fl & FL_CLASS_MASK, wave = cls >= 2;
-    const double sgn = (cls & 1) ? -1.0 : 1.0;
-    const double P0 = (double)y[F_P], P1 = (double)y[F_P + 1], P2 = (double)y[F_P + 2];
-    const double cin = wave ? M.lcs[la] : M.lcp[la];
-    const double pin = sqrt(P0 * P0 + P1 * P1 + P2 * P2), om = cin * pin;
-    const double ph2 = P0 * P0 + P1 * P1;
-    double nsh[3] = {0.0, 1.0, 0.0};
-    if (ph2 > 0.0) {
-        const double phn = sqrt(ph2);
-        nsh[0] = -P1 / phn;
-        nsh[1] = P0 / phn;
-    }
-    // incident displacement
-    Cd U[3];
-    {
-        const double Ph[3] = {P0 / pin, P1 / pin, P2 / pin};
-        const Cd a0 = {(double)y[F_A0], (double)y[F_A0 + 1]};
-        if (!wave) {
-            for (int d = 0; d < 3; d++) U[d] = cscale(a0, Ph[d]);
-        } else {
-            const Cd a1 = {(double)y[F_A1], (double)y[F_A1 + 1]};
-            double Pd[3] = {P0, P1, P2}, Nsv[3], Nsh[3];
-            s_frame<double>(Pd, (fl & FL_REF_E1) != 0, Nsv, Nsh);
-            for (int d = 0; d < 3; d++) U[d] = cadd(cscale(a0, Nsv[d]), cscale(a1, Nsh[d]));
-        }
-    }
-    const double lam[2] = {M.lrho[la] * (M.lcp[la] * M.lcp[la] - 2.0 * M.lcs[la] * M.lcs[la]),
-                           M.lrho[lb] * (M.lcp[lb] * M.lcp[lb] - 2.0 * M.lcs[lb] * M.lcs[lb])};
-    const double mu[2] = {M.lrho[la] * M.lcs[la] * M.lcs[la], M.lrho[lb] * M.lcs[lb] * M.lcs[lb]};
-    auto traction = [&](int side, const Cd P[3], const Cd N[3], Cd T[3]) {
-        const Cd pn = cadd(cadd(cmulx(P[0], N[0]), cmulx(P[1], N[1])), cmulx(P[2], N[2]));
-        for (int i = 0; i < 3; i++) T[i] = cscale(cadd(cmulx(P[i], N[2]), cmulx(P[2], N[i])), mu[side]);
-        T[2] = cadd(T[2], cscale(pn, lam[side]));
-    };
-    Cd Tin[3];
-    {
-        const Cd Pc[3] = {{P0, 0.0}, {P1, 0.0}, {P2, 0.0}};
-        traction(0, Pc, U, Tin);
-    }
-    const double sz = P2 >= 0.0 ? 1.0 : -1.0;
-    Cd Pw[4][3];
-    double pnw[4], cw[4];
-    bool prop[4];
-    for (int w = 0; w < 4; w++) {
-        const int trans = w >= 2, sw = w & 1, L = trans ? lb : la;
-        cw[w] = sw ? M.lcs[L] : M.lcp[L];
-        pnw[w] = om / cw[w];
-        const double pz2 = pnw[w] * pnw[w] - ph2, side = trans ? sz : -sz;
-        Pw[w][0] = {P0, 0.0};
-        Pw[w][1] = {P1, 0.0};
-        if (pz2 >= 0.0) {
-            Pw[w][2] = {side * sqrt(pz2), 0.0};
-            prop[w] = true;
-        } else {
-            Pw[w][2] = {0.0, sgn * side * sqrt(-pz2)};  // decays away from the interface
-            prop[w] = false;
-        }
-    }
-    auto pol = [&](int w, int which, Cd N[3]) {
-        if (which == 0) {
-            for (int d = 0; d < 3; d++) N[d] = cscale(Pw[w][d], 1.0 / pnw[w]);
-        } else if (which == 2) {
-            for (int d = 0; d < 3; d++) N[d] = {nsh[d], 0.0};
-        } else {
-            const double ip = 1.0 / pnw[w];
-            N[0] = cscale(csub2(cscale(Pw[w][2], nsh[1]), cscale(Pw[w][1], nsh[2])), ip);
-            N[1] = cscale(csub2(cscale(Pw[w][0], nsh[2]), cscale(Pw[w][2], nsh[0])), ip);
-            N[2] = cscale(csub2(cscale(Pw[w][1], nsh[0]), cscale(Pw[w][0], nsh[1])), ip);
-        }
-    };
-    Cd A[6][6], b[6], x[6];
-    const int wv[6] = {0, 1, 1, 2, 3, 3}, pl[6] = {0, 1, 2, 0, 1, 2};
-    for (int u = 0; u < 6; u++) {
-        const int w = wv[u], trans = w >= 2;
-        Cd N[3], T[3];
-        pol(w, pl[u], N);
-        traction(trans, Pw[w], N, T);
-        const double s = trans ? -1.0 : 1.0;
-        for (int d = 0; d < 3; d++) {
-            A[d][u] = cscale(N[d], s);
-            A[3 + d][u] = cscale(T[d], s);
-        }
-    }
-    for (int d = 0; d < 3; d++) {
-        b[d] = cscale(U[d], -1.0);
-        b[3 + d] = cscale(Tin[d], -1.0);
-    }
-    ev.n = 0;
-    if (!csolve6_dev(A, b, x)) return;
-    const double ain = sqrt(cabs2(U[0]) + cabs2(U[1]) + cabs2(U[2]));
-    const int gen = (fl >> 8) & 15;
-    for (int w = 0; w < 4; w++) {
-        if (!prop[w]) continue;
-        const int sw = w & 1, trans = w >= 2;
-        const Cd a0 = sw ? x[w == 1 ? 1 : 4] : x[w == 0 ? 0 : 3];
-        const Cd a1 = sw ? x[w == 1 ? 2 : 5] : Cd{0.0, 0.0};
-        const double amag = sqrt(cabs2(a0) + cabs2(a1));
-        if (!(amag >= rel_min * ain) || amag == 0.0) continue;
-        const int k = ev.n++;
-        ev.slot[k] = w;
-        for (int d = 0; d < 3; d++) ev.P[k][d] = Pw[w][d].r;
-        ev.kappa[k] = (cw[w] / cin) * (cw[w] / cin);
-        int cc = (sw ? 2 : 0) | (cls & 1);
-        int flc = cc | ((trans ? lb : la) << 4) | ((gen + 1) << 8) | (fl & (3 << FL_ROOT_SHIFT));
-        if (!sw) {
-            ev.a0[k] = a0;
-            ev.a1[k] = {0.0, 0.0};
-        } else {
-            // global SV/SH vectors -> the child's own frame (e3 unless its P is near vertical)
-            Cd Nsv[3];
-            pol(w, 1, Nsv);
-            Cd Ag[3];
-            for (int d = 0; d < 3; d++) Ag[d] = cadd(cmulx(a0, Nsv[d]), cscale(a1, nsh[d]));
-            double Pc[3] = {ev.P[k][0], ev.P[k][1], ev.P[k][2]};
-            const bool r1 = (Pc[0] * Pc[0] + Pc[1] * Pc[1]) < 0.01 * (Pc[0] * Pc[0] + Pc[1] * Pc[1] + Pc[2] * Pc[2]);
-            if (r1) flc |= FL_REF_E1;
-            double fsv[3], fsh[3];
-            s_frame<double>(Pc, r1, fsv, fsh);
-            Cd s0 = {0.0, 0.0}, s1 = {0.0, 0.0};
-            for (int d = 0; d < 3; d++) {
-                s0 = cadd(s0, cscale(Ag[d], fsv[d]));
-                s1 = cadd(s1, cscale(Ag[d], fsh[d]));
-            }
-            ev.a0[k] = s0;
-            ev.a1[k] = s1;
-        }
-        ev.flags[k] = flc;
-    }
-}
-
-// Write child k of the event into out[] (NF reals): Q at the crossing, new P, dzQ F, dzP F^{-T},
-// amplitudes.
-template <typename R>
-__device__ void make_child(const R *yc, const EventOut &ev, int k, R *out) {
+// Child k of the event into out[] (NF reals): Q at the crossing, new P, dzQ F, dzP F^{-T}, amplitudes.  F is I but
+// for its row along the normal, so in any frame dzQ' = dzQ + (dzQ n) g^T and dzP' = dzP - (dzP g) n^T / f22.
+template <typename R, int SHAPE>
+__device__ __forceinline__ void make_child(const R *yc, const EventOut &ev, const double n[3], int k, R *out) {
 #pragma unroll
-    for (int f = 0; f < NF; f++) out[f] = yc[f];
-    const double pz_in = (double)yc[F_P + 2];
-    const double f20 = (ev.kappa[k] - 1.0) * (double)yc[F_P] / pz_in;
-    const double f21 = (ev.kappa[k] - 1.0) * (double)yc[F_P + 1] / pz_in;
-    const double f22 = ev.kappa[k] * ev.P[k][2] / pz_in;
-    // F = I except the last row (f20, f21, f22); F^{-T} = I except the last column (-f20/f22, -f21/f22, 1/f22)
+    for (int d = 0; d < 3; d++) out[F_Q + d] = yc[F_Q + d];
+    const double gh = ev.gh[k], f22 = ev.f22[k], if22 = 1.0 / f22;
+    const double g0 = gh * ev.Ph[0] + (SHAPE == 0 ? 0.0 : (f22 - 1.0) * n[0]),
+                 g1 = gh * ev.Ph[1] + (SHAPE == 0 ? 0.0 : (f22 - 1.0) * n[1]),
+                 g2 = SHAPE == 0 ? 0.0 : gh * ev.Ph[2] + (f22 - 1.0) * n[2];
+#pragma unroll
     for (int m = 0; m < 3; m++) {
+#pragma unroll
         for (int c = 0; c < 2; c++) {  // re, im
-            const double q0 = yc[F_DQ + 2 * (3 * m) + c], q1 = yc[F_DQ + 2 * (3 * m + 1) + c],
-                         q2 = yc[F_DQ + 2 * (3 * m + 2) + c];
-            out[F_DQ + 2 * (3 * m) + c] = (R)(q0 + q2 * f20);
-            out[F_DQ + 2 * (3 * m + 1) + c] = (R)(q1 + q2 * f21);
-            out[F_DQ + 2 * (3 * m + 2) + c] = (R)(q2 * f22);
-            const double p0 = yc[F_DP + 2 * (3 * m) + c], p1 = yc[F_DP + 2 * (3 * m + 1) + c],
-                         p2 = yc[F_DP + 2 * (3 * m + 2) + c];
-            out[F_DP + 2 * (3 * m) + c] = (R)p0;
-            out[F_DP + 2 * (3 * m + 1) + c] = (R)p1;
-            out[F_DP + 2 * (3 * m + 2) + c] = (R)((p2 - p0 * f20 - p1 * f21) / f22);
+            const int e0 = 2 * (3 * m) + c, e1 = e0 + 2, e2 = e0 + 4;
+            const double q0 = yc[F_DQ + e0], q1 = yc[F_DQ + e1], q2 = yc[F_DQ + e2];
+            const double p0 = yc[F_DP + e0], p1 = yc[F_DP + e1], p2 = yc[F_DP + e2];
+            if (SHAPE == 0) {
+                out[F_DQ + e0] = (R)(q0 + q2 * g0);
+                out[F_DQ + e1] = (R)(q1 + q2 * g1);
+                out[F_DQ + e2] = (R)(q2 * f22);
+                out[F_DP + e0] = yc[F_DP + e0];
+                out[F_DP + e1] = yc[F_DP + e1];
+                out[F_DP + e2] = (R)((p2 - p0 * g0 - p1 * g1) * if22);
+            } else {
+                const double qn = q0 * n[0] + q1 * n[1] + q2 * n[2], pg = -if22 * (p0 * g0 + p1 * g1 + p2 * g2);
+                out[F_DQ + e0] = (R)(q0 + qn * g0);
+                out[F_DQ + e1] = (R)(q1 + qn * g1);
+                out[F_DQ + e2] = (R)(q2 + qn * g2);
+                out[F_DP + e0] = (R)(p0 + pg * n[0]);
+                out[F_DP + e1] = (R)(p1 + pg * n[1]);
+                out[F_DP + e2] = (R)(p2 + pg * n[2]);
+            }
         }
     }
+#pragma unroll
     for (int d = 0; d < 3; d++) out[F_P + d] = (R)ev.P[k][d];
     out[F_A0] = (R)ev.a0[k].r;
     out[F_A0 + 1] = (R)ev.a0[k].i;
@@ -319,15 +311,14 @@ __device__ __forceinline__ bool shell_clear(const ModelDev &M, int L, const floa
 __device__ __forceinline__ bool shell_clear(const ModelDev &, int, const double *, const double *) { return false; }
 
 // Undulating layers: height of interface i above (x1, x2), and its slopes dh/dx1, dh/dx2.
-__device__ __forceinline__ double surf_h(const ModelDev &M, int i, double x1, double x2) {
-    return M.zif[i] + M.uamp[i] * cos(M.uk[0] * x1) * cos(M.uk[1] * x2);
-}
-__device__ __forceinline__ void surf_grad(const ModelDev &M, int i, double x1, double x2, double &h1, double &h2) {
+__device__ __forceinline__ double surf_cos(const ModelDev &M, const double *q) { return cos(M.uk[0] * q[0]) * cos(M.uk[1] * q[1]); }
+__device__ __forceinline__ double surf_at(const ModelDev &M, int i, double x1, double x2, double &h1, double &h2) {
     double s1, c1, s2, c2;
     sincos(M.uk[0] * x1, &s1, &c1);
     sincos(M.uk[1] * x2, &s2, &c2);
     h1 = -M.uamp[i] * M.uk[0] * s1 * c2;
     h2 = -M.uamp[i] * M.uk[1] * c1 * s2;
+    return M.zif[i] + M.uamp[i] * (c1 * c2);
 }
 
 // FP32 screen for undulating layers: true when the end point q1 lies clearly between the interfaces that
@@ -351,6 +342,19 @@ __device__ __forceinline__ bool surf_clear(const ModelDev &M, int L, const float
 }
 __device__ __forceinline__ bool surf_clear(const ModelDev &, int, const double *) { return false; }
 
+// The step's end point q1 on or below the lower interface of layer L, or above the upper one: a crossing.
+__device__ __forceinline__ bool surf_met(const ModelDev &M, int L, bool down, const double q1[3], double cc1, double &g1) {
+    const int i = down ? L : L - 1;
+    if (i < 0 || i > M.nlay - 2) return false;
+    g1 = q1[2] - (M.zif[i] + M.uamp[i] * cc1);
+    return down ? g1 >= 0.0 : g1 < 0.0;
+}
+__device__ __noinline__ bool surf_crosses(const ModelDev &M, int L, const double q1[3]) {
+    const double cc1 = surf_cos(M, q1);
+    double g;
+    return surf_met(M, L, true, q1, cc1, g) || surf_met(M, L, false, q1, cc1, g);
+}
+
 // Undulating layers: the first crossing of the straight path q0 -> q1 of one step with an interface that
 // bounds layer L.  An end point on or below the lower interface (above the upper one) means a crossing;
 // g(th) = x3(th) - h(x1(th), x2(th)) then changes sign on [0, 1] and its root is found by Newton's method
@@ -361,20 +365,21 @@ __device__ __forceinline__ bool surf_clear(const ModelDev &, int, const double *
 __device__ __noinline__ bool surf_crossing(const ModelDev &M, int L, const double q0[3], const double q1[3], double &th, int &lb,
                               int &iface) {
     const double d[3] = {q1[0] - q0[0], q1[1] - q0[1], q1[2] - q0[2]};
+    const double cc0 = surf_cos(M, q0), cc1 = surf_cos(M, q1);
     bool hit = false;
     for (int side = 0; side < 2; side++) {
         const bool down = side == 0;
+        double g1;
+        if (!surf_met(M, L, down, q1, cc1, g1)) continue;
         const int i = down ? L : L - 1;
-        if (i < 0 || i > M.nlay - 2) continue;
-        const double g0 = q0[2] - surf_h(M, i, q0[0], q0[1]), g1 = q1[2] - surf_h(M, i, q1[0], q1[1]);
-        if (down ? !(g1 >= 0.0) : !(g1 < 0.0)) continue;
+        const double g0 = q0[2] - (M.zif[i] + M.uamp[i] * cc0);
         double t;
         if ((g0 < 0.0) == down) {
             double lo = 0.0, hi = 1.0, glo = g0;   // g(lo) and g(hi) of opposite signs
             t = g0 / (g0 - g1);
             for (int it = 0; it < 100 && hi - lo > 1e-15; it++) {
-                const double x1 = q0[0] + t * d[0], x2 = q0[1] + t * d[1];
-                const double g = q0[2] + t * d[2] - surf_h(M, i, x1, x2);
+                double h1, h2;
+                const double g = q0[2] + t * d[2] - surf_at(M, i, q0[0] + t * d[0], q0[1] + t * d[1], h1, h2);
                 if (g == 0.0) break;
                 if ((g < 0.0) == (glo < 0.0)) {
                     lo = t;
@@ -382,8 +387,6 @@ __device__ __noinline__ bool surf_crossing(const ModelDev &M, int L, const doubl
                 } else {
                     hi = t;
                 }
-                double h1, h2;
-                surf_grad(M, i, x1, x2, h1, h2);
                 const double dg = d[2] - h1 * d[0] - h2 * d[1];
                 double tn = dg != 0.0 ? t - g / dg : 0.5 * (lo + hi);
                 if (!(tn > lo && tn < hi)) tn = 0.5 * (lo + hi);
@@ -443,12 +446,12 @@ template <typename R> struct Planes {
 
 // Does the step q0 -> q1 (compensations c0, c1) meet an interface of layer L?  Planes: the end point.  Curved
 // layers: FP32 steps that stay clear of the interfaces by a margin far above the rounding of the screen are
-// decided by the screen, the rest by the exact FP64 test, which also gives the crossing.
+// decided by the screen, the rest by the exact FP64 test, which with WHERE also gives the crossing.
 struct Crossing {
     double th, rho;
     int lb, iface;
 };
-template <typename R, int SHAPE>
+template <typename R, int SHAPE, bool WHERE>
 __device__ __forceinline__ bool step_crosses(const ModelDev &M, int L, const Planes<R> &pl, const R *q0, const R *c0,
                                              const R *q1, const R *c1, Crossing &x) {
     if (SHAPE == 0) return q1[2] < pl.top || q1[2] >= pl.bot;
@@ -459,7 +462,8 @@ __device__ __forceinline__ bool step_crosses(const ModelDev &M, int L, const Pla
         a[d] = (double)q0[d] - (double)c0[d];
         b[d] = (double)q1[d] - (double)c1[d];
     }
-    return SHAPE == 1 ? shell_crossing(M, L, a, b, x.th, x.lb, x.rho) : surf_crossing(M, L, a, b, x.th, x.lb, x.iface);
+    if (SHAPE == 1) return shell_crossing(M, L, a, b, x.th, x.lb, x.rho);
+    return WHERE ? surf_crossing(M, L, a, b, x.th, x.lb, x.iface) : surf_crosses(M, L, b);
 }
 
 // Steps s .. nsteps-1 of a beam up to the first one that meets an interface; returns that step's index (nsteps
@@ -482,7 +486,7 @@ __device__ __forceinline__ int layered_run(const ModelDev &M, int fl, R *y, R *q
             R q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
             straight_q<R>(S, dt, q, qn);
             Crossing x;
-            if (!force_first && step_crosses<R, SHAPE>(M, L, pl, y + F_Q, qc, q, qn, x)) {
+            if (!force_first && step_crosses<R, SHAPE, false>(M, L, pl, y + F_Q, qc, q, qn, x)) {
                 open = false;
                 break;
             }
@@ -527,8 +531,8 @@ __device__ __forceinline__ void push_event(int2 *__restrict__ list, unsigned *__
 // meets an interface; such beams are listed with their step (or die, past their last allowed interface).
 // One state stream per group instead of one per step: 49 reals read and 28 written per beam (P and dzP stay),
 // which bounds it.  442 k beams growing to 0.9 M, 300 steps in groups of 5, FP32: 69.6 ms (a launch per step
-// with four right-hand sides, events inside) -> 3.8 ms of these kernels and 8.7 ms of event kernels; with
-// undulating interfaces 187 -> 15.6 and 22.1 ms.
+// with four right-hand sides, events inside) -> 3.8 ms of these kernels and 4.1 ms of event kernels; with
+// undulating interfaces (an FP64 test of the end point where the FP32 screen cannot decide) 187 -> 5.5 and 9.9 ms.
 template <typename R, int SHAPE>
 __global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
                                                          int64_t cap, const unsigned long long *__restrict__ counts,
@@ -558,14 +562,15 @@ __global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restr
 
 // The listed beams: the event of step s at its interface, then every child finishes that step and advances
 // like the beams of layered_run_kernel; children that meet another interface go to the next list.  A thread
-// per event: an event costs thousands of FP64 operations, and a kernel of its own keeps whole warps on them
-// (inside the step kernel one lane of a warp held the other 31).
+// per event, in a kernel of its own so that whole warps are on events (inside the step kernel one lane of a warp held
+// the other 31).  A few thousand events a launch are one or two warps per SM: the length of an event's FP64 chain
+// bounds it.  With the 6x6 system of an event eliminated in general and the state rotated to the interface's frame and
+// back for every child these kernels took 8.7 ms (flat) and 22.1 ms (undulating) where they now take 4.1 and 9.9.
 //
 // In curved layers (SHAPE 1: spheres, SHAPE 2: undulating interfaces) the crossing is put on the interface in
 // FP64 (radially onto the sphere, vertically onto the undulating surface; its FP32 rounding goes to the Q
-// compensation), the beam is rotated into the local frame whose third axis is the interface's normal there, the
-// flat-interface event runs in that frame (Sec. 3.1: the tangent plane stands in for the interface), and every
-// child is rotated back.
+// compensation) and the event runs with the interface's normal there (Sec. 3.1: the tangent plane stands in for the
+// interface), in global coordinates.
 template <typename R, int SHAPE>
 __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
                                                           int32_t *__restrict__ ids, long long *__restrict__ path,
@@ -591,7 +596,7 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
             Straight<R> S;
             straight_setup<R>(sg, c, y, B, S);
             straight_q<R>(S, dt, q, qn);
-            hit = step_crosses<R, SHAPE>(M, L, pl, y + F_Q, qc, q, qn, x);
+            hit = step_crosses<R, SHAPE, true>(M, L, pl, y + F_Q, qc, q, qn, x);
             if (hit) {
                 if (SHAPE == 0) {
                     const bool down = q[2] >= pl.bot;
@@ -613,13 +618,12 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
             continue;
         }
         straight_step<R>(sg, c, y, (R)x.th * dt, qc);
-        double Rl[9];
-        int fll = fl;
+        double nrm[3] = {0.0, 0.0, 1.0};
         if (SHAPE == 0) {
             y[F_Q + 2] = x.lb > L ? pl.bot : pl.top;
             qc[2] = R(0);                 // the interface depth is exact
         } else {
-            double p[3], nrm[3];
+            double p[3];
             for (int d = 0; d < 3; d++) p[d] = (double)y[F_Q + d] - (double)qc[d];
             if (SHAPE == 1) {
                 double r[3], rn = 0.0;
@@ -633,24 +637,19 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
                     p[d] = M.ctr[d] + x.rho * nrm[d];
                 }
             } else {
-                p[2] = surf_h(M, x.iface, p[0], p[1]);
                 double h1, h2;
-                surf_grad(M, x.iface, p[0], p[1], h1, h2);
-                const double nn = sqrt(1.0 + h1 * h1 + h2 * h2);
-                nrm[0] = -h1 / nn;
-                nrm[1] = -h2 / nn;
-                nrm[2] = 1.0 / nn;
+                p[2] = surf_at(M, x.iface, p[0], p[1], h1, h2);
+                nrm[2] = rsqrt(1.0 + h1 * h1 + h2 * h2);
+                nrm[0] = -h1 * nrm[2];
+                nrm[1] = -h2 * nrm[2];
             }
             for (int d = 0; d < 3; d++) {
                 y[F_Q + d] = (R)p[d];
                 qc[d] = (R)((double)y[F_Q + d] - p[d]);
             }
-            frame_from_normal(nrm, Rl);
-            rotate_state<R>(Rl, false, false, y, fll);   // Q stays global: the event does not read it
         }
         EventOut ev;
-        interface_event<R>(M, fll, y, x.lb, rel_min, ev);
-        if (ev.n == 0) {
+        if (!interface_event<R, SHAPE>(M, fl, y, nrm, x.lb, rel_min, ev) || ev.n == 0) {
             flags[b] = fl | FL_DEAD;
             continue;
         }
@@ -658,9 +657,8 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
         const int32_t id = ids[b];
         for (int k = 0; k < ev.n; k++) {
             R ch[NF], qch[3] = {qc[0], qc[1], qc[2]};
-            make_child<R>(y, ev, k, ch);
+            make_child<R, SHAPE>(y, ev, nrm, k, ch);
             int flc = ev.flags[k];
-            if (SHAPE != 0) rotate_state<R>(Rl, true, false, ch, flc);
             straight_step<R>((flc & 1) ? R(-1) : R(1), layer_speed<R>(M, (flc & FL_CLASS_MASK) >= 2, (flc >> 4) & 15), ch,
                              SHAPE == 0 ? (R(1) - (R)x.th) * dt : R(1.0 - x.th) * dt, qch);
             int sc = nsteps;
