@@ -390,11 +390,9 @@ __device__ __noinline__ bool surf_crossing(const ModelDev &M, int L, const doubl
                 const double dg = d[2] - h1 * d[0] - h2 * d[1];
                 double tn = dg != 0.0 ? t - g / dg : 0.5 * (lo + hi);
                 if (!(tn > lo && tn < hi)) tn = 0.5 * (lo + hi);
-                if (fabs(tn - t) < 1e-16) {
-                    t = tn;
-                    break;
-                }
+                const double step = fabs(tn - t);
                 t = tn;
+                if (step < 1e-12) break;   // the next correction is of the order of its square
             }
         } else {
             t = g0 != g1 ? g0 / (g0 - g1) : 0.0;   // no motion across the surface: the start itself
@@ -466,42 +464,58 @@ __device__ __forceinline__ bool step_crosses(const ModelDev &M, int L, const Pla
     return WHERE ? surf_crossing(M, L, a, b, x.th, x.lb, x.iface) : surf_crosses(M, L, b);
 }
 
+// At most m steps of a beam from its expansion S, the first at time t0 of it: Q, its compensation and the amplitudes
+// in y, qc (dzQ is left to the caller).  Returns the steps made; open: no interface was met.
+template <typename R, int SHAPE>
+__device__ __forceinline__ int straight_run(const ModelDev &M, int L, const Planes<R> &pl, const Straight<R> &S, R t0, R *y,
+                                            R *qc, R dt, int m, bool force_first, bool &open) {
+    C2<R> g1 = straight_gamma<R>(S, t0);
+    int i = 0;
+    for (; i < m; i++) {
+        R q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
+        straight_q<R>(S, dt, q, qn);
+        Crossing x;
+        if (!force_first && step_crosses<R, SHAPE, false>(M, L, pl, y + F_Q, qc, q, qn, x)) {
+            open = false;
+            break;
+        }
+        force_first = false;
+        const R t = t0 + R(i) * dt;
+        const C2<R> g2 = straight_gamma<R>(S, t + R(0.5) * dt), g4 = straight_gamma<R>(S, t + dt);
+        straight_amplitudes<R>(y, straight_gain<R>(dt, g1, g2, g4));
+        g1 = g4;
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            y[F_Q + d] = q[d];
+            qc[d] = qn[d];
+        }
+    }
+    return i;
+}
+
 // Steps s .. nsteps-1 of a beam up to the first one that meets an interface; returns that step's index (nsteps
 // without one), the state at its start in y, qc.  Every step but that one is the closed form of straight.cuh.
+// lead > 0: a part of a step of that length comes first (a child's way from its interface to the step's end).
 template <typename R, int SHAPE>
 __device__ __forceinline__ int layered_run(const ModelDev &M, int fl, R *y, R *qc, R dt, int s, int nsteps,
-                                           bool force_first) {
+                                           bool force_first, bool part = false, R lead = R(0)) {
     const int wave = (fl & FL_CLASS_MASK) >= 2, L = (fl >> 4) & 15;
     const R sg = (fl & 1) ? R(-1) : R(1), c = layer_speed<R>(M, wave, L);
     const Planes<R> pl(M, L);
     bool open = true;
-    while (open && s < nsteps) {
+    while (open && (part || s < nsteps)) {
         R B[18];
         Straight<R> S;
         straight_setup<R>(sg, c, y, B, S);
-        const int m = min(STRAIGHT_RENEW, nsteps - s);
-        C2<R> g1 = straight_gamma<R>(S, R(0));
-        int i = 0;
-        for (; i < m; i++) {
-            R q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
-            straight_q<R>(S, dt, q, qn);
-            Crossing x;
-            if (!force_first && step_crosses<R, SHAPE, false>(M, L, pl, y + F_Q, qc, q, qn, x)) {
-                open = false;
-                break;
-            }
-            force_first = false;
-            const R t = R(i) * dt;
-            const C2<R> g2 = straight_gamma<R>(S, t + R(0.5) * dt), g4 = straight_gamma<R>(S, t + dt);
-            straight_amplitudes<R>(y, straight_gain<R>(dt, g1, g2, g4));
-            g1 = g4;
-#pragma unroll
-            for (int d = 0; d < 3; d++) {
-                y[F_Q + d] = q[d];
-                qc[d] = qn[d];
-            }
+        R t0 = R(0);
+        if (part) {
+            straight_part<R>(S, lead, y, qc);
+            t0 = lead;
+            part = false;
         }
-        const R T = R(i) * dt;
+        const int i = straight_run<R, SHAPE>(M, L, pl, S, t0, y, qc, dt, min(STRAIGHT_RENEW, nsteps - s), force_first, open);
+        force_first = false;
+        const R T = t0 + R(i) * dt;
 #pragma unroll
         for (int f = 0; f < 18; f++) y[F_DQ + f] += T * B[f];
         s += i;
@@ -531,8 +545,8 @@ __device__ __forceinline__ void push_event(int2 *__restrict__ list, unsigned *__
 // meets an interface; such beams are listed with their step (or die, past their last allowed interface).
 // One state stream per group instead of one per step: 49 reals read and 28 written per beam (P and dzP stay),
 // which bounds it.  442 k beams growing to 0.9 M, 300 steps in groups of 5, FP32: 69.6 ms (a launch per step
-// with four right-hand sides, events inside) -> 3.8 ms of these kernels and 4.1 ms of event kernels; with
-// undulating interfaces (an FP64 test of the end point where the FP32 screen cannot decide) 187 -> 5.5 and 9.9 ms.
+// with four right-hand sides, events inside) -> 3.8 ms of these kernels and 3.8 ms of event kernels; with
+// undulating interfaces (an FP64 test of the end point where the FP32 screen cannot decide) 187 -> 5.5 and 7.9 ms.
 template <typename R, int SHAPE>
 __global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
                                                          int64_t cap, const unsigned long long *__restrict__ counts,
@@ -565,7 +579,7 @@ __global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restr
 // per event, in a kernel of its own so that whole warps are on events (inside the step kernel one lane of a warp held
 // the other 31).  A few thousand events a launch are one or two warps per SM: the length of an event's FP64 chain
 // bounds it.  With the 6x6 system of an event eliminated in general and the state rotated to the interface's frame and
-// back for every child these kernels took 8.7 ms (flat) and 22.1 ms (undulating) where they now take 4.1 and 9.9.
+// back for every child these kernels took 8.7 ms (flat) and 22.1 ms (undulating) where they now take 3.8 and 7.9.
 //
 // In curved layers (SHAPE 1: spheres, SHAPE 2: undulating interfaces) the crossing is put on the interface in
 // FP64 (radially onto the sphere, vertically onto the undulating surface; its FP32 rounding goes to the Q
@@ -590,10 +604,11 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
         load_beam<R>(st, cap, b, y, qc);
         Crossing x{0.0, 0.0, L, 0};
         bool hit = false;
+        R B[18];
+        Straight<R> S;
         while (s < nsteps) {
             // the step's end point as layered_run forms it
-            R B[18], q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
-            Straight<R> S;
+            R q[3] = {y[F_Q], y[F_Q + 1], y[F_Q + 2]}, qn[3] = {qc[0], qc[1], qc[2]};
             straight_setup<R>(sg, c, y, B, S);
             straight_q<R>(S, dt, q, qn);
             hit = step_crosses<R, SHAPE, true>(M, L, pl, y + F_Q, qc, q, qn, x);
@@ -617,7 +632,10 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
             for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
             continue;
         }
-        straight_step<R>(sg, c, y, (R)x.th * dt, qc);
+        const R head = (R)x.th * dt;
+        straight_part<R>(S, head, y, qc);
+#pragma unroll
+        for (int f = 0; f < 18; f++) y[F_DQ + f] += head * B[f];
         double nrm[3] = {0.0, 0.0, 1.0};
         if (SHAPE == 0) {
             y[F_Q + 2] = x.lb > L ? pl.bot : pl.top;
@@ -659,10 +677,9 @@ __global__ void __launch_bounds__(64) layered_event_kernel(ModelDev M, R *__rest
             R ch[NF], qch[3] = {qc[0], qc[1], qc[2]};
             make_child<R, SHAPE>(y, ev, nrm, k, ch);
             int flc = ev.flags[k];
-            straight_step<R>((flc & 1) ? R(-1) : R(1), layer_speed<R>(M, (flc & FL_CLASS_MASK) >= 2, (flc >> 4) & 15), ch,
-                             SHAPE == 0 ? (R(1) - (R)x.th) * dt : R(1.0 - x.th) * dt, qch);
-            int sc = nsteps;
-            if (!(flc & FL_DEAD)) sc = layered_run<R, SHAPE>(M, flc, ch, qch, dt, s + 1, nsteps, false);
+            // the rest of the step, and the steps that follow
+            const int sc = layered_run<R, SHAPE>(M, flc, ch, qch, dt, s + 1, nsteps, false, true,
+                                                 SHAPE == 0 ? (R(1) - (R)x.th) * dt : R(1.0 - x.th) * dt);
             const bool again = sc < nsteps;
             if (again && ((flc >> 8) & 15) >= gmax) flc |= FL_DEAD;
             const int64_t dst = store_child<R>(st, flags, ids, path, cap, counts, b, k, ch, qch, flc, id, pp, ev.slot[k]);

@@ -117,16 +117,11 @@ template <typename R> __device__ __forceinline__ void straight_q(const Straight<
     for (int d = 0; d < 3; d++) kahan_add<R>(q[d], qc[d], h * S.v[d]);
 }
 
-// one whole step of size h in place (compensation qc carried)
-template <typename R> __device__ __forceinline__ void straight_step(R sg, R c, R *y, R h, R *qc) {
-    R B[18];
-    Straight<R> S;
-    straight_setup<R>(sg, c, y, B, S);
+// Q and the amplitudes over a step h from the expansion's start (dzQ += h B is the caller's)
+template <typename R> __device__ __forceinline__ void straight_part(const Straight<R> &S, R h, R *y, R *qc) {
     straight_amplitudes<R>(y, straight_gain<R>(h, straight_gamma<R>(S, R(0)), straight_gamma<R>(S, R(0.5) * h),
                                                straight_gamma<R>(S, h)));
     straight_q<R>(S, h, y + F_Q, qc);
-#pragma unroll
-    for (int f = 0; f < 18; f++) y[F_DQ + f] += h * B[f];
 }
 
 }  // namespace fga
