@@ -299,7 +299,7 @@ void HostBuf::release() {
 }
 void Workspace::release() {
     for (DevBuf *d : {&keys, &keys_alt, &vals, &vals_alt, &hist, &scan_blocks, &cell_start, &rec, &items, &tiles,
-                      &partial, &pts, &status, &rec_amax})
+                      &partial, &pts, &status, &rec_amax, &gauss_tables})
         d->release();
     for (HostBuf *h : {&h_cell_start, &h_items, &h_tiles}) h->release();
 }

@@ -208,7 +208,7 @@ void pool_object(int d);
 
 // scratch used by binning and the Gaussian sum
 struct Workspace {
-    DevBuf keys, keys_alt, vals, vals_alt, hist, scan_blocks, cell_start, rec, items, tiles, partial, pts;
+    DevBuf keys, keys_alt, vals, vals_alt, hist, scan_blocks, cell_start, rec, items, tiles, partial, pts, gauss_tables;
     DevBuf rec_amax;   // per sample of a window: bound of the records' amplitude entries (FP32 path)
     // status words of one call: [0] a bounded wait of the tensor-core lattice sum ran out,
     // [1] non-finite values in the beam state or the outputs
