@@ -590,20 +590,21 @@ __global__ void __launch_bounds__(32 * GD_WARPS) gather_f64_kernel(const double 
     }
 }
 
-// The same sum in FP32.  A warp takes 32 points of the tile and a quarter of the item's beams, staged 32 at a time
-// in shared memory field by field (the next 32 in flight in registers), so that two consecutive beams are the two
-// halves of packed FP32x2 operands: coordinates and accumulators are packed once, and a pair of beams costs 30
-// packed FMAs, 6 MUFU and 12 other instructions for 64 (beam, point) pairs.  Bound by the FMA pipe (62 cycles a
-// warp and 64 pairs; MUFU 48).  Against one beam and point per lane with uniform loads (41 instructions per 32
-// pairs, long-scoreboard stalls): 1.05 M beams x 5,003 points 8.2 -> 5.3 ms, 100
-// samples of 256 receivers and 1.05 M beams 43.0 -> 21.2 ms (issue slots 65%, FMA pipe 55%).
-constexpr int GF_BEAMS = 32;
+// The same sum in FP32.  A warp takes 32 points of the tile and a quarter of the item's beams.  Those whose window
+// reaches the points' box are staged in shared memory field by field (the next 32 in flight in registers), so
+// that two consecutive beams are the two halves of packed FP32x2 operands: coordinates and accumulators are packed
+// once, and a pair of beams costs 30 packed FMAs, 6 MUFU and 12 other instructions for 64 (beam, point) pairs.  Bound
+// by the FMA pipe (62 cycles a warp and 64 pairs; MUFU 48).  Against one beam and point per lane with uniform loads (41
+// instructions per 32 pairs, long-scoreboard stalls): 1.05 M beams x 5,003 points 8.2 -> 5.3 ms, 100 samples of 256
+// receivers and 1.05 M beams 43.0 -> 21.2 ms.  With compact tiles 4.20 and 21.2 ms, staging only what reaches the box
+// 3.99 and 18.6 ms.
+constexpr int GF_STAGE = 64;
 __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict__ rec, int64_t rec_stride,
                                                          const double *__restrict__ pts,
                                                          const int32_t *__restrict__ tile_pts,
                                                          const int4 *__restrict__ items, float k, float rw2,
                                                          float *__restrict__ partial, int count_pairs) {
-    __shared__ float stage[4][2][REC][GF_BEAMS];
+    __shared__ float stage[4][REC][GF_STAGE];
     __shared__ float red[4][32][6];
     __shared__ unsigned npairs;
     if (threadIdx.x == 0) npairs = 0;
@@ -639,25 +640,34 @@ __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict
             n1 = n2 = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
-    fetch(b0);
-    int buf = 0;
-    for (int64_t b = b0; b < b1; b += GF_BEAMS, buf ^= 1) {
-        float(*st)[GF_BEAMS] = stage[warp][buf];
-        st[0][lane] = -n0.x;
-        st[1][lane] = -n0.y;
-        st[2][lane] = -n0.z;
-        st[3][lane] = k * n0.w;
-        st[4][lane] = k * n1.x;
-        st[5][lane] = k * n1.y;
-        st[6][lane] = n1.z;
-        st[7][lane] = n1.w;
-        st[8][lane] = n2.x;
-        st[9][lane] = n2.y;
-        st[10][lane] = n2.z;
-        st[11][lane] = n2.w;
-        __syncwarp();   // the other half was last read before the previous synchronisation of this kind
-        if (b + GF_BEAMS < b1) fetch(b + GF_BEAMS);
-        const int nb = (int)(b1 - b < GF_BEAMS ? b1 - b : GF_BEAMS);
+    // the points' box: beams whose window does not reach it are not staged
+    const float far = __int_as_float(0x7f800000);
+    float lo[3] = {pi >= 0 ? x0 : far, pi >= 0 ? x1 : far, pi >= 0 ? x2 : far};
+    float hi[3] = {pi >= 0 ? x0 : -far, pi >= 0 ? x1 : -far, pi >= 0 ? x2 : -far};
+#pragma unroll
+    for (int d = 0; d < 3; d++)
+        for (int o = 16; o; o >>= 1) {
+            lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+            hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+        }
+    const float reach2 = fmaxf(rw2 * 1.00001f, 1e-37f);
+    auto put = [&](int slot) {
+        float *st = &stage[warp][0][slot];
+        st[0 * GF_STAGE] = -n0.x;
+        st[1 * GF_STAGE] = -n0.y;
+        st[2 * GF_STAGE] = -n0.z;
+        st[3 * GF_STAGE] = k * n0.w;
+        st[4 * GF_STAGE] = k * n1.x;
+        st[5 * GF_STAGE] = k * n1.y;
+        st[6 * GF_STAGE] = n1.z;
+        st[7 * GF_STAGE] = n1.w;
+        st[8 * GF_STAGE] = n2.x;
+        st[9 * GF_STAGE] = n2.y;
+        st[10 * GF_STAGE] = n2.z;
+        st[11 * GF_STAGE] = n2.w;
+    };
+    auto sum = [&](int first, int nb) {
+        const float(*st)[GF_STAGE] = reinterpret_cast<const float(*)[GF_STAGE]>(&stage[warp][0][first]);
         for (int j = 0; j < nb; j += 4) {
             float4 f[6];
 #pragma unroll
@@ -692,6 +702,36 @@ __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict
                 }
             }
         }
+    };
+    // the stage is a ring of two halves: a half is summed once it is full, the beams that follow fill the other
+    int at = 0, pending = 0;
+    fetch(b0);
+    for (int64_t b = b0; b < b1; b += 32) {
+        const float e0 = fmaxf(fmaxf(lo[0] - n0.x, n0.x - hi[0]), 0.f), e1 = fmaxf(fmaxf(lo[1] - n0.y, n0.y - hi[1]), 0.f),
+                    e2 = fmaxf(fmaxf(lo[2] - n0.z, n0.z - hi[2]), 0.f);
+        const bool keep = b + lane < b1 && e0 * e0 + e1 * e1 + e2 * e2 <= reach2;
+        const unsigned kept = __ballot_sync(0xffffffffu, keep);
+        if (keep) put((at + __popc(kept & ((1u << lane) - 1u))) & (GF_STAGE - 1));
+        __syncwarp();
+        if (b + 32 < b1) fetch(b + 32);
+        const int nk = __popc(kept), half = (at - pending) & (GF_STAGE - 1);
+        at = (at + nk) & (GF_STAGE - 1);
+        pending += nk;
+        if (pending >= GF_STAGE / 2) {
+            sum(half, GF_STAGE / 2);
+            pending -= GF_STAGE / 2;
+        }
+        __syncwarp();   // the half just read may be written next
+    }
+    if (pending > 0) {
+        // up to three beams outside every window fill the last group of four
+        if (lane < (-pending & 3)) {
+            n0 = make_float4(-1e15f, -1e15f, -1e15f, 0.f);
+            n1 = n2 = make_float4(0.f, 0.f, 0.f, 0.f);
+            put((at + lane) & (GF_STAGE - 1));
+        }
+        __syncwarp();
+        sum((at - pending) & (GF_STAGE - 1), pending);
     }
 #pragma unroll
     for (int j = 0; j < 6; j++) red[warp][lane][j] = acc[j].x + acc[j].y;
