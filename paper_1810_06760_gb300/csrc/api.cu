@@ -650,15 +650,15 @@ fga_status fga_propagate(const fga_model *m, fga_beams *b, double dt, int nsteps
     return FGA_OK;
 }
 
-// sort the beams' current centres on a grid; returns the permutation and the bucket starts (device)
-static fga_status bin_beams(const fga_beams *b, const BinGrid &g, int32_t **perm, cudaStream_t s) {
+// sort the beams' current centres on a grid; returns the permutation and the bucket starts (device).  drop: of the
+// beams inside the grid only
+static fga_status bin_beams(const fga_beams *b, const BinGrid &g, bool drop, int32_t **perm, cudaStream_t s) {
     Workspace &ws = b->ws;
     const int nbk = 4 * (g.ncells + 1);
-    FGA_TRY(ws.keys.ensure(sizeof(int32_t) * (size_t)std::max<int64_t>(b->nb, 1)));
     FGA_TRY(ws.cell_start.ensure(sizeof(int32_t) * (size_t)(nbk + 1)));
     const int kind = b->precision == FGA_PREC_FP64 ? Q_F64_SOA : Q_F32_SOA;
-    FGA_TRY(bin_centres(g, b->state.p, kind, b->cap, b->nb, b->flags.as<int32_t>(), ws.keys.as<int32_t>(), s));
-    return sort_keys_to_perm(ws, ws.keys.as<int32_t>(), b->nb, nbk, perm, ws.cell_start.as<int32_t>(), s);
+    return sort_centres(ws, g, b->state.p, kind, b->cap, b->nb, b->flags.as<int32_t>(), drop, nbk, perm,
+                        ws.cell_start.as<int32_t>(), nullptr, s);
 }
 
 static fga_status host_points(const double *x_dev, int64_t n, std::vector<double> &out, cudaStream_t s) {
@@ -713,7 +713,7 @@ static fga_status reconstruct_now(const fga_beams *b, const double *x_dev, const
     Workspace &ws = b->ws;
     const BinGrid g = make_grid(xh.data(), n, rw);
     int32_t *perm = nullptr;
-    FGA_TRY(bin_beams(b, g, &perm, s));
+    FGA_TRY(bin_beams(b, g, true, &perm, s));
     SumPlan plan;
     FGA_TRY(build_sum_plan(ws, g, ws.cell_start.as<int32_t>(), 4, xh.data(), n, 1, s, plan));  // syncs
     const size_t rb = b->precision == FGA_PREC_FP64 ? 8 : 4;
@@ -803,7 +803,7 @@ static fga_status reconstruct_lattice_now(const fga_beams *b, const fga_lattice 
     const std::vector<double> corners = lattice_corners(L);
     const BinGrid g = make_grid(corners.data(), 8, rw);
     int32_t *perm = nullptr;
-    FGA_TRY(bin_beams(b, g, &perm, s));
+    FGA_TRY(bin_beams(b, g, true, &perm, s));
     LatticePlan plan;
     FGA_TRY(build_lattice_plan(ws, g, ws.cell_start.as<int32_t>(), *L, s, plan, b->precision == FGA_PREC_FP32, b->k,
                                rw));  // syncs
@@ -1025,7 +1025,7 @@ fga_status solve_impl(const fga_model *m, const fga_init_desc *init, const fga_s
         int32_t *perm = nullptr;
         {
             NvtxRange nr("fga_solve: binning");
-            FGA_TRY(bin_beams(b, grx, &perm, s));
+            FGA_TRY(bin_beams(b, grx, false, &perm, s));
             FGA_TRY(permute_beams(b, perm, s));
         }
         SumPlan plan;
@@ -1386,11 +1386,8 @@ fga_status fga_bin(const float *Q, int64_t n, const float origin[3], float inv_h
     g.inv_h = inv_h;
     g.clamp = true;
     static thread_local Workspace ws;  // scratch of the standalone binning entry point
-    FGA_TRY(ws.keys.ensure(sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1)));
-    FGA_TRY(bin_centres(g, Q, Q_F32_AOS3, 0, n, nullptr, ws.keys.as<int32_t>(), s));
-    if (keys && n > 0) FGA_CUDA(cudaMemcpyAsync(keys, ws.keys.p, 4 * (size_t)n, cudaMemcpyDeviceToDevice, s));
     int32_t *pv = nullptr;
-    FGA_TRY(sort_keys_to_perm(ws, ws.keys.as<int32_t>(), n, g.ncells, &pv, cell_start, s));
+    FGA_TRY(sort_centres(ws, g, Q, Q_F32_AOS3, 0, n, nullptr, false, g.ncells, &pv, cell_start, keys, s));
     if (n > 0) FGA_CUDA(cudaMemcpyAsync(perm, pv, 4 * (size_t)n, cudaMemcpyDeviceToDevice, s));
     FGA_CUDA(cudaStreamSynchronize(s));
     return FGA_OK;

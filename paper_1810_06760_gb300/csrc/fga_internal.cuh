@@ -290,11 +290,9 @@ struct BinGrid {
 };
 // exclusive prefix sum of n uint32 in place on stream s (synchronises s before returning)
 fga_status scan_exclusive_u32(uint32_t *a, int64_t n, cudaStream_t s);
-fga_status bin_centres(const BinGrid &g, const void *Q_src, int q_kind, int64_t q_stride, int64_t n,
-                       const int32_t *cls_or_null, int32_t *keys, cudaStream_t s);
-fga_status radix_sort_pairs(Workspace &ws, int32_t *keys, int32_t *vals, int64_t n, int bits,
-                            int32_t **keys_out, int32_t **vals_out, cudaStream_t s);
-fga_status cell_starts(const int32_t *sorted_keys, int64_t n, int nbuckets, int32_t *cell_start, cudaStream_t s);
+fga_status sort_centres(Workspace &ws, const BinGrid &g, const void *Q_src, int q_kind, int64_t q_stride, int64_t n,
+                        const int32_t *cls_or_null, bool drop, int nbuckets, int32_t **perm_out, int32_t *cell_start,
+                        int32_t *keys_copy, cudaStream_t s);
 fga_status permute_beams(fga_beams *b, const int32_t *perm, cudaStream_t s);
 // binning grid covering every point of a set, expanded by `reach`, with cells >= reach
 BinGrid make_grid(const double *pts_host, int64_t n, double reach);

@@ -80,8 +80,6 @@ fga_status run_lattice(Workspace &ws, const LatticePlan &plan, int precision, co
                        const float *amax = nullptr);
 int64_t read_lattice_pair_counter(bool reset);
 
-fga_status sort_keys_to_perm(Workspace &ws, int32_t *keys, int64_t n, int nbuckets, int32_t **perm_out,
-                             int32_t *cell_start, cudaStream_t s);
 fga_status build_sum_plan(Workspace &ws, const BinGrid &g, const int32_t *cell_start_dev, int nclasses,
                           const double *pts_host, int64_t npts, int samples, cudaStream_t s, SumPlan &plan);
 constexpr size_t SUM_PARTIAL_MAX = (size_t)256 << 20;   // bytes of partial sums per launch of several samples
