@@ -274,10 +274,12 @@ __global__ void __launch_bounds__(128) rk4_cell_kernel(ModelDev M, float *__rest
 }
 
 // Constant media: nsteps RK4 steps in closed form (straight.cuh), one launch for all classes
-// (blockIdx.y the class).  Bound by the state's HBM stream in FP32 (49 reals read and 28 written per beam
-// and launch: P and dzP do not change) and by the FP64 pipe in FP64 (two reciprocals and ~80 operations a
-// step).  Against the general kernel's four right-hand sides per step: point-force experiment, 13.9 M beams
-// x 79 steps FP32, 63.7 -> 4.3 ms; homogeneous experiment, 373 k beams x 100 steps FP64, 126.7 -> 8.1 ms.
+// (blockIdx.y the class).  Bound by the issue slots in FP32 (about 100 instructions a step, slots 80% used; the state's
+// stream, 49 reals read and 28 written per beam and launch, is a quarter of the time) and by the FP64 pipe in FP64.  The
+// steps gather the amplitudes' gain in one complex factor, applied at samples and at the end, and in FP64 two
+// reciprocals share a division.  Against the general kernel's four right-hand sides per step: point-force experiment,
+// 13.9 M beams x 79 steps FP32, 63.7 -> 3.8 ms; homogeneous experiment, 373 k beams x 100 steps FP64, 126.7 -> 7.6 ms
+// (4.3 and 8.1 ms with both amplitudes advanced every step and a division per reciprocal).
 template <typename R>
 __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ st, const int32_t *__restrict__ flags,
                                                    int64_t cap, ClassBlocks cc, R dt, int nsteps, int n_samp,
@@ -301,33 +303,51 @@ __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ 
         Straight<R> S;
         straight_setup<R>(sg, c, y, B, S);
         const int m = min(STRAIGHT_RENEW, nsteps - n0);
-        C2<R> g1 = straight_gamma<R>(S, R(0));
+        C2<R> g1 = straight_gamma<R>(S, R(0)), fac = {R(1), R(0)};   // fac: what the amplitudes have gained
+        R rs = R(0);   // s, counted in FP64 (a conversion is an operation of the FP64 pipe)
         for (int s = 0; s < m; s++) {
-            const R t = R(s) * dt;
-            const C2<R> g2 = straight_gamma<R>(S, t + R(0.5) * dt), g4 = straight_gamma<R>(S, t + dt);
+            const R t = (sizeof(R) == 4 ? R(s) : rs) * dt;
+            rs += R(1);
+            C2<R> g2, g4;
+            straight_gamma2<R>(S, t + R(0.5) * dt, t + dt, g2, g4);
             R y0[NF];   // Q, P and the amplitudes at the step's start (the rest is not read by a record)
 #pragma unroll
             for (int f = 0; f < 6; f++) y0[f] = y[f];
-#pragma unroll
-            for (int f = F_A0; f < NF; f++) y0[f] = y[f];
             straight_q<R>(S, dt, y + F_Q, qc);
-            straight_amplitudes<R>(y, straight_gain<R>(dt, g1, g2, g4));
+            const C2<R> f0 = fac, gain = straight_gain<R>(dt, g1, g2, g4), inc = cmul(gain, fac);
+            fac = {fac.r + inc.r, fac.i + inc.i};
             g1 = g4;
             while (js < n_samp && samp_step[js] == n0 + s) {
                 float mloc = 0.f;
                 if (i < cc.n_in[cls]) {
                     const R sl[6] = {S.v[0], S.v[1], S.v[2], R(0), R(0), R(0)};
-                    R r[REC];
+                    R r[REC], y1[NF];
+#pragma unroll
+                    for (int f = 0; f < 6; f++) y1[f] = y[f];
+#pragma unroll
+                    for (int f = F_A0; f < NF; f += 2) {
+                        const C2<R> a = {y[f], y[f + 1]}, b0 = cmul(f0, a), b1 = cmul(fac, a);
+                        y0[f] = b0.r;
+                        y0[f + 1] = b0.i;
+                        y1[f] = b1.r;
+                        y1[f + 1] = b1.i;
+                    }
                     if (wave)
-                        beam_record6<R, 1>(ref_e1, y0, sl, y, sl, dt, samp_theta[js], w, r);
+                        beam_record6<R, 1>(ref_e1, y0, sl, y1, sl, dt, samp_theta[js], w, r);
                     else
-                        beam_record6<R, 0>(ref_e1, y0, sl, y, sl, dt, samp_theta[js], w, r);
+                        beam_record6<R, 0>(ref_e1, y0, sl, y1, sl, dt, samp_theta[js], w, r);
                     store_record<R>(rec, (int64_t)js * rec_stride + cc.rec_off[cls] + i, r);
                     mloc = record_bound<R>(r);
                 }
                 if (amax) sample_bound(amax + js, mloc);
                 js++;
             }
+        }
+#pragma unroll
+        for (int f = F_A0; f < NF; f += 2) {
+            const C2<R> a = cmul(fac, C2<R>{y[f], y[f + 1]});
+            y[f] = a.r;
+            y[f + 1] = a.i;
         }
         const R T = R(m) * dt;
 #pragma unroll
