@@ -540,7 +540,7 @@ __device__ __forceinline__ void gauss_phase_table(double ph, double am, const Ga
 }
 static_assert(EX_N == 1 << 10, "the power of two is the index above its table part");
 
-// FP64: a warp takes 32 points of the tile and a quarter of the item's beams, staged 32 at a time.  Bound by the FP64 pipe
+// FP64: a warp takes 32 points of the tile and every fourth 32 of the item's beams, staged.  Bound by the FP64 pipe
 // (a warp instruction in 16 cycles): 53 operations per pair, of which sine, cosine and exponential are 28 by table
 // against about 65 of the library's.  With one beam at a time for all lanes 54% of the lanes were idle: outside its
 // window, or without a point (scattered receivers are a few to a cell).  So a tile of n <= 16 points takes every point
@@ -595,13 +595,12 @@ __global__ void __launch_bounds__(32 * GD_WARPS) gather_f64_kernel(const double 
     const double o0 = pts[3 * (int64_t)p0], o1 = pts[3 * (int64_t)p0 + 1], o2 = pts[3 * (int64_t)p0 + 2];
     const float f0 = (float)(x0 - o0), f1 = (float)(x1 - o1), f2 = (float)(x2 - o2);
     const float screen = fmaxf((float)(rw2 * 1.00001), 1e-37f);
-    const int64_t len = (int64_t)it.z - it.y;
-    const int64_t b0 = it.y + (len * warp) / GD_WARPS, b1 = it.y + (len * (warp + 1)) / GD_WARPS;
+    const int64_t b0 = it.y + 32 * warp, b1 = it.z;   // stages in turn: the warps' shares of the window are alike
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     const double hk = -0.5 * k;
     double(*R)[REC] = S.rec[warp];
     float(*Q)[3] = S.q[warp];
-    for (int64_t b = b0; b < b1; b += 32) {
+    for (int64_t b = b0; b < b1; b += 32 * GD_WARPS) {
         const int m = (int)min((int64_t)32, b1 - b);
         const double2 *src = reinterpret_cast<const double2 *>(rec + b * REC);
         __syncwarp();
@@ -671,14 +670,14 @@ __global__ void __launch_bounds__(32 * GD_WARPS) gather_f64_kernel(const double 
     }
 }
 
-// The same sum in FP32.  A warp takes 32 points of the tile and a quarter of the item's beams.  Those whose window
+// The same sum in FP32.  A warp takes 32 points of the tile and every fourth 32 of the item's beams.  Those whose window
 // reaches the points' box are staged in shared memory field by field (the next 32 in flight in registers), so
 // that two consecutive beams are the two halves of packed FP32x2 operands: coordinates and accumulators are packed
 // once, and a pair of beams costs 30 packed FMAs, 6 MUFU and 12 other instructions for 64 (beam, point) pairs.  Bound
 // by the FMA pipe (62 cycles a warp and 64 pairs; MUFU 48).  Against one beam and point per lane with uniform loads (41
 // instructions per 32 pairs, long-scoreboard stalls): 1.05 M beams x 5,003 points 8.2 -> 5.3 ms, 100 samples of 256
 // receivers and 1.05 M beams 43.0 -> 21.2 ms.  With compact tiles 4.20 and 21.2 ms, staging only what reaches the box
-// 3.99 and 18.6 ms.
+// 3.99 and 18.6 ms, the warps taking 32 beams in turn instead of a quarter of the item each 3.81 and 17.3 ms.
 constexpr int GF_STAGE = 64;
 __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict__ rec, int64_t rec_stride,
                                                          const double *__restrict__ pts,
@@ -696,8 +695,7 @@ __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict
     const float x0 = pi >= 0 ? (float)pts[3 * (int64_t)pi] : 1e15f, x1 = pi >= 0 ? (float)pts[3 * (int64_t)pi + 1] : 1e15f,
                 x2 = pi >= 0 ? (float)pts[3 * (int64_t)pi + 2] : 1e15f;
     const float2 X0 = make_float2(x0, x0), X1 = make_float2(x1, x1), X2 = make_float2(x2, x2);
-    const int64_t len = (int64_t)it.z - it.y;
-    const int64_t b0 = it.y + (len * warp) / 4, b1 = it.y + (len * (warp + 1)) / 4;
+    const int64_t b0 = it.y + 32 * warp, b1 = it.z;   // 32 beams in turn: the warps' shares of the window are alike
     const float *r0 = rec + blockIdx.y * rec_stride;
     const float hk2 = -0.72134752044448170368f * k;   // -k/2 in units of log 2
     constexpr double TWO_PI = 6.283185307179586476925286766559;
@@ -787,14 +785,14 @@ __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict
     // the stage is a ring of two halves: a half is summed once it is full, the beams that follow fill the other
     int at = 0, pending = 0;
     fetch(b0);
-    for (int64_t b = b0; b < b1; b += 32) {
+    for (int64_t b = b0; b < b1; b += 128) {
         const float e0 = fmaxf(fmaxf(lo[0] - n0.x, n0.x - hi[0]), 0.f), e1 = fmaxf(fmaxf(lo[1] - n0.y, n0.y - hi[1]), 0.f),
                     e2 = fmaxf(fmaxf(lo[2] - n0.z, n0.z - hi[2]), 0.f);
         const bool keep = b + lane < b1 && e0 * e0 + e1 * e1 + e2 * e2 <= reach2;
         const unsigned kept = __ballot_sync(0xffffffffu, keep);
         if (keep) put((at + __popc(kept & ((1u << lane) - 1u))) & (GF_STAGE - 1));
         __syncwarp();
-        if (b + 32 < b1) fetch(b + 32);
+        if (b + 128 < b1) fetch(b + 128);
         const int nk = __popc(kept), half = (at - pending) & (GF_STAGE - 1);
         at = (at + nk) & (GF_STAGE - 1);
         pending += nk;
