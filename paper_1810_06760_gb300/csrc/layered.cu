@@ -545,33 +545,35 @@ __device__ __forceinline__ void push_event(int2 *__restrict__ list, unsigned *__
 // meets an interface; such beams are listed with their step (or die, past their last allowed interface).
 // One state stream per group instead of one per step: 49 reals read and 28 written per beam (P and dzP stay),
 // which bounds it.  442 k beams growing to 0.9 M, 300 steps in groups of 5, FP32: 69.6 ms (a launch per step
-// with four right-hand sides, events inside) -> 3.8 ms of these kernels and 3.8 ms of event kernels; with
-// undulating interfaces (an FP64 test of the end point where the FP32 screen cannot decide) 187 -> 5.5 and 7.9 ms.
+// with four right-hand sides, events inside) -> 3.2 ms of these kernels and 3.8 ms of event kernels; with
+// undulating interfaces (an FP64 test of the end point where the FP32 screen cannot decide) 187 -> 5.2 and 7.9 ms.
+// The grid strides over the live beams: blocks for the whole reserved capacity, eight times the first population, cost 0.6 ms.
 template <typename R, int SHAPE>
 __global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
                                                          int64_t cap, const unsigned long long *__restrict__ counts,
                                                          R dt, int nsteps, int gmax, int2 *__restrict__ list,
                                                          unsigned *__restrict__ nlist) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= cap || (unsigned long long)b >= counts[0]) return;
-    const int fl = flags[b];
-    if (fl & FL_DEAD) return;
-    R y[NF], qc[3];
-    load_beam<R>(st, cap, b, y, qc);
-    const int s = layered_run<R, SHAPE>(M, fl, y, qc, dt, 0, nsteps, false);
+    const int64_t n = min((unsigned long long)cap, counts[0]);
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+        const int fl = flags[b];
+        if (fl & FL_DEAD) continue;
+        R y[NF], qc[3];
+        load_beam<R>(st, cap, b, y, qc);
+        const int s = layered_run<R, SHAPE>(M, fl, y, qc, dt, 0, nsteps, false);
 #pragma unroll
-    for (int f = 0; f < 3; f++) st[(int64_t)f * cap + b] = y[f];
+        for (int f = 0; f < 3; f++) st[(int64_t)f * cap + b] = y[f];
 #pragma unroll
-    for (int f = F_DQ; f < F_DP; f++) st[(int64_t)f * cap + b] = y[f];
+        for (int f = F_DQ; f < F_DP; f++) st[(int64_t)f * cap + b] = y[f];
 #pragma unroll
-    for (int f = F_A0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
+        for (int f = F_A0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
 #pragma unroll
-    for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
-    if (s == nsteps) return;
-    if (((fl >> 8) & 15) >= gmax)
-        flags[b] = fl | FL_DEAD;
-    else
-        push_event(list, nlist, b, s);
+        for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
+        if (s == nsteps) continue;
+        if (((fl >> 8) & 15) >= gmax)
+            flags[b] = fl | FL_DEAD;
+        else
+            push_event(list, nlist, b, s);
+    }
 }
 
 // The listed beams: the event of step s at its interface, then every child finishes that step and advances
@@ -705,7 +707,7 @@ fga_status launch_layered_steps(const fga_model *m, fga_beams *b, double dt, int
         unsigned long long *counts = b->counts.as<unsigned long long>();
         {
             ProfScope ps(P_PROP, s);
-            layered_run_kernel<R, SHAPE><<<(unsigned)((b->cap + 127) / 128), 128, 0, s>>>(
+            layered_run_kernel<R, SHAPE><<<(unsigned)std::min<int64_t>((b->cap + 127) / 128, 152 * 12), 128, 0, s>>>(
                 m->dev, b->state.as<R>(), b->flags.as<int32_t>(), b->cap, counts, (R)dt, nsteps, b->gmax, list[0], ctr);
         }
         for (int r = 0; r < rounds; r++) {

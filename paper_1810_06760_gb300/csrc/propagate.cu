@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(128) rk4_cell_kernel(ModelDev M, float *__rest
 // stream, 49 reals read and 28 written per beam and launch, is a quarter of the time) and by the FP64 pipe in FP64.  The
 // steps gather the amplitudes' gain in one complex factor, applied at samples and at the end, and in FP64 two
 // reciprocals share a division.  Against the general kernel's four right-hand sides per step: point-force experiment,
-// 13.9 M beams x 79 steps FP32, 63.7 -> 3.8 ms; homogeneous experiment, 373 k beams x 100 steps FP64, 126.7 -> 7.6 ms
+// 13.9 M beams x 79 steps FP32, 63.7 -> 3.8 ms; homogeneous experiment, 373 k beams x 100 steps FP64, 126.7 -> 7.7 ms
 // (4.3 and 8.1 ms with both amplitudes advanced every step and a division per reciprocal).
 template <typename R>
 __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ st, const int32_t *__restrict__ flags,
