@@ -83,17 +83,33 @@ __device__ __forceinline__ bool interface_event(const ModelDev &M, int fl, const
 #pragma unroll
     for (int d = 0; d < 3; d++) ev.Ph[d] = SHAPE == 0 ? (d < 2 ? P[d] : 0.0) : P[d] - pz * n[d];
     const double ph2 = ev.Ph[0] * ev.Ph[0] + ev.Ph[1] * ev.Ph[1] + ev.Ph[2] * ev.Ph[2];
-    double ph = 0.0, nsh[3] = {0.0, 1.0, 0.0};
-    if (ph2 > 0.0) {
-        const double ip = rsqrt(ph2);
-        ph = ph2 * ip;
-        nsh[0] = SHAPE == 0 ? -ip * P[1] : ip * (n[1] * ev.Ph[2] - n[2] * ev.Ph[1]);
-        nsh[1] = SHAPE == 0 ? ip * P[0] : ip * (n[2] * ev.Ph[0] - n[0] * ev.Ph[2]);
-        nsh[2] = SHAPE == 0 ? 0.0 : ip * (n[0] * ev.Ph[1] - n[1] * ev.Ph[0]);
-    } else if (SHAPE != 0) {
-        double Rl[9];
-        frame_from_normal(n, Rl);
-        for (int d = 0; d < 3; d++) nsh[d] = Rl[3 + d];
+    const double ph = sqrt(ph2);
+    double nsh[3] = {0.0, 1.0, 0.0};
+    if (SHAPE == 0) {
+        if (ph2 > 0.0) {
+            const double ip = rsqrt(ph2);
+            nsh[0] = -ip * P[1];
+            nsh[1] = ip * P[0];
+        }
+    } else {
+        // Near normal incidence n x P is rounding, part of it along n.  That part is taken out and what is left is
+        // normalised by itself, so that nsh is a unit vector normal to n and P, whose direction in the interface does not
+        // matter there (divided by |P_h|, rounding along n and all, S beams lost up to all of their amplitude); where
+        // nothing but rounding is left, any direction in the interface.
+        double v[3] = {n[1] * P[2] - n[2] * P[1], n[2] * P[0] - n[0] * P[2], n[0] * P[1] - n[1] * P[0]};
+        const double vn = v[0] * n[0] + v[1] * n[1] + v[2] * n[2];
+#pragma unroll
+        for (int d = 0; d < 3; d++) v[d] -= vn * n[d];
+        const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        if (v2 > 1e-28 * pin * pin) {
+            const double iv = rsqrt(v2);
+#pragma unroll
+            for (int d = 0; d < 3; d++) nsh[d] = iv * v[d];
+        } else {
+            double Rl[9];
+            frame_from_normal(n, Rl);
+            for (int d = 0; d < 3; d++) nsh[d] = Rl[3 + d];
+        }
     }
     // incident amplitudes along P/|P|, or along SV and SH of the interface
     const Cd a0 = {(double)y[F_A0], (double)y[F_A0 + 1]}, a1 = {(double)y[F_A1], (double)y[F_A1 + 1]};
