@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
             if (warp < 3) {   // 16 bytes of one record per thread
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (lane < nb)
-                    v = __ldg(reinterpret_cast<const float4 *>(rec + (it.y + keptc[kb0 + lane]) * REC) + warp);
+                    v = __ldg(reinterpret_cast<const float4 *>(rec + ((int64_t)it.y + keptc[kb0 + lane]) * REC) + warp);
                 float *d = dst + 4 * warp * LT_RS + lane;
                 d[0] = v.x;
                 d[LT_RS] = v.y;
