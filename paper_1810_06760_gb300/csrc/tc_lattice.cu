@@ -27,7 +27,7 @@
 // warp forms one chunk of points for its 32 lanes' beams without divergence or bank conflicts, and an operand task
 // reads 16-byte runs, multiplies two beams per packed FP32x2 operation and splits them in pairs; rows that share E2
 // and columns that share E0 are formed by one thread.  The operands' power-of-two scales are folded into the
-// factors, and the copies of B' that repeat or negate another are stored, not formed again.  Bound by shared
+// amplitudes and the factors, and the copies of B' that repeat or negate another are stored, not formed again.  Bound by shared
 // memory: 960 wavefronts of operand reads by the tensor cores and 1,790 of stores and loads per block of 32 beams,
 // 86% of its 3,210 cycles (tensor pipe 36%).  61 x 64 x 57 points (64 tiles), 1.05 M beams: 16.1 -> 12.8 ms; 64^3
 // snapshot of 8.4 M beams 136 -> 99 ms.
@@ -153,8 +153,6 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
         }
     }
     const float sy = 16384.0f;
-    // the A_c factor carries the amplitude scale on whichever side it sits
-    const float sA_scale = crow ? sx : sy, sB_scale = crow ? sy : sx;
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -209,11 +207,13 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (lane < nb)
                     v = __ldg(reinterpret_cast<const float4 *>(rec + ((int64_t)it.y + keptc[kb0 + lane]) * REC) + warp);
+                // the amplitudes (fields 6 to 11) carry their operand's scale
+                const float s01 = warp == 2 ? sx : 1.0f, s23 = warp >= 1 ? sx : 1.0f;
                 float *d = dst + 4 * warp * LT_RS + lane;
-                d[0] = v.x;
-                d[LT_RS] = v.y;
-                d[2 * LT_RS] = v.z;
-                d[3 * LT_RS] = v.w;
+                d[0] = v.x * s01;
+                d[LT_RS] = v.y * s01;
+                d[2 * LT_RS] = v.z * s23;
+                d[3 * LT_RS] = v.w * s23;
             }
         };
         // a warp per chunk of points, a lane per beam
@@ -227,8 +227,10 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
                 float *dst = sE + (off + a0) * LT_ES + lane;
                 const float Qd = sR[d * LT_RS + lane], Pd = sR[(3 + d) * LT_RS + lane];
                 const float x = sX[off + a0] - Qd;
-                // E0 and E1 carry the operand scales (powers of two); padding beams are zero
-                const float scl = lane < nb ? (d == 0 ? sB_scale : (d == 1 ? sA_scale : 1.0f)) : 0.0f;
+                // the operand without amplitudes takes its scale on E0 (components as rows) or E1: 2^14 keeps a run's
+                // first value from underflowing, which the amplitudes' scale, as small as they are large, would not;
+                // padding beams are zero
+                const float scl = lane < nb ? (d == (crow ? 0 : 1) ? sy : 1.0f) : 0.0f;
                 float er, ei;
                 gauss_phase_exp<float>(k * Pd * x, hk * x * x, &er, &ei);
                 er *= scl;
