@@ -45,7 +45,8 @@ fga_status build_lattice_plan(Workspace &ws, const BinGrid &g, const int32_t *ce
 // each ratio times exp(-k h^2).  In FP32 a first value with k (x - Q)^2 / 2 > 87 underflows and
 // zeroes the run; a kept beam lies within rw of the tile, and the values lost that way stay below
 // e^-14 of its amplitude when a run spans at most recurrence_span_max(k, rw).  The ratio itself is
-// finite while k h (span + rw + h) <= 87 (recurrence_ratio_ok); otherwise the run is one point.
+// finite while k h (span + rw + h) <= 87 (recurrence_ratio_ok); otherwise the run is one point.  That holds for beams within
+// rw of the run; the volume kernel bounds the ratio of beams farther along the tile, the plane kernel caps the tile.
 double recurrence_span_max(double k, double rw);
 bool recurrence_ratio_ok(double k, double step, double span, double rw);
 void tile_shape_tc(const fga_lattice &L, int T[3]);

@@ -240,7 +240,9 @@ __global__ void __launch_bounds__(LT_THREADS, MINB) lattice_tc_kernel(const floa
                 if (a1 - a0 > 1) {
                     const float h = X.dx[d];
                     float rr, ri;
-                    gauss_phase_exp<float>(k * Pd * h, -k * h * (x + 0.5f * h), &rr, &ri);
+                    // a beam beyond the far end of a long tile has a ratio past the largest float here; its values on this
+                    // run, below e^-18 of its amplitude, start from a first one that underflows: the bound keeps 0 x ratio 0
+                    gauss_phase_exp<float>(k * Pd * h, fminf(-k * h * (x + 0.5f * h), 87.0f), &rr, &ri);
                     if (lane >= nb) rr = ri = 0.0f;
                     const float g = __expf(-k * h * h);
                     for (int a = a0 + 1; a < a1; a++) {
