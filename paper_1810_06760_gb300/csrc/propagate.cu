@@ -252,7 +252,7 @@ __device__ __forceinline__ void rk4_cell_body(const ModelDev &M, float *__restri
         for (int d = 0; d < 3; d++) tmp[F_Q + d] = tq[d];
     }
 #pragma unroll
-    for (int f = 0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
+    for (int f = 0; f < NW; f++) st[(int64_t)f * cap + b] = y[f];
 #pragma unroll
     for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
 }
@@ -345,6 +345,7 @@ __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ 
         }
 #pragma unroll
         for (int f = F_A0; f < NF; f += 2) {
+            if (f != F_A0 && !wave) break;   // a P beam has one amplitude
             const C2<R> a = cmul(fac, C2<R>{y[f], y[f + 1]});
             y[f] = a.r;
             y[f + 1] = a.i;
