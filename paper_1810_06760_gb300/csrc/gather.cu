@@ -988,8 +988,8 @@ fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void
     const size_t rb = precision == FGA_PREC_FP64 ? 8 : 4;
     // as many samples per launch as keep the partial sums under SUM_PARTIAL_MAX bytes
     const size_t per_sample = rb * 32 * 6 * (size_t)std::max(plan.nitems, 1);
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)ns, SUM_PARTIAL_MAX / per_sample, 65535}));
-    FGA_TRY(ws.partial.ensure(per_sample * (size_t)chunk));
+    int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)ns, SUM_PARTIAL_MAX / per_sample, 65535}));
+    FGA_TRY(ensure_scratch(ws.partial, chunk, 1, [&](int c) { return per_sample * (size_t)c; }));
     GaussTables *tables = nullptr;
     if (rb == 8 && plan.nitems > 0) {
         FGA_TRY(ws.gauss_tables.ensure(sizeof(GaussTables)));

@@ -1,6 +1,8 @@
 // Internal interface of binning and the Gaussian sum.
 #pragma once
 
+#include <algorithm>
+
 #include "fga_internal.cuh"
 
 namespace fga {
@@ -88,6 +90,16 @@ constexpr size_t SUM_PARTIAL_MAX = (size_t)256 << 20;   // bytes of partial sums
 fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void *rec, int64_t rec_stride, int ns,
                    const double *pts_dev, double k, double rw, void *u_out, int64_t u_stride, cudaStream_t s,
                    int cat = P_GATHER);
+// scratch of bytes(n) for a launch over n units (samples, items); where it does not fit the device or the caller's bound,
+// for fewer of them, down to least
+template <class F> fga_status ensure_scratch(DevBuf &b, int &n, int least, F bytes) {
+    fga_status st = b.ensure(bytes(n));
+    while (st == FGA_ERR_OOM && n > least) {
+        n = std::max(least, n / 2);
+        st = b.ensure(bytes(n));
+    }
+    return st;
+}
 // bucket starts copied to the host by build_sum_plan (valid after it returns)
 const int32_t *plan_host_cell_start(const Workspace &ws);
 

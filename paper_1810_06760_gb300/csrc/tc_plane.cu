@@ -602,18 +602,21 @@ fga_status run_plane_tc(Workspace &ws, const LatticePlan &plan, const void *rec,
                         double rw, void *u, int64_t u_stride, cudaStream_t s, int cat, const float *amax_in) {
     const int T0 = plan.T[0], T1 = plan.T[1], ncol = 12 * ((T1 + 3) / 4);
     const size_t per_item = sizeof(float) * 2 * (size_t)ncol * 128;
-    // partial sums of at most PLANE_PARTIAL_MAX bytes per launch: as many samples as fit, or else as many tiles
+    // partial sums of at most PLANE_PARTIAL_MAX bytes per launch: as many samples as fit, or else as many tiles (the
+    // same where that much does not fit the device or the caller's bound)
     const size_t max_items = PLANE_PARTIAL_MAX / per_item;
     const int32_t *starts = plan.h_item_start;
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)ns, max_items / std::max(plan.nitems, 1), 65535}));
-    const bool by_tile = (size_t)plan.nitems > max_items;
-    int most = plan.nitems;
-    if (by_tile) {
-        most = (int)max_items;
-        for (int t = 0; t < plan.ntiles; t++) most = std::max(most, starts[t + 1] - starts[t]);
-    }
-    const size_t pbytes = per_item * (size_t)std::max(most, 1) * (size_t)chunk;
-    FGA_TRY(ws.partial.ensure(pbytes + 64));
+    int tile_items = 1;   // items of the largest tile
+    for (int t = 0; t < plan.ntiles; t++) tile_items = std::max(tile_items, starts[t + 1] - starts[t]);
+    int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)ns, max_items / std::max(plan.nitems, 1), 65535}));
+    int most = std::max(plan.nitems, 1);   // items of a launch and sample
+    if ((size_t)plan.nitems > max_items) most = std::max((int)max_items, tile_items);
+    auto bytes = [&](int items, int samples) { return per_item * (size_t)items * (size_t)samples; };
+    fga_status fits = ensure_scratch(ws.partial, chunk, 1, [&](int c) { return bytes(most, c) + 64; });
+    if (fits == FGA_ERR_OOM) fits = ensure_scratch(ws.partial, most, tile_items, [&](int m) { return bytes(m, 1) + 64; });
+    FGA_TRY(fits);
+    const bool by_tile = plan.nitems > most;
+    const size_t pbytes = bytes(most, chunk);
     float *amax = reinterpret_cast<float *>(ws.partial.as<char>() + pbytes);
     if (!ws.status.p) FGA_TRY(status_reset(ws, s));
     prof_add_pairs_tested(plan.pairs_tested * ns);
