@@ -4,6 +4,7 @@
 // them in a fixed order (no atomics, deterministic).
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <numeric>
 
@@ -679,12 +680,17 @@ __global__ void __launch_bounds__(32 * GD_WARPS) gather_f64_kernel(const double 
 // receivers and 1.05 M beams 43.0 -> 21.2 ms.  With compact tiles 4.20 and 21.2 ms, staging only what reaches the box
 // 3.99 and 18.6 ms, the warps taking 32 beams in turn instead of a quarter of the item each 3.81 and 17.3 ms.
 constexpr int GF_STAGE = 64;
+struct alignas(16) GatherF32Stage {   // for its 16-byte reads (an array of floats alone is aligned to 4 bytes)
+    float f[REC][GF_STAGE];
+};
+static_assert(alignof(GatherF32Stage) % sizeof(float4) == 0 && GF_STAGE * sizeof(float) % sizeof(float4) == 0 &&
+              offsetof(GatherF32Stage, f) == 0, "16-byte reads of a field's beams");
 __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict__ rec, int64_t rec_stride,
                                                          const double *__restrict__ pts,
                                                          const int32_t *__restrict__ tile_pts,
                                                          const int4 *__restrict__ items, float k, float rw2,
                                                          float *__restrict__ partial, int count_pairs) {
-    __shared__ float stage[4][REC][GF_STAGE];
+    __shared__ GatherF32Stage stage[4];
     __shared__ float red[4][32][6];
     __shared__ unsigned npairs;
     if (threadIdx.x == 0) npairs = 0;
@@ -731,7 +737,7 @@ __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict
         }
     const float reach2 = fmaxf(rw2 * 1.00001f, 1e-37f);
     auto put = [&](int slot) {
-        float *st = &stage[warp][0][slot];
+        float *st = &stage[warp].f[0][slot];
         st[0 * GF_STAGE] = -n0.x;
         st[1 * GF_STAGE] = -n0.y;
         st[2 * GF_STAGE] = -n0.z;
@@ -746,7 +752,7 @@ __global__ void __launch_bounds__(128) gather_f32_kernel(const float *__restrict
         st[11 * GF_STAGE] = n2.w;
     };
     auto sum = [&](int first, int nb) {
-        const float(*st)[GF_STAGE] = reinterpret_cast<const float(*)[GF_STAGE]>(&stage[warp][0][first]);
+        const float(*st)[GF_STAGE] = reinterpret_cast<const float(*)[GF_STAGE]>(&stage[warp].f[0][first]);
         for (int j = 0; j < nb; j += 4) {
             float4 f[6];
 #pragma unroll
