@@ -6,9 +6,9 @@
 #include <cstring>
 #include <map>
 #include <memory>
-#include <mutex>
 #include <vector>
 
+#include "block_pool.h"
 #include "fga_beam.cuh"
 #include "gather.cuh"
 
@@ -26,84 +26,30 @@ fga_status cuda_fail(cudaError_t e, const char *what) {
     return e == cudaErrorMemoryAllocation ? FGA_ERR_OOM : FGA_ERR_CUDA;
 }
 
-// Idle blocks.  A released device or pinned block goes to a process-wide pool, per device, and serves a later
-// request of nearly its size: cudaMalloc, cudaMallocHost and their frees took 1.2 of the 1.8 ms of a small solve
-// and 10-25 ms of a large one (about 30 buffers, some of gigabytes).  Like cudaFree, whose implicit device
-// synchronisation ordered every reuse, a block released since the device was last known to be idle is handed out
-// only after a device synchronisation (one for all such blocks), so any stream and thread may release and take.
-// Idle blocks are bounded (POOL_DEV_MAX: 6% of the GPU; the largest go first), are given back when an allocation
-// fails or would pass the caller's bound, when the bound is set, and when the last model, beam set and server is
-// destroyed.
 namespace {
-constexpr size_t POOL_DEV_MAX = (size_t)16 << 30, POOL_HOST_MAX = (size_t)64 << 20;
-struct Pool {
-    struct Block {
-        void *p;
-        bool dirty;
-        int dev;   // device whose work may still use a dirty block
-    };
-    std::mutex mu;
-    std::map<int, std::multimap<size_t, Block>> dev;   // by device
-    std::multimap<size_t, Block> host;
-    size_t dev_bytes = 0, host_bytes = 0;
-    int objects = 0;   // models, beam sets and servers alive
+constexpr size_t POOL_DEV_MAX = (size_t)16 << 30;    // idle device bytes kept: 6% of the GPU
+constexpr size_t POOL_HOST_MAX = (size_t)64 << 20;
+struct CudaRt {
+    static int device() {
+        int d = 0;
+        cudaGetDevice(&d);
+        return d;
+    }
+    static bool synchronize() { return cudaDeviceSynchronize() == cudaSuccess; }
+    static void free_device(void *p) { cudaFree(p); }
+    static void free_host(void *p) { cudaFreeHost(p); }
 };
-Pool &pool() {
-    static Pool *p = new Pool();   // never destroyed: blocks may be released while the process exits
+// device bytes held by the library's own buffers, and the caller's bound on them (0: none)
+std::atomic<int64_t> g_dev_bytes{0}, g_dev_limit{0};
+BlockPool<CudaRt> &pool() {
+    // never destroyed: blocks may be released while the process exits
+    static auto *p = new BlockPool<CudaRt>(POOL_DEV_MAX, POOL_HOST_MAX, g_dev_bytes);
     return *p;
-}
-int current_device() {
-    int d = 0;
-    cudaGetDevice(&d);
-    return d;
-}
-// a block of at least need bytes, at most an eighth larger; the pool's lock is held
-void *pool_take(Pool &P, std::multimap<size_t, Pool::Block> &c, size_t &total, size_t need, size_t *size) {
-    auto it = c.lower_bound(need);
-    if (it == c.end() || it->first > need + need / 8 + 4096) return nullptr;
-    if (it->second.dirty) {
-        const int d = current_device();
-        if (it->second.dev != d || cudaDeviceSynchronize() != cudaSuccess) return nullptr;   // no reuse
-        for (auto &kv : P.dev[d]) kv.second.dirty = false;
-        for (auto &kv : P.host)
-            if (kv.second.dev == d) kv.second.dirty = false;
-    }
-    void *p = it->second.p;
-    *size = it->first;
-    total -= it->first;
-    c.erase(it);
-    return p;
-}
-// free idle device blocks, largest first, until at most keep bytes are left; the lock is held
-void pool_trim(Pool &P, size_t keep) {
-    while (P.dev_bytes > keep) {
-        std::multimap<size_t, Pool::Block> *best = nullptr;
-        for (auto &d : P.dev)
-            if (!d.second.empty() && (!best || std::prev(d.second.end())->first > std::prev(best->end())->first))
-                best = &d.second;
-        if (!best) break;
-        auto it = std::prev(best->end());
-        cudaFree(it->second.p);
-        P.dev_bytes -= it->first;
-        best->erase(it);
-    }
 }
 }  // namespace
 
-size_t pool_idle_bytes() {
-    std::lock_guard<std::mutex> lk(pool().mu);
-    return pool().dev_bytes;
-}
-void pool_object(int d) {
-    Pool &P = pool();
-    std::lock_guard<std::mutex> lk(P.mu);
-    P.objects += d;
-    if (P.objects > 0) return;
-    pool_trim(P, 0);
-    for (auto &kv : P.host) cudaFreeHost(kv.second.p);
-    P.host.clear();
-    P.host_bytes = 0;
-}
+size_t pool_idle_bytes() { return pool().idle_bytes(CudaRt::device()); }
+void pool_object(int d) { pool().object(d); }
 
 // Per-thread block cache of a server worker, in the place of the pool.  A thread that issues all its work on
 // one stream (a server worker) turns it on: released blocks go to the thread's cache and are handed
@@ -130,25 +76,18 @@ void *cache_take(std::multimap<size_t, void *> &c, size_t &total, size_t need, s
 }
 }  // namespace
 
-// device bytes held by the library's own buffers, and the caller's bound on them (0: none)
-std::atomic<int64_t> g_dev_bytes{0}, g_dev_limit{0};
-
 // allocated bytes besides the idle pool are g_dev_bytes; the bound holds for both together
 static cudaError_t dev_alloc(void **p, size_t need) {
     const int64_t lim = g_dev_limit.load();
     if (lim > 0) {
         const int64_t room = lim - g_dev_bytes.load() - (int64_t)need;
         if (room < 0) return cudaErrorMemoryAllocation;
-        std::lock_guard<std::mutex> lk(pool().mu);
-        pool_trim(pool(), (size_t)room);
+        pool().trim((size_t)room);
     }
     cudaError_t e = cudaMalloc(p, need);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        {
-            std::lock_guard<std::mutex> lk(pool().mu);
-            pool_trim(pool(), 0);
-        }
+        pool().trim_device(CudaRt::device());
         e = cudaMalloc(p, need);
     }
     if (e == cudaSuccess) g_dev_bytes += (int64_t)need;
@@ -186,6 +125,7 @@ fga_status DevBuf::ensure(size_t need) {
     if (need <= bytes && p) return FGA_OK;
     release();
     if (need == 0) need = 16;
+    device = CudaRt::device();
     if (tl_cache.on) {
         size_t got = 0;
         if (void *q = cache_take(tl_cache.dev, tl_cache.dev_bytes, need, &got)) {
@@ -194,16 +134,12 @@ fga_status DevBuf::ensure(size_t need) {
             return FGA_OK;
         }
     } else {
-        Pool &P = pool();
-        std::lock_guard<std::mutex> lk(P.mu);
         const int64_t lim = g_dev_limit.load();
-        device = current_device();
         size_t got = 0;
         if (lim <= 0 || g_dev_bytes.load() + (int64_t)(need + need / 8 + 4096) <= lim)
-            if (void *q = pool_take(P, P.dev[current_device()], P.dev_bytes, need, &got)) {
+            if (void *q = pool().take_device(device, need, &got)) {
                 p = q;
                 bytes = got;
-                g_dev_bytes += (int64_t)got;
                 return FGA_OK;
             }
     }
@@ -230,15 +166,8 @@ void DevBuf::release() {
         if (tl_cache.on) {
             tl_cache.dev.emplace(bytes, p);
             tl_cache.dev_bytes += bytes;
-        } else if (bytes > POOL_DEV_MAX) {
-            dev_free(p, bytes);
         } else {
-            Pool &P = pool();
-            std::lock_guard<std::mutex> lk(P.mu);
-            pool_trim(P, POOL_DEV_MAX - bytes);
-            P.dev[device].emplace(bytes, Pool::Block{p, true, device});
-            P.dev_bytes += bytes;
-            g_dev_bytes -= (int64_t)bytes;
+            pool().put_device(p, bytes, device);
         }
     }
     p = nullptr;
@@ -248,6 +177,7 @@ fga_status HostBuf::ensure(size_t need) {
     if (need <= bytes && p) return FGA_OK;
     release();
     if (need == 0) need = 16;
+    device = CudaRt::device();
     if (tl_cache.on) {
         size_t got = 0;
         if (void *q = cache_take(tl_cache.host, tl_cache.host_bytes, need, &got)) {
@@ -256,11 +186,8 @@ fga_status HostBuf::ensure(size_t need) {
             return FGA_OK;
         }
     } else {
-        Pool &P = pool();
-        std::lock_guard<std::mutex> lk(P.mu);
-        device = current_device();
         size_t got = 0;
-        if (void *q = pool_take(P, P.host, P.host_bytes, need, &got)) {
+        if (void *q = pool().take_host(need, &got)) {
             p = q;
             bytes = got;
             return FGA_OK;
@@ -284,14 +211,7 @@ void HostBuf::release() {
             tl_cache.host.emplace(bytes, p);
             tl_cache.host_bytes += bytes;
         } else {
-            Pool &P = pool();
-            std::lock_guard<std::mutex> lk(P.mu);
-            if (P.host_bytes + bytes <= POOL_HOST_MAX) {
-                P.host.emplace(bytes, Pool::Block{p, true, device});
-                P.host_bytes += bytes;
-            } else {
-                cudaFreeHost(p);
-            }
+            pool().put_host(p, bytes, device);
         }
     }
     p = nullptr;
@@ -446,8 +366,7 @@ int fga_version(void) { return 10000; }
 
 fga_status fga_set_device_memory_limit(double bytes) {
     g_dev_limit.store(bytes > 0 ? (int64_t)bytes : 0);
-    std::lock_guard<std::mutex> lk(pool().mu);
-    pool_trim(pool(), 0);
+    pool().trim(0);
     return FGA_OK;
 }
 

@@ -201,8 +201,8 @@ void block_cache_disable();
 void block_cache_trim(size_t keep_bytes);
 size_t block_cache_bytes();
 
-// idle blocks of the process-wide pool (see api.cu): their bytes; models, beam sets and servers created (1) and
-// destroyed (-1) -- the pool is emptied when none is left
+// idle blocks of the process-wide pool (block_pool.h): their bytes on the current device; models and beam sets created
+// (1) and destroyed (-1) -- the pool is emptied when none is left
 size_t pool_idle_bytes();
 void pool_object(int d);
 
