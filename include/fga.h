@@ -461,9 +461,10 @@ fga_status fga_profile_read(fga_profile_t *out, int reset);
  * of fga_reconstruct_noalloc): an allocation that would pass it fails with FGA_ERR_OOM before cudaMalloc
  * is called.  bytes <= 0 removes the bound (the default).  fga_device_memory_in_use reports the bytes
  * currently allocated for such buffers, without idle blocks.  Released blocks stay idle in the library for later
- * calls, up to 16 GiB; they are given back to the device when an allocation needs them, when this function
- * is called, and when the last model, beam set and server is destroyed.  Process-wide; meant for hosts that share a GPU, and for testing
- * the out-of-memory paths without exhausting the device. */
+ * calls: up to 16 GiB while a model or beam set exists, up to 512 MiB otherwise.  They are given back to the device
+ * when an allocation needs them, when this function is called, and when the last model or beam set is destroyed.
+ * Process-wide; meant for hosts that share a GPU, and for testing the out-of-memory paths without exhausting the
+ * device. */
 fga_status fga_set_device_memory_limit(double bytes);
 double fga_device_memory_in_use(void);
 

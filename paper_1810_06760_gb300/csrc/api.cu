@@ -27,7 +27,8 @@ fga_status cuda_fail(cudaError_t e, const char *what) {
 }
 
 namespace {
-constexpr size_t POOL_DEV_MAX = (size_t)16 << 30;    // idle device bytes kept: 6% of the GPU
+constexpr size_t POOL_DEV_MAX = (size_t)16 << 30;    // idle device bytes kept, 6% of the GPU
+constexpr size_t POOL_ALONE_MAX = (size_t)512 << 20;  // with no model or beam set alive
 constexpr size_t POOL_HOST_MAX = (size_t)64 << 20;
 struct CudaRt {
     static int device() {
@@ -43,7 +44,7 @@ struct CudaRt {
 std::atomic<int64_t> g_dev_bytes{0}, g_dev_limit{0};
 BlockPool<CudaRt> &pool() {
     // never destroyed: blocks may be released while the process exits
-    static auto *p = new BlockPool<CudaRt>(POOL_DEV_MAX, POOL_HOST_MAX, g_dev_bytes);
+    static auto *p = new BlockPool<CudaRt>(POOL_DEV_MAX, POOL_ALONE_MAX, POOL_HOST_MAX, g_dev_bytes);
     return *p;
 }
 }  // namespace

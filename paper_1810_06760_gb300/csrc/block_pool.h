@@ -4,7 +4,8 @@
 // synchronisation ordered every reuse, a block released since the device was last known to be idle is handed out
 // only after a device synchronisation (one for all such blocks), so any stream and thread may release and take.
 // Idle blocks are bounded (the largest go first), are given back when an allocation fails or would pass the caller's
-// bound, when the bound is set, and when the last model and beam set is destroyed.
+// bound, when the bound is set, and when the last model or beam set is destroyed.  Calls that need neither (the transform
+// alone) release their scratch with no such end in sight: then the bound is a small one.
 //
 // Host code without CUDA types, so that several devices can be tested on a machine without any.  Rt is the runtime:
 //   static int device(); static bool synchronize(); static void free_device(void *); static void free_host(void *);
@@ -31,7 +32,7 @@ template <class Rt> class BlockPool {
         Blocks blocks;
         size_t bytes = 0;
     };
-    const size_t dev_max, host_max;
+    const size_t dev_max, alone_max, host_max;   // alone: with no model or beam set alive
     std::mutex mu;
     std::map<int, Device> dev;
     Blocks host;
@@ -81,8 +82,8 @@ template <class Rt> class BlockPool {
     }
 
 public:
-    BlockPool(size_t dev_max_, size_t host_max_, std::atomic<int64_t> &used)
-        : dev_max(dev_max_), host_max(host_max_), in_use(used) {}
+    BlockPool(size_t dev_max_, size_t alone_max_, size_t host_max_, std::atomic<int64_t> &used)
+        : dev_max(dev_max_), alone_max(alone_max_), host_max(host_max_), in_use(used) {}
 
     // idle bytes of one device: a reserve for allocations on that device only
     size_t idle_bytes(int d) {
@@ -103,10 +104,11 @@ public:
     }
     void put_device(void *p, size_t bytes, int d) {
         std::lock_guard<std::mutex> lk(mu);
-        if (bytes > dev_max) {
+        const size_t max = objects > 0 ? dev_max : alone_max;
+        if (bytes > max) {
             Rt::free_device(p);
         } else {
-            trim_locked(dev_max - bytes);
+            trim_locked(max - bytes);
             Device &D = dev[d];
             D.blocks.emplace(bytes, Block{p, true, d});
             D.bytes += bytes;

@@ -1,6 +1,6 @@
 """The pool of idle blocks (csrc/block_pool.h) on a runtime of two devices that only counts: a device's idle bytes are its
 own, blocks are handed out on their device only, a failed allocation trims the device it was made on, blocks released since
-the last synchronisation wait for one, the bounds hold and the last object empties the pool."""
+the last synchronisation wait for one, the bounds hold, a small one with no object alive, and the last object empties the pool."""
 import subprocess
 from pathlib import Path
 
@@ -26,7 +26,7 @@ static void *blk(long i) { return (void *)i; }
 int main() {
     std::atomic<int64_t> used{0};
     const size_t MB = 1 << 20;
-    fga::BlockPool<Rt> pool(100 * MB, 10 * MB, used);
+    fga::BlockPool<Rt> pool(100 * MB, 25 * MB, 10 * MB, used);
     pool.object(1);
     size_t got = 0;
     // two blocks on device 0, one on device 1
@@ -67,6 +67,12 @@ int main() {
     CHECK(!freed.count(3) && host_frees == 1);
     pool.object(-1);
     CHECK(freed.count(3) && host_frees == 2 && pool.idle_bytes(1) == 0);
+    // with none alive a small bound holds
+    pool.put_device(blk(9), 10 * MB, 0);
+    pool.put_device(blk(10), 26 * MB, 0);
+    CHECK(freed.count(10) && !freed.count(9) && pool.idle_bytes(0) == 10 * MB);
+    pool.put_device(blk(11), 16 * MB, 1);
+    CHECK(freed.count(9) && pool.idle_bytes(0) == 0 && pool.idle_bytes(1) == 16 * MB);
     std::printf("ok\n");
     return 0;
 }
