@@ -462,11 +462,14 @@ fga_status fga_profile_read(fga_profile_t *out, int reset);
  * is called.  bytes <= 0 removes the bound (the default).  fga_device_memory_in_use reports the bytes
  * currently allocated for such buffers, without idle blocks.  Released blocks stay idle in the library for later
  * calls: up to 16 GiB while a model or beam set exists, up to 512 MiB otherwise.  They are given back to the device
- * when an allocation needs them, when this function is called, and when the last model or beam set is destroyed.
- * Process-wide; meant for hosts that share a GPU, and for testing the out-of-memory paths without exhausting the
+ * when an allocation of the library needs them, when this function or fga_release_idle_memory is called, and when the last
+ * model or beam set is destroyed.  Process-wide; meant for hosts that share a GPU, and for testing the out-of-memory paths without exhausting the
  * device. */
 fga_status fga_set_device_memory_limit(double bytes);
 double fga_device_memory_in_use(void);
+/* Gives the idle blocks (device and pinned) back at once, for other users of the device's memory, such as another
+ * allocator in this process; the bound above stays as it is.  Later calls allocate anew. */
+fga_status fga_release_idle_memory(void);
 
 /* Message of the last failing call on this thread (always NUL-terminated; truncated to cap). */
 void fga_last_error(char *buf, size_t cap);

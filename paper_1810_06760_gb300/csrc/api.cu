@@ -371,6 +371,11 @@ fga_status fga_set_device_memory_limit(double bytes) {
     return FGA_OK;
 }
 
+fga_status fga_release_idle_memory(void) {
+    pool().release();
+    return FGA_OK;
+}
+
 double fga_device_memory_in_use(void) { return (double)g_dev_bytes.load(); }
 
 fga_status fga_model_create(fga_model **out, const fga_model_desc *d, const float *grid_p, const float *grid_s,

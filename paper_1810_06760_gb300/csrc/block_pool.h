@@ -4,7 +4,7 @@
 // synchronisation ordered every reuse, a block released since the device was last known to be idle is handed out
 // only after a device synchronisation (one for all such blocks), so any stream and thread may release and take.
 // Idle blocks are bounded (the largest go first), are given back when an allocation fails or would pass the caller's
-// bound, when the bound is set, and when the last model or beam set is destroyed.  Calls that need neither (the transform
+// bound, when the bound is set, on request, and when the last model or beam set is destroyed.  Calls that need neither (the transform
 // alone) release their scratch with no such end in sight: then the bound is a small one.
 //
 // Host code without CUDA types, so that several devices can be tested on a machine without any.  Rt is the runtime:
@@ -80,6 +80,12 @@ template <class Rt> class BlockPool {
             free_largest(*best);
         }
     }
+    void release_locked() {
+        trim_locked(0);
+        for (auto &kv : host) Rt::free_host(kv.second.p);
+        host.clear();
+        host_bytes = 0;
+    }
 
 public:
     BlockPool(size_t dev_max_, size_t alone_max_, size_t host_max_, std::atomic<int64_t> &used)
@@ -138,11 +144,12 @@ public:
     void object(int d) {
         std::lock_guard<std::mutex> lk(mu);
         objects += d;
-        if (objects > 0) return;
-        trim_locked(0);
-        for (auto &kv : host) Rt::free_host(kv.second.p);
-        host.clear();
-        host_bytes = 0;
+        if (objects <= 0) release_locked();
+    }
+    // every idle block, whatever is alive
+    void release() {
+        std::lock_guard<std::mutex> lk(mu);
+        release_locked();
     }
 };
 

@@ -29,7 +29,7 @@ EXPORTED = ["fga_model_create", "fga_model_destroy", "fga_decompose", "fga_trans
             "fga_beams_export_all", "fga_beams_destroy", "fga_beams_params", "fga_beams_import", "fga_bin", "fga_profile_enable", "fga_profile_read",
             "fga_solve_vjp", "fga_server_create", "fga_server_submit", "fga_server_wait", "fga_server_stats",
             "fga_server_destroy", "fga_server_cancel", "fga_traveltime_adjoint", "fga_set_device_memory_limit",
-            "fga_device_memory_in_use", "fga_point_force_field", "fga_last_error", "fga_version"]
+            "fga_device_memory_in_use", "fga_release_idle_memory", "fga_point_force_field", "fga_last_error", "fga_version"]
 PROFILE_CATEGORIES = ["decompose", "propagate", "binning", "records", "gauss_sum", "gauss_reduce", "gauss_sum_state",
                       "interfaces", "adjoint_forward", "adjoint_reverse", "adjoint_init", "misfit"]
 
@@ -603,6 +603,11 @@ def set_device_memory_limit(nbytes: float) -> None:
 
 def device_memory_in_use() -> float:
     return float(lib().fga_device_memory_in_use())
+
+
+def release_idle_memory() -> None:
+    """fga_release_idle_memory: the blocks the library keeps idle go back to the device, for other allocators."""
+    _check(lib().fga_release_idle_memory())
 
 
 def profile_enable(mode: int) -> None:

@@ -61,12 +61,18 @@ int main() {
     pool.put_host(blk(7), 6 * MB, 1);
     pool.put_host(blk(8), 6 * MB, 1);
     CHECK(host_frees == 1);
+    // on request everything goes, whatever is alive; the bytes in use do not change
+    pool.put_device(blk(12), 5 * MB, 0);
+    const int64_t before = used;
+    pool.release();
+    CHECK(freed.count(3) && freed.count(12) && host_frees == 2 && pool.idle_bytes(0) + pool.idle_bytes(1) == 0 && used == before);
+    pool.put_device(blk(13), 30 * MB, 1);
     // the last object empties the pool
     pool.object(1);
     pool.object(-1);
-    CHECK(!freed.count(3) && host_frees == 1);
+    CHECK(!freed.count(13));
     pool.object(-1);
-    CHECK(freed.count(3) && host_frees == 2 && pool.idle_bytes(1) == 0);
+    CHECK(freed.count(13) && pool.idle_bytes(1) == 0);
     // with none alive a small bound holds
     pool.put_device(blk(9), 10 * MB, 0);
     pool.put_device(blk(10), 26 * MB, 0);

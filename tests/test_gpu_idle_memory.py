@@ -37,3 +37,30 @@ fga.transform(descs[1][0], out=out)
 print(before - free())
 """)
     assert kept <= (512 << 20) + (16 << 20)
+
+
+def test_idle_blocks_go_back_on_request_and_the_bound_stays():
+    given, refused = _run("""
+w = W.smooth(nq=8, np_=6, ny=24, nsteps=8, n_samples=8, rx_side=8, snap_side=0, grid_n=17)
+model = fga.model_from_medium(w.medium, 'cuda')
+f = torch.as_tensor(w.f, device='cuda')
+desc = fga.init_desc(w.k, f, None, w.y0, w.dy, w.mesh, w.classes, fga.PREC_FP32)
+solve = lambda: fga.solve(model, desc, w.dt, w.nsteps, w.times, rw=w.rw, rx_axes=w.rx_axes)
+u = solve()[0]
+fga.set_device_memory_limit(fga.device_memory_in_use() + 2e9)
+assert torch.equal(u, solve()[0])
+torch.cuda.synchronize()
+held = torch.cuda.mem_get_info()[0]
+fga.release_idle_memory()
+print(torch.cuda.mem_get_info()[0] - held)
+assert torch.equal(u, solve()[0])
+big = W.smooth(nq=16, np_=8, ny=24, nsteps=8, n_samples=8, rx_side=8, snap_side=0, grid_n=17)   # 1.6 GB of beams, twice
+try:
+    fga.solve(model, fga.init_desc(big.k, f, None, w.y0, w.dy, big.mesh, big.classes, fga.PREC_FP32), w.dt, w.nsteps,
+              w.times, rw=w.rw, rx_axes=w.rx_axes)
+    print(0)
+except fga.FGAError as e:
+    print(1 if e.status == fga.FGA_ERR_OOM else -1)
+""")
+    # the beam set and its sorted copy alone are 2 x 196 B x 442,368 beams = 173 MB
+    assert given > 150e6 and refused == 1
