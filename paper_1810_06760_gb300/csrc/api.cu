@@ -103,7 +103,6 @@ void block_cache_enable(cudaStream_t s) {
     tl_cache.on = true;
     tl_cache.stream = s;
 }
-size_t block_cache_bytes() { return tl_cache.dev_bytes; }
 void block_cache_trim(size_t keep) {
     // largest blocks first
     while (tl_cache.dev_bytes > keep && !tl_cache.dev.empty()) {

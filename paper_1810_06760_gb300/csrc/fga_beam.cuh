@@ -237,7 +237,6 @@ template <typename R> struct C2 {
 template <typename R> __device__ __forceinline__ C2<R> cmul(C2<R> a, C2<R> b) {
     return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r};
 }
-template <typename R> __device__ __forceinline__ C2<R> csub(C2<R> a, C2<R> b) { return {a.r - b.r, a.i - b.i}; }
 template <typename R> __device__ __forceinline__ C2<R> cmulsub(C2<R> a, C2<R> b, C2<R> c, C2<R> d) {
     // a*b - c*d
     return {a.r * b.r - a.i * b.i - (c.r * d.r - c.i * d.i), a.r * b.i + a.i * b.r - (c.r * d.i + c.i * d.r)};

@@ -199,7 +199,6 @@ struct HostBuf {
 void block_cache_enable(cudaStream_t s);
 void block_cache_disable();
 void block_cache_trim(size_t keep_bytes);
-size_t block_cache_bytes();
 
 // idle blocks of the process-wide pool (block_pool.h): their bytes on the current device; models and beam sets created
 // (1) and destroyed (-1) -- the pool is emptied when none is left

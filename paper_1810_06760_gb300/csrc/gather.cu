@@ -986,8 +986,6 @@ fga_status build_sum_plan(Workspace &ws, const BinGrid &g, const int32_t *cell_s
     return FGA_OK;
 }
 
-const int32_t *plan_host_cell_start(const Workspace &ws) { return ws.h_cell_start.as<int32_t>(); }
-
 fga_status run_sum(Workspace &ws, const SumPlan &plan, int precision, const void *rec, int64_t rec_stride, int ns,
                    const double *pts_dev, double k, double rw, void *u_out, int64_t u_stride, cudaStream_t s, int cat) {
     if (plan.ntiles == 0) return FGA_OK;

@@ -100,8 +100,6 @@ template <class F> fga_status ensure_scratch(DevBuf &b, int &n, int least, F byt
     }
     return st;
 }
-// bucket starts copied to the host by build_sum_plan (valid after it returns)
-const int32_t *plan_host_cell_start(const Workspace &ws);
 
 // acc += a * b for complex a, b as two fused multiply-add chains (the compiler may not reassociate
 // acc + (ar br - ai bi) into FMAs itself)

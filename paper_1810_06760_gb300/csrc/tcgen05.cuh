@@ -30,17 +30,6 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
     return d;                // base offset 0, relative LBO, swizzle none
 }
 
-// the same with explicit byte offsets between K-adjacent (lbo) and row-adjacent (sbo) core matrices
-// (multiples of 16 bytes; padded layouts spread one warp's stores over all banks)
-__device__ __forceinline__ uint64_t smem_desc_lbo_sbo(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
 // K-major operand of K extent 16 (rows of 32 bytes) in the 32-byte swizzle: within a group of 8 rows (256
 // bytes, SBO; groups contiguous) the two 16-byte halves of rows 4..7 are exchanged.  Base 256-byte aligned.
 __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
@@ -106,15 +95,6 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
     return false;
 }
 
-// 8 consecutive K elements (k % 8 == 0) of one row: one 16-byte store of their FP16 values
-__device__ __forceinline__ void store8(unsigned char *base, uint32_t off, const __half h[8]) {
-    uint4 v;
-    v.x = (uint32_t)__half_as_ushort(h[0]) | ((uint32_t)__half_as_ushort(h[1]) << 16);
-    v.y = (uint32_t)__half_as_ushort(h[2]) | ((uint32_t)__half_as_ushort(h[3]) << 16);
-    v.z = (uint32_t)__half_as_ushort(h[4]) | ((uint32_t)__half_as_ushort(h[5]) << 16);
-    v.w = (uint32_t)__half_as_ushort(h[6]) | ((uint32_t)__half_as_ushort(h[7]) << 16);
-    *reinterpret_cast<uint4 *>(base + off) = v;
-}
 // hi/lo split of 8 values scaled by s, stored as two 16-byte rows (hi and lo operand copies); pairs of
 // values are rounded to FP16 together (one f16x2 conversion per pair)
 __device__ __forceinline__ void split8(unsigned char *hi, unsigned char *lo, uint32_t off, const float x[8], float s) {
