@@ -567,10 +567,10 @@ __device__ __forceinline__ void push_event(int2 *__restrict__ list, unsigned *__
 template <typename R, int SHAPE>
 __global__ void __launch_bounds__(128) layered_run_kernel(ModelDev M, R *__restrict__ st, int32_t *__restrict__ flags,
                                                          int64_t cap, const unsigned long long *__restrict__ counts,
-                                                         R dt, int nsteps, int gmax, int2 *__restrict__ list,
-                                                         unsigned *__restrict__ nlist) {
-    const int64_t n = min((unsigned long long)cap, counts[0]);
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+                                                         int64_t first, int64_t end, R dt, int nsteps, int gmax,
+                                                         int2 *__restrict__ list, unsigned *__restrict__ nlist) {
+    const int64_t n = min((unsigned long long)end, counts[0]);   // slots first .. end - 1
+    for (int64_t b = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
         const int fl = flags[b];
         if (fl & FL_DEAD) continue;
         R y[NF], qc[3];
@@ -711,43 +711,54 @@ fga_status launch_layered_steps(const fga_model *m, fga_beams *b, double dt, int
     // event lists: two of cap entries, and a counter per round (a lineage meets at most gmax interfaces, 16 by
     // its flag bits, and at most one per step)
     const int rounds = std::max(1, std::min(std::min(b->gmax, 16), nsteps));
-    const size_t lb = sizeof(int2) * (size_t)b->cap, nb_ctr = sizeof(unsigned) * 20;
-    FGA_TRY(b->events.ensure(2 * lb + nb_ctr));
-    int2 *list[2] = {b->events.as<int2>(), b->events.as<int2>() + b->cap};
-    unsigned *ctr = reinterpret_cast<unsigned *>(b->events.as<char>() + 2 * lb);
-    FGA_CUDA(cudaMemsetAsync(ctr, 0, nb_ctr, s));
-    prof_add_beam_steps(b->nb * (int64_t)nsteps);
-    auto go = [&](auto real, auto shape) {
+    const size_t nb_ctr = sizeof(unsigned) * 20;
+    // Where they do not fit (the device or the caller's bound): one shorter list.  The group is then taken step by step,
+    // so that children meet no second interface in it, and slots entries of the population at a time.
+    const int64_t cap = b->cap;
+    int slots = (int)cap;
+    FGA_TRY(ensure_scratch(b->events, slots, 1024, [&](int n) { return sizeof(int2) * (n == cap ? 2 : 1) * (size_t)n + nb_ctr; }));
+    const bool whole = slots == cap;
+    int2 *list[2] = {b->events.as<int2>(), b->events.as<int2>() + (whole ? cap : 0)};
+    unsigned *ctr = reinterpret_cast<unsigned *>(b->events.as<char>() + sizeof(int2) * (whole ? 2 : 1) * (size_t)slots);
+    auto go = [&](auto real, auto shape, int64_t first, int64_t end, int steps, int rounds) -> fga_status {
         using R = decltype(real);
         constexpr int SHAPE = decltype(shape)::value;
         unsigned long long *counts = b->counts.as<unsigned long long>();
+        FGA_CUDA(cudaMemsetAsync(ctr, 0, nb_ctr, s));
         {
             ProfScope ps(P_PROP, s);
-            layered_run_kernel<R, SHAPE><<<(unsigned)std::min<int64_t>((b->cap + 127) / 128, 152 * 12), 128, 0, s>>>(
-                m->dev, b->state.as<R>(), b->flags.as<int32_t>(), b->cap, counts, (R)dt, nsteps, b->gmax, list[0], ctr);
+            layered_run_kernel<R, SHAPE><<<(unsigned)std::min<int64_t>((end - first + 127) / 128, 152 * 12), 128, 0, s>>>(
+                m->dev, b->state.as<R>(), b->flags.as<int32_t>(), cap, counts, first, end, (R)dt, steps, b->gmax, list[0], ctr);
         }
         for (int r = 0; r < rounds; r++) {
             ProfScope ps(P_OTHER_LAYER, s);
             layered_event_kernel<R, SHAPE><<<152 * 8, 64, 0, s>>>(
-                m->dev, b->state.as<R>(), b->flags.as<int32_t>(), b->id.as<int32_t>(), b->path.as<long long>(), b->cap,
-                counts, (R)dt, nsteps, b->gmax, b->rel_min, list[r & 1], ctr + r, list[(r + 1) & 1], ctr + r + 1);
+                m->dev, b->state.as<R>(), b->flags.as<int32_t>(), b->id.as<int32_t>(), b->path.as<long long>(), cap,
+                counts, (R)dt, steps, b->gmax, b->rel_min, list[r & 1], ctr + r, list[(r + 1) & 1], ctr + r + 1);
         }
+        FGA_CUDA(cudaGetLastError());
+        return FGA_OK;
+    };
+    auto run = [&](auto real, auto shape) -> fga_status {
+        prof_add_beam_steps(b->nb * (int64_t)nsteps);
+        if (whole) return go(real, shape, 0, cap, nsteps, rounds);
+        for (int n = 0; n < nsteps; n++) {
+            unsigned long long live = 0;   // the population of this step: children join at the next
+            FGA_CUDA(cudaMemcpyAsync(&live, b->counts.p, sizeof live, cudaMemcpyDeviceToHost, s));
+            FGA_CUDA(cudaStreamSynchronize(s));
+            const int64_t nb = (int64_t)std::min<unsigned long long>(live, (unsigned long long)cap);
+            for (int64_t first = 0; first < nb; first += slots)
+                FGA_TRY(go(real, shape, first, std::min(first + slots, nb), 1, 1));
+        }
+        return FGA_OK;
     };
     using std::integral_constant;
     auto shape = [&](auto real) {
-        if (m->dev.shells)
-            go(real, integral_constant<int, 1>{});
-        else if (m->dev.undul)
-            go(real, integral_constant<int, 2>{});
-        else
-            go(real, integral_constant<int, 0>{});
+        return m->dev.shells  ? run(real, integral_constant<int, 1>{})
+               : m->dev.undul ? run(real, integral_constant<int, 2>{})
+                              : run(real, integral_constant<int, 0>{});
     };
-    if (b->precision == FGA_PREC_FP64)
-        shape(double{});
-    else
-        shape(float{});
-    FGA_CUDA(cudaGetLastError());
-    return FGA_OK;
+    return b->precision == FGA_PREC_FP64 ? shape(double{}) : shape(float{});
 }
 
 }  // namespace fga
