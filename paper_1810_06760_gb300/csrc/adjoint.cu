@@ -1106,7 +1106,9 @@ fga_status run_vjp(const fga_model *m, const fga_init_desc *init, const fga_solv
         int dev = 0, sms = 152;
         FGA_CUDA(cudaGetDevice(&dev));
         FGA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        ctas = 2 * sms;
+        // no more than a class fills: the scratch is then never larger than the state slots it stands for
+        const int64_t most = *std::max_element(b->n_cls, b->n_cls + 4);
+        ctas = (int)std::min<int64_t>(2 * sms, std::max<int64_t>(1, (most + ADJ_THREADS - 1) / ADJ_THREADS));
         FGA_TRY(scr.ensure(sizeof(R) * 2 * NF * ADJ_THREADS * (size_t)ctas));
     }
     R *CK = ck.as<R>(), *SEG = seg.as<R>(), *YB = yb.as<R>(), *RS = rs.as<R>();
