@@ -158,7 +158,7 @@ struct ClassBlocks {
 // next right-hand side formed as soon as this one's speed is known (the copies of new cells overlap with the rest
 // of it).  One launch for all classes (blockIdx.y the class), so that small beam sets fill the SMs once instead of
 // four times.  694 instructions per warp and right-hand side at 8 warps an SM (251 registers): the FMA pipe is
-// 55% busy, the issue slots 59%, the L1 data pipe 57% (rk4_kernel: 34%, 32%, 80% once the beams have spread).
+// 54% busy, the issue slots 59%, the L1 data pipe 53% on 0.44 M beams (rk4_kernel: 34%, 32%, 80% once the beams have spread).
 // Propagation, 200 steps: 0.44 M beams 21.5 -> 10.8 ms, 2.7 M beams 108.4 -> 65.1 ms; 8.4 M beams x 100 steps with
 // 250 samples 162 -> 112 ms.  Capped at 168 registers for 10 warps it spills: 113.6 ms on the 2.7 M beams.
 template <int WAVE>
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(128) rk4_cell_kernel(ModelDev M, float *__rest
 }
 
 // Constant media: nsteps RK4 steps in closed form (straight.cuh), one launch for all classes
-// (blockIdx.y the class).  Bound by the issue slots in FP32 (about 100 instructions a step, slots 80% used; the state's
+// (blockIdx.y the class).  Bound by the issue slots in FP32 (about 100 instructions a step, slots 86% used; the state's
 // stream, 49 reals read and 28 written per beam and launch, is a quarter of the time) and by the FP64 pipe in FP64.  The
 // steps gather the amplitudes' gain in one complex factor, applied at samples and at the end, and in FP64 two
 // reciprocals share a division.  Against the general kernel's four right-hand sides per step: point-force experiment,
@@ -345,7 +345,6 @@ __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ 
         }
 #pragma unroll
         for (int f = F_A0; f < NF; f += 2) {
-            if (f != F_A0 && !wave) break;   // a P beam has one amplitude
             const C2<R> a = cmul(fac, C2<R>{y[f], y[f + 1]});
             y[f] = a.r;
             y[f + 1] = a.i;
@@ -359,7 +358,8 @@ __global__ void __launch_bounds__(128) const_kernel(ModelDev M, R *__restrict__ 
 #pragma unroll
     for (int f = F_DQ; f < F_DP; f++) st[(int64_t)f * cap + b] = y[f];
 #pragma unroll
-    for (int f = F_A0; f < NF; f++) st[(int64_t)f * cap + b] = y[f];
+    for (int f = F_A0; f < NF; f++)
+        if (f < F_A1 || wave) st[(int64_t)f * cap + b] = y[f];   // a P beam has one amplitude
 #pragma unroll
     for (int d = 0; d < 3; d++) st[(int64_t)(F_QC + d) * cap + b] = qc[d];
 }
