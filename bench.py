@@ -33,9 +33,9 @@ FLOP_PER_PAIR_OUT = 9.0       # dx, r^2, compare
 MUFU_PER_PAIR_IN = 3.0        # exp2, sin, cos
 FLOP_PER_LATTICE_PAIR_IN = 26.0   # window test (add, compare) + 3 complex multiply-adds
 # DRAM bytes (dram__bytes_read + write) per launch of each category's kernel on the full smooth workload,
-# from ncu captures summarised under profiles/; a category is absent until its current kernel is captured
-# (the plane kernel that takes all samples of a window and the RK4 kernel with cell columns are not yet).
-TRAFFIC_BYTES_PER_LAUNCH = {}
+# from the ncu captures summarised in profiles/smooth_full_dram.md: rk4_cell_kernel, all classes and about 21 steps a launch.
+# The plane kernel's launches differ in their number of samples (1.06 GB a sample), so its category has no one figure.
+TRAFFIC_BYTES_PER_LAUNCH = {"propagate": 6.41e10}
 
 
 def parse():

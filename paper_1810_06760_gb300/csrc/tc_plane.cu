@@ -31,8 +31,8 @@
 //  - A group's last block of an item is marked; when every group has sent it, the accumulator (one of two, 256
 //    columns each) is handed to the epilogue warps, which copy it to the item's partial sums while the next item
 //    accumulates in the other one.
-// What bounds it: the producers' issue slots (860 warp instructions per 16 beams, 62% of the slots used; tensor
-// pipe 34%, shared memory 46%; 378 cycles per 16 beams and SM).  Sums of a solve, against one launch per sample with
+// What bounds it: the producers' issue slots (860 warp instructions per 16 beams and 378 cycles of an SM; on 0.44 M beams
+// and one window of samples of 16 x 16 receivers 58% of the slots, tensor pipe 30%, shared memory 39%).  Sums of a solve, against one launch per sample with
 // seven single-warp producers and padded operands: 200 samples of 2.7 M beams on 16 x 16 receivers 48.7 -> 26.9 ms
 // (0.44 M beams: 13.4 -> 5.7 ms), 250 samples of 8.4 M beams on 20 x 20 receivers 192 -> 118 ms; the reductions
 // 4.9 -> 1.0, 3.3 -> 0.5 and 7.1 -> 3.2 ms.
@@ -670,7 +670,10 @@ fga_status run_plane_tc(Workspace &ws, const LatticePlan &plan, const void *rec,
                                           PL_SMEM));                                                                  \
             plane_tc_kernel<CNT, JT, IT><<<grid, PL_THREADS, PL_SMEM, s>>>(A);                                        \
         } while (0)
-                // quarters of 5 x 5 (the 20 x 20 plane of the benchmark) and 4 x 4 points (16 x 16) unrolled
+                // Tiles of 17 to 20 and of 13 to 16 points on both axes (quarters of 5 x 5 and 4 x 4 points) have their loops
+                // unrolled, which takes a seventh off the sums: 138.6 -> 117.7 ms on 250 samples of 8.4 M beams on 20 x 20
+                // receivers, 31.4 -> 26.9 ms on 200 of 2.7 M on 16 x 16.  Other tiles take the general loops: a variant for each
+                // of the 30 pairs of quarters would multiply the build.
                 if (cnt) FGA_PLANE(true, 0, 0);
                 else if (J == 5 && I == 5) FGA_PLANE(false, 5, 5);
                 else if (J == 4 && I == 4) FGA_PLANE(false, 4, 4);
